@@ -39,9 +39,10 @@ __global__ void batch_solid_tiles_kernel(const Model m, unsigned char* flags, in
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= ntx * nty) return;
   const int x0 = (t % ntx) * tx, y0 = (t / ntx) * ty;
+  const int xe = x0 + tx < m.nx ? x0 + tx : m.nx, ye = y0 + ty < m.ny ? y0 + ty : m.ny;
   bool any = false;
-  for (int ly = -1; ly <= ty; ++ly)
-    for (int lx = -1; lx <= tx; ++lx) any |= solid_mapped(m, x0 + lx, y0 + ly);
+  for (int y = y0 - 1; y <= ye; ++y)
+    for (int x = x0 - 1; x <= xe; ++x) any |= solid_mapped(m, x, y);
   flags[t] = any ? 1 : 0;
 }
 
@@ -53,7 +54,7 @@ int batch_variant_stages(int v) { return batch::kVariants[v].stages; }
 
 cudaError_t batch_plan_build(const BatchMember* members, int count, int storage, int flow, int v,
                              int order, BatchPlan* plan) {
-  const int ty = batch::kVariants[v].ty, tx = 32;
+  const int ty = batch::kVariants[v].ty, tx = batch::kVariants[v].tx;
   const size_t es = storage == ST_FP32 ? 4 : 2;
   const int qfg = (flow ? 9 : 0) + 9;
   const int hx = int(16 / es);

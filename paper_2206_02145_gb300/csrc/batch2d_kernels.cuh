@@ -61,19 +61,18 @@ static_assert(offsetof(BatchDesc, m) % 16 == 0 &&
 // stage's model slot holds another instance's model, the model is copied into
 // it by the TMA with the tile data (same barrier).  The computation then reads
 // everything from shared memory: no global lookups on a tile's critical path.
-template <typename T, bool FLOW, int TX, int TY, int S, bool MASK, bool CHM>
-__global__ void __launch_bounds__(TX* TY, (640 / (TX * TY)) > 2 ? 640 / (TX * TY) : 2)
+template <typename T, bool FLOW, int TX, int TY, bool PAIR, int S, bool MASK, bool CHM>
+__global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(),
+                                  512 / tile_threads<TX, TY, PAIR>())
     step2d_batch_kernel(const BatchDesc* __restrict__ descs, const BatchSeg* __restrict__ segs,
                         const int* __restrict__ cta_seg) {
   using L = Tiles2D<T, FLOW, TX, TY>;
   constexpr int SX = TX + 2, SY = TY + 2;
   constexpr int STAGE = L::STAGE + kModelSlot;
-  extern __shared__ unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[S];
   __shared__ float sh_phi[SY][SX];
   __shared__ StageMeta meta[S];
-  unsigned char* smem = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   const int tid = threadIdx.x;
   const int sb = cta_seg[blockIdx.x], se = cta_seg[blockIdx.x + 1];
   int ntiles = 0;  // this CTA's tiles (every thread)
@@ -146,10 +145,9 @@ __global__ void __launch_bounds__(TX* TY, (640 / (TX * TY)) > 2 ? 640 / (TX * TY
     }
     const StageMeta mt = meta[s];
     unsigned char* st = smem + s * STAGE;
-    tile_2d<T, FLOW, TX, TY, MASK, CHM>(*reinterpret_cast<const Model*>(st + L::STAGE),
-                                        static_cast<const T*>(mt.src), static_cast<T*>(mt.dst),
-                                        mt.ring_cur, mt.err, mt.x0, mt.y0, mt.c, st,
-                                        &sh_phi[0][0]);
+    tile_2d<T, FLOW, TX, TY, PAIR, MASK, CHM>(
+        *reinterpret_cast<const Model*>(st + L::STAGE), static_cast<const T*>(mt.src),
+        static_cast<T*>(mt.dst), mt.ring_cur, mt.err, mt.x0, mt.y0, mt.c, st, &sh_phi[0][0], false);
     __syncthreads();  // stage s (tile data, model slot, meta) and sh_phi are free again
     if (tid == 0) {
       fence_proxy_async_smem();
@@ -158,27 +156,27 @@ __global__ void __launch_bounds__(TX* TY, (640 / (TX * TY)) > 2 ? 640 / (TX * TY
   }
 }
 
-// Compiled variants: (tile rows, pipeline stages).
+// Compiled variants: tile columns and rows, pipeline stages, nodes per thread.
 struct Variant {
-  int ty, stages;
+  int tx, ty, stages, nodes;
 };
-constexpr Variant kVariants[] = {{4, 2}, {8, 2}, {2, 3}, {4, 3}};
+constexpr Variant kVariants[] = {{64, 4, 2, 2}, {32, 8, 2, 2}, {32, 4, 2, 2}, {32, 4, 2, 1}};
 constexpr int kNumVariants = int(sizeof(kVariants) / sizeof(kVariants[0]));
 
-template <typename T, bool FLOW, int TY, int S, bool MASK, bool CHM>
+template <typename T, bool FLOW, int TX, int TY, int S, bool PAIR, bool MASK, bool CHM>
 struct VariantImpl {
-  static constexpr int TX = 32;
+  static constexpr int THREADS = tile_threads<TX, TY, PAIR>();
   using L = Tiles2D<T, FLOW, TX, TY>;
   static cudaError_t setup(int* ctas, int* smem) {
-    auto kern = step2d_batch_kernel<T, FLOW, TX, TY, S, MASK, CHM>;
-    *smem = S * (L::STAGE + kModelSlot) + 128;
+    auto kern = step2d_batch_kernel<T, FLOW, TX, TY, PAIR, S, MASK, CHM>;
+    *smem = S * (L::STAGE + kModelSlot);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
       return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TX * TY, *smem)) !=
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, *smem)) !=
         cudaSuccess)
       return e;
     *ctas = sms * (per_sm > 0 ? per_sm : 1);
@@ -186,8 +184,8 @@ struct VariantImpl {
   }
   static cudaError_t launch(const BatchDesc* d, const BatchSeg* segs, const int* cta_seg,
                             int grid, int smem, cudaStream_t s) {
-    step2d_batch_kernel<T, FLOW, TX, TY, S, MASK, CHM>
-        <<<grid, TX * TY, smem, s>>>(d, segs, cta_seg);
+    step2d_batch_kernel<T, FLOW, TX, TY, PAIR, S, MASK, CHM>
+        <<<grid, THREADS, smem, s>>>(d, segs, cta_seg);
     return cudaGetLastError();
   }
 };
@@ -195,16 +193,17 @@ struct VariantImpl {
 template <typename T, bool FLOW, bool MASK, bool CHM>
 cudaError_t dispatch_v(int v, bool setup, int* ctas, int* smem, const BatchDesc* d,
                        const BatchSeg* segs, const int* cta_seg, int grid, cudaStream_t s) {
-#define LBPF_VARIANT(I, TY, S)                                                          \
-  case I:                                                                               \
-    return setup ? VariantImpl<T, FLOW, TY, S, MASK, CHM>::setup(ctas, smem)            \
-                 : VariantImpl<T, FLOW, TY, S, MASK, CHM>::launch(d, segs, cta_seg, grid, \
-                                                                  *smem, s);
+#define LBPF_VARIANT(I)                                                                    \
+  case I: {                                                                                \
+    using V = VariantImpl<T, FLOW, kVariants[I].tx, kVariants[I].ty, kVariants[I].stages,  \
+                          kVariants[I].nodes == 2, MASK, CHM>;                             \
+    return setup ? V::setup(ctas, smem) : V::launch(d, segs, cta_seg, grid, *smem, s);     \
+  }
   switch (v) {
-    LBPF_VARIANT(0, 4, 2)
-    LBPF_VARIANT(1, 8, 2)
-    LBPF_VARIANT(2, 2, 3)
-    LBPF_VARIANT(3, 4, 3)
+    LBPF_VARIANT(0)
+    LBPF_VARIANT(1)
+    LBPF_VARIANT(2)
+    LBPF_VARIANT(3)
     default: return cudaErrorInvalidValue;
   }
 #undef LBPF_VARIANT

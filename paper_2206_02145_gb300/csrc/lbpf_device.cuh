@@ -49,16 +49,33 @@ __device__ __forceinline__ R d3q7_w(int a) {
 }
 
 // ---- arithmetic helpers -------------------------------------------------------
-__device__ __forceinline__ float rsqrt_r(float v) { return rsqrtf(v); }
 // Reciprocal of the per-node relaxation and velocity denominators (all in
-// [0.5, ~10]): in FP32 the hardware approximation (2 ulp) instead of the
-// IEEE-exact division sequence; in FP64 the exact division.
-__device__ __forceinline__ float rcp_r(float v) { return __fdividef(1.0f, v); }
+// [0.5, ~10]) and reciprocal root of |grad phi|^2 (> 1e-12 where it is used):
+// in FP32 the hardware approximations (2 ulp), one instruction each in the
+// form without denormal handling (denormal arguments do not occur; the forms
+// with it scale and compare around each, 40 issue slots per two nodes); in
+// FP64 the exact division and root.
+__device__ __forceinline__ float rcp_r(float v) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float rsqrt_r(float v) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
 __device__ __forceinline__ double rcp_r(double v) { return 1.0 / v; }
 __device__ __forceinline__ double rsqrt_r(double v) { return rsqrt(v); }
-template <typename R>
-__device__ __forceinline__ R clamp1(R v) {
-  return v < R(-1) ? R(-1) : (v > R(1) ? R(1) : v);
+// clamp to [-1, 1]; NaN stays NaN
+__device__ __forceinline__ double clamp1(double v) {
+  return v < -1.0 ? -1.0 : (v > 1.0 ? 1.0 : v);
+}
+__device__ __forceinline__ float clamp1(float v) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(v), "f"(-1.0f));
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(r), "f"(1.0f));
+  return r;
 }
 __device__ __forceinline__ bool finite_r(float v) { return isfinite(v); }
 
@@ -117,45 +134,145 @@ struct Pop<__nv_bfloat16> {
   }
 };
 
+// ---- one or two nodes per thread ------------------------------------------------
+// The per-node arithmetic is written once over a number type N: float or
+// double (one node) or float2 (two nodes of a thread, one per lane, on the
+// packed FP32 instructions of sm_100 and later: one issue slot for both).
+// Every lane rounds exactly like the scalar form, so a node's result does not
+// depend on how many nodes its thread holds.
+template <typename N>
+struct Lanes {
+  using S = N;
+  static constexpr int V = 1;
+};
+template <>
+struct Lanes<float2> {
+  using S = float;
+  static constexpr int V = 2;
+};
+__device__ __forceinline__ float2 fma_r(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul_r(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add_r(float2 a, float2 b) { return __fadd2_rn(a, b); }
+// a b for a product whose only use is a sum: the assembler fuses such a packed
+// multiply and add into one rounding (the scalar ones it does not, and neither
+// a packed product with several uses), so the packed form takes a -0 that the
+// compiler does not know to be one as its addend
+__device__ __forceinline__ float prod_r(float a, float b, float) { return mul_r(a, b); }
+__device__ __forceinline__ double prod_r(double a, double b, double) { return mul_r(a, b); }
+__device__ __forceinline__ float2 prod_r(float2 a, float2 b, float mzero) {
+  return __ffma2_rn(a, b, make_float2(mzero, mzero));
+}
+__device__ __forceinline__ float neg_r(float a) { return -a; }
+__device__ __forceinline__ double neg_r(double a) { return -a; }
+__device__ __forceinline__ float2 neg_r(float2 a) { return make_float2(-a.x, -a.y); }
+template <typename N>
+__device__ __forceinline__ N sub_r(N a, N b) { return add_r(a, neg_r(b)); }
+__device__ __forceinline__ float2 rcp_r(float2 v) { return make_float2(rcp_r(v.x), rcp_r(v.y)); }
+__device__ __forceinline__ float2 rsqrt_r(float2 v) {
+  return make_float2(rsqrt_r(v.x), rsqrt_r(v.y));
+}
+__device__ __forceinline__ float2 clamp1(float2 v) { return make_float2(clamp1(v.x), clamp1(v.y)); }
+template <typename N>
+__device__ __forceinline__ N splat(typename Lanes<N>::S v) {
+  if constexpr (Lanes<N>::V == 2) return make_float2(v, v);
+  else return v;
+}
+// are a, b and c finite (in every lane)?
+template <typename N>
+__device__ __forceinline__ bool all_finite(N a, N b, N c) {
+  const N z = splat<N>(typename Lanes<N>::S(0));
+  const N t = fma_r(c, z, fma_r(b, z, mul_r(a, z)));
+  if constexpr (Lanes<N>::V == 2) return t.x + t.y == 0.f;
+  else return t == typename Lanes<N>::S(0);
+}
+// v where |grad phi|^2 = g2 > 1e-12, elsewhere w
+__device__ __forceinline__ float where_steep(float g2, float v, float w) {
+  return g2 > 1e-12f ? v : w;
+}
+__device__ __forceinline__ double where_steep(double g2, double v, double w) {
+  return g2 > 1e-12 ? v : w;
+}
+__device__ __forceinline__ float2 where_steep(float2 g2, float2 v, float2 w) {
+  return make_float2(where_steep(g2.x, v.x, w.x), where_steep(g2.y, v.y, w.y));
+}
+__device__ __forceinline__ bool any_steep(float g2) { return g2 > 1e-12f; }
+__device__ __forceinline__ bool any_steep(double g2) { return g2 > 1e-12; }
+__device__ __forceinline__ bool any_steep(float2 g2) { return g2.x > 1e-12f || g2.y > 1e-12f; }
+
 // ---- anisotropy (Eq. 3) and flux vector N (Eq. 21) ----------------------------
-// n = -grad/|grad| (solid -> liquid).  k-fold: cos/sin(k theta) are the real and
-// imaginary parts of (n_x + i n_y)^k, rotated by k theta0, so no atan2 is needed.
+// n = -grad/|grad| (solid -> liquid); a_s = 1 and N = 0 where |grad|^2 <= 1e-12.
+// k-fold: cos/sin(k theta) are the real and imaginary parts of (n_x + i
+// n_y)^k, rotated by k theta0, so no atan2 is needed.
 // N = fac |grad|^2 a_s d(a_s)/d(grad):
 //   k-fold: N = fac k eps a_s sin(k(theta - theta0)) (g_y, -g_x)
 //   cubic : N_i = fac 16 eps a_s |grad| (n_i S - n_i^3), S = sum n_j^4
-template <typename R>
-__device__ __forceinline__ void aniso(const Model& m, R gx, R gy, R gz, R& as, R& Nx, R& Ny,
-                                      R& Nz) {
-  as = R(1);
-  Nx = Ny = Nz = R(0);
-  R g2 = gx * gx + gy * gy + gz * gz;
-  const Coef<R>& c = coef<R>(m);
-  if (!(g2 > R(1e-12)) || c.eps == R(0)) return;
-  const R ig = rsqrt_r(g2);
-  const R nx = -gx * ig, ny = -gy * ig, nz = -gz * ig;
-  const R eps = c.eps, fac = c.aniso_fac;
+template <typename N>
+__device__ __forceinline__ void aniso_cubic(const Coef<typename Lanes<N>::S>& c, const N* n,
+                                            N g2, N ig, int dim, N& a, N* out) {
+  using S1 = typename Lanes<N>::S;
+  N n2[3], S = splat<N>(S1(0));
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    if (d < dim) n2[d] = mul_r(n[d], n[d]);
+  S = fma_r(n2[0], n2[0], mul_r(n2[1], n2[1]));
+  if (dim == 3) S = fma_r(n2[2], n2[2], S);
+  a = fma_r(splat<N>(S1(4) * c.eps), S, splat<N>(fma_r(S1(-3), c.eps, S1(1))));
+  const N amp = mul_r(mul_r(splat<N>(c.aniso_fac * S1(16) * c.eps), a), mul_r(g2, ig));
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    if (d < dim) out[d] = mul_r(mul_r(amp, n[d]), sub_r(S, n2[d]));
+}
+
+template <typename N>
+__device__ __forceinline__ void aniso_2d(const Model& m, N gx, N gy, N& as, N& Nx, N& Ny) {
+  using S1 = typename Lanes<N>::S;
+  const Coef<S1>& c = coef<S1>(m);
+  as = splat<N>(S1(1));
+  Nx = Ny = splat<N>(S1(0));
+  const N g2 = fma_r(gx, gx, mul_r(gy, gy));
+  if (!any_steep(g2) || c.eps == S1(0)) return;
+  // (n = 0 on a flat lane: the k-fold form then gives a_s = 1, N = 0 by itself)
+  const N ig = where_steep(g2, rsqrt_r(g2), splat<N>(S1(0)));
+  const N n[2] = {mul_r(neg_r(gx), ig), mul_r(neg_r(gy), ig)};
   if (m.fold > 0) {
-    R ck = nx, sk = ny;
+    N ck = n[0], sk = n[1];
     for (int j = 1; j < m.fold; ++j) {
-      const R c2 = ck * nx - sk * ny;
-      sk = ck * ny + sk * nx;
+      const N c2 = fma_r(ck, n[0], neg_r(mul_r(sk, n[1])));
+      sk = fma_r(ck, n[1], mul_r(sk, n[0]));
       ck = c2;
     }
-    const R cosd = ck * c.ck0 + sk * c.sk0;
-    const R sind = sk * c.ck0 - ck * c.sk0;
-    as = R(1) + eps * cosd;
-    const R amp = fac * R(m.fold) * eps * as * sind;
-    Nx = amp * gy;
-    Ny = -amp * gx;
+    const N ck0 = splat<N>(c.ck0), sk0 = splat<N>(c.sk0);
+    const N cosd = fma_r(ck, ck0, mul_r(sk, sk0));
+    const N sind = fma_r(sk, ck0, neg_r(mul_r(ck, sk0)));
+    as = fma_r(splat<N>(c.eps), cosd, splat<N>(S1(1)));
+    const N amp = mul_r(mul_r(splat<N>(c.aniso_fac * S1(m.fold) * c.eps), as), sind);
+    Nx = mul_r(amp, gy);
+    Ny = mul_r(neg_r(amp), gx);
   } else {
-    const R nx2 = nx * nx, ny2 = ny * ny, nz2 = nz * nz;
-    const R S = nx2 * nx2 + ny2 * ny2 + nz2 * nz2;
-    as = R(1) - R(3) * eps + R(4) * eps * S;
-    const R amp = fac * R(16) * eps * as * (g2 * ig);
-    Nx = amp * nx * (S - nx2);
-    Ny = amp * ny * (S - ny2);
-    Nz = amp * nz * (S - nz2);
+    N a, out[2];
+    aniso_cubic<N>(c, n, g2, ig, 2, a, out);
+    as = where_steep(g2, a, as);
+    Nx = out[0];
+    Ny = out[1];
   }
+}
+
+template <typename N>
+__device__ __forceinline__ void aniso_3d(const Model& m, const N (&g)[3], N& as, N (&Nv)[3]) {
+  using S1 = typename Lanes<N>::S;
+  const Coef<S1>& c = coef<S1>(m);
+  as = splat<N>(S1(1));
+#pragma unroll
+  for (int d = 0; d < 3; ++d) Nv[d] = splat<N>(S1(0));
+  const N g2 = fma_r(g[2], g[2], fma_r(g[0], g[0], mul_r(g[1], g[1])));
+  if (!any_steep(g2) || c.eps == S1(0)) return;
+  // (n = 0 on a flat lane, so N = 0 there by itself)
+  const N ig = where_steep(g2, rsqrt_r(g2), splat<N>(S1(0)));
+  N n[3], a;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) n[d] = mul_r(neg_r(g[d]), ig);
+  aniso_cubic<N>(c, n, g2, ig, 3, a, Nv);
+  as = where_steep(g2, a, as);
 }
 
 // periodic wrap of a coordinate that is at most one period out of range

@@ -26,6 +26,7 @@ struct Coef {
   R body[3];
   R u_in, U_in, ref_f, ref_g, ref_h;
   R chm_wb, chm_wh;  // central Hermite MRT: trace and higher-order rates
+  R mzero;           // -0, an addend the compiler cannot fold away (prod_r)
 };
 
 // Derived model constants (FP64 on the host; the kernels use cf / cd).  Device layout: every population is its own array of
@@ -105,6 +106,7 @@ inline void finalize(Model& m) {
     c.ref_h = R(m.ref_h);
     c.chm_wb = R(m.chm_wb);
     c.chm_wh = R(m.chm_wh);
+    c.mzero = R(-0.0);
   };
   fill(m.cf);
   fill(m.cd);

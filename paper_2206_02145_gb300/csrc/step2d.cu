@@ -18,18 +18,35 @@
 // a_s^2 h(r + c, t+1) = h*(r) - (1 - a_s^2(r)) h(r + c, t), i.e. needs the old
 // h of the destination node.
 //
-// step2d_tma_kernel (FP32 and 16-bit storage): persistent CTAs stream 32 x 4
-// tiles through a 2-stage shared-memory pipeline, 4 CTAs of 128 threads per SM
-// (tile, depth and CTAs per SM chosen by a sweep on GB300).  Per tile one thread issues
-// three TMA tensor loads on one mbarrier: f and g of the tile, h of the tile
-// plus halo (box starting 16 bytes left of the tile so that its innermost
+// step2d_tma_kernel (FP32 and 16-bit storage): persistent CTAs of 128 threads
+// stream tiles through a 2-stage shared-memory pipeline.  Per tile one thread
+// issues three TMA tensor loads on one mbarrier: f and g of the tile, h of the
+// tile plus halo (box starting 16 bytes left of the tile so that its innermost
 // coordinate stays aligned), and the phi ring of the tile.  While a tile is
 // computed and pushed, the next one is in flight.  Halo positions outside
-// the domain (the TMA fills them with zeros) are patched with the mapped
-// periodic / zero-gradient values on edge tiles only.
+// the domain (the TMA fills them with zeros) are patched on edge tiles only.
+//
+// What bounds it, and the shape taken for that (1024^2 and 2480 x 2080 coupled
+// FP32 steps; GB300, 6.69 TB/s copy):
+//  - issue slots and latency.  A thread of a large grid holds two nodes, 2 rows
+//    apart, on the packed two-lane FP32 instructions (lbpf_device.cuh):
+//    480 warp instructions per 32 nodes instead of 754 (FP16: 606 for 906);
+//  - how the memory is asked.  Tiles are 64 x 4 (256-byte rows: 64 x 4 moves
+//    the step's bytes without arithmetic in 36 us, 32 x 8 in 38), and where
+//    the state exceeds the L2 at most kStageBytes of stages are resident per
+//    SM: with all CTAs that fit the h halos are read twice (666 MB from DRAM
+//    per 2480 x 2080 step against 587) and the step is slower.
+//  1024^2: 48.4 -> 40.2 us (0.72 -> 0.87 of the copy rate), FP16 38.2 -> 28.9;
+//  2480 x 2080: 250 -> 199 us, FP16 -> 119.
+// Grids of fewer than kPairTiles tiles take 32 x 4 tiles with one node per
+// thread: more CTAs, a shorter chain per tile (512^2: 10.5 us against 12.4;
+// 640^2: 14.2 against 13.9).
 //
 // step2d_kernel (FP64 storage): one thread per node, one tile per CTA, the
 // same per-node code.
+#include <algorithm>
+#include <numeric>
+
 #include "step2d_tile.cuh"
 #include "tma_host.h"
 
@@ -98,43 +115,27 @@ __global__ void __launch_bounds__(TX* TY)
   __syncthreads();
   const bool solids = m.solid && m.solid_tiles[blockIdx.y * gridDim.x + blockIdx.x];
   if (!active) return;
-  if (solids && m.solid[idx]) {
-    ring_cur[idx] = sh_phi[ty + 1][tx + 1];  // a solid node keeps its state
-    return;
-  }
-  TileView<R, R, SX, SX * SY, 0> hs{&sh_h[0][0][0]};
-  if (!solids && x0 >= 1 && x0 + TX <= nx - 1 && y0 >= 1 && y0 + TY <= ny - 1)
-    collide_push_2d<T, R, FLOW, true, SX, true, CHM>(m, x, y, tx + 1, ty + 1, f, g, h,
-                                                sh_phi[ty + 1][tx + 1], dphi_prev,
-                                                &sh_phi[0][0], hs, NoUView{},
-                                                static_cast<T*>(dp.p[0]), ring_cur, err);
-  else
-    collide_push_2d<T, R, FLOW, false, SX, true, CHM>(m, x, y, tx + 1, ty + 1, f, g, h,
-                                                 sh_phi[ty + 1][tx + 1], dphi_prev,
-                                                 &sh_phi[0][0], hs, NoUView{},
-                                                 static_cast<T*>(dp.p[0]), ring_cur, err, solids);
+  R Unew;
+  const unsigned o = unsigned(ty * px + tx) * unsigned(sizeof(T));
+  auto work = [&](auto edge) {
+    collide_push_2d<T, R, FLOW, CHM, true, decltype(edge)::value, false, SX, 0>(
+        m, x, y, [&](int q) { return q < QF ? f[q] : g[q - QF]; }, h, sh_phi[ty + 1][tx + 1],
+        dphi_prev, &sh_phi[ty + 1][tx + 1],
+        [&](int a, int dy, int dx) { return sh_h[a][ty + 1 + dy][tx + 1 + dx]; },
+        [](int, int) { return R(0); }, R(coef<R>(m).ref_g),
+        static_cast<T*>(dp.p[0]) + (size_t(y0) * px + x0), o, o, err, Unew, solids);
+  };
+  if (solids || x0 < 1 || x0 + TX > nx - 1 || y0 < 1 || y0 + TY > ny - 1) work(std::true_type{});
+  else work(std::false_type{});
+  ring_cur[idx] = sh_phi[ty + 1][tx + 1];
 }
 
 // ---- TMA-pipelined persistent kernel ------------------------------------------
 
-// Pipeline depth and resident CTAs per SM of the persistent kernel.
-#ifndef LBPF_2D_STAGES
-#define LBPF_2D_STAGES 2
-#endif
-#ifndef LBPF_2D_MIN_CTAS
-#define LBPF_2D_MIN_CTAS 4
-#endif
-#ifndef LBPF_2D_TY
-#define LBPF_2D_TY 4
-#endif
-
-// MASK: the variant with the solid-node path (its extra registers held to
-// five CTAs per SM, which measured faster than four at more registers); CHM:
-// the central Hermite MRT flow collision (likewise).  CUR: how the threads
-// learn the origin of their CTA's next tile (below).
-template <typename T, bool FLOW, int TX, int TY, int S, bool MASK, bool CHM,
-          bool CUR = sizeof(T) == 2>
-__global__ void __launch_bounds__(TX* TY, (MASK || CHM) ? 5 : LBPF_2D_MIN_CTAS)
+// MASK: the variant with the solid-node path; CHM: the central Hermite MRT
+// flow collision; PAIR: two nodes per thread (step2d_tile.cuh).
+template <typename T, bool FLOW, int TX, int TY, bool PAIR, int S, bool MASK, bool CHM>
+__global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(), 4)
     step2d_tma_kernel(const __grid_constant__ CUtensorMap tm_fg,
                       const __grid_constant__ CUtensorMap tm_h,
                       const __grid_constant__ CUtensorMap tm_ring,
@@ -146,27 +147,17 @@ __global__ void __launch_bounds__(TX* TY, (MASK || CHM) ? 5 : LBPF_2D_MIN_CTAS)
   using R = float;
   using L = Tiles2D<T, FLOW, TX, TY>;
   constexpr int SX = TX + 2, SY = TY + 2;
-  extern __shared__ unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[S];
   __shared__ R sh_phi[SY][SX];
-  __shared__ int2 org[S];  // !CUR: origin of the tile in each stage
-  unsigned char* smem = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
 
   const int tid = threadIdx.x;
   const int first = blockIdx.x, G = gridDim.x;
 
-  // The CTA's tiles are first, first + G, first + 2G, ...  Their origins
-  // reach the threads without a division by ntx in every thread:
-  //  - CUR (16-bit storage): every thread steps the tile's column and row by
-  //    (G mod ntx, G div ntx) with one carry; thread 0 loads the tile S steps
-  //    ahead of the one being computed;
-  //  - otherwise (FP32): thread 0 divides once per tile it loads and writes the
-  //    origin into the stage's slot of org before it arrives on the stage's
-  //    mbarrier, whose completion publishes it to the other threads.
-  // Same-box timings of the 1024^2 coupled step (dividing in every thread /
-  // cursor / published origin): FP16 39.6 / 38.35 / 38.5 us, FP32 48.7 / 49.05
-  // (two more registers) / 48.5 us.
+  // The CTA's tiles are first, first + G, first + 2G, ... in row-major order.
+  // Columns and rows advance by (G mod ntx, G div ntx) with one carry, in
+  // uniform registers (every thread of the CTA has the same), so that the
+  // tile's origin is a uniform base of all its addresses.
   struct Cursor {
     int tile, col, row;
   };
@@ -180,41 +171,30 @@ __global__ void __launch_bounds__(TX* TY, (MASK || CHM) ? 5 : LBPF_2D_MIN_CTAS)
       ++q.row;
     }
   };
-  auto issue_xy = [&](int x0, int y0, int s) {
+  auto issue = [&](const Cursor& q, int s) {
     issue_tile_2d<T, FLOW, TX, TY>(&tm_fg, &tm_h, &tm_ring, &tm_uown, &tm_uhal, c, &full[s],
-                                   smem + s * L::STAGE, x0, y0);
-  };
-  auto issue_org = [&](int tile, int s) {  // thread 0, !CUR
-    const int2 o = make_int2((tile % ntx) * TX, (tile / ntx) * TY);
-    org[s] = o;
-    issue_xy(o.x, o.y, s);
+                                   smem + s * L::STAGE, q.col * TX, q.row * TY);
   };
   Cursor work{first, first % ntx, first / ntx};
+  Cursor load = work;  // the next tile to load, S tiles ahead of the work
 
   if (tid == 0) {
     for (int s = 0; s < S; ++s) mbar_init(&full[s], 1);
     fence_barrier_init();
   }
   __syncthreads();
-  if (tid == 0) {
-    if constexpr (CUR) {
-      Cursor q = work;
-      for (int k = 0; k < S && q.tile < ntiles; ++k) {
-        issue_xy(q.col * TX, q.row * TY, k);
-        advance(q);
-      }
-    } else {
-      for (int k = 0; k < S; ++k)
-        if (first + k * G < ntiles) issue_org(first + k * G, k);
-    }
+#pragma unroll
+  for (int k = 0; k < S; ++k) {
+    if (tid == 0 && load.tile < ntiles) issue(load, k);
+    advance(load);
   }
 
-  for (int k = 0;; ++k) {
-    const int tile = first + k * G;
-    if (tile >= ntiles) break;
+  for (int k = 0; work.tile < ntiles; ++k) {
     const int s = k % S;
     const bool ok = mbar_wait_bounded(&full[s], uint32_t((k / S) & 1), kSpin);
-    if (__syncthreads_or(!ok)) {
+    if (!tile_2d<T, FLOW, TX, TY, PAIR, MASK, CHM>(m, src, dst, ring_cur, err, work.col * TX,
+                                                   work.row * TY, c, smem + s * L::STAGE,
+                                                   &sh_phi[0][0], !ok)) {
       // a tile never arrived: report, let the copies in flight land, stop
       if (tid == 0) {
         atomicOr(err, 2u);
@@ -227,53 +207,45 @@ __global__ void __launch_bounds__(TX* TY, (MASK || CHM) ? 5 : LBPF_2D_MIN_CTAS)
       __syncthreads();
       return;
     }
-    int x0, y0;
-    if constexpr (CUR) {
-      x0 = work.col * TX;
-      y0 = work.row * TY;
-    } else {
-      const int2 o = org[s];
-      x0 = o.x;
-      y0 = o.y;
+    __syncthreads();  // stage s and sh_phi are free again
+    if (tid == 0 && load.tile < ntiles) {
+      fence_proxy_async_smem();
+      issue(load, s);
     }
-    tile_2d<T, FLOW, TX, TY, MASK, CHM>(m, src, dst, ring_cur, err, x0, y0, c,
-                                        smem + s * L::STAGE, &sh_phi[0][0]);
-    __syncthreads();  // stage s, its origin slot and sh_phi are free again
-    if constexpr (CUR) {
-      if (tid == 0) {
-        Cursor q = work;
-        for (int j = 0; j < S; ++j) advance(q);
-        if (q.tile < ntiles) {
-          fence_proxy_async_smem();
-          issue_xy(q.col * TX, q.row * TY, s);
-        }
-      }
-      advance(work);
-    } else {
-      if (tid == 0 && tile + S * G < ntiles) {
-        fence_proxy_async_smem();
-        issue_org(tile + S * G, s);
-      }
-    }
+    advance(load);
+    advance(work);
   }
 }
 
 // ---- host side: tensor maps and launches -------------------------------------------
-constexpr int kTX = 32, kTY = LBPF_2D_TY, kStages = LBPF_2D_STAGES;
+constexpr int kStages = 2;
+constexpr int kPairX = 64, kPairY = 4;    // tile with two nodes per thread
+constexpr int kPairTiles = 1500;          // fewest of them (about ten a SM)
+constexpr int kStageBytes = 142 * 1024;  // stages per SM where the state exceeds the L2
+constexpr int kSmallX = 32, kSmallY = 4;  // ... with one (small grids, and the FP64 kernel)
 
-// one thread per kTX x kTY tile: does the tile or its one-node halo (mapped
+// Does the step take the tiles with two nodes per thread?
+bool pair_tiles(const Model& m) {
+  if (m.storage == ST_FP64) return false;
+  return (long long)((m.nx + kPairX - 1) / kPairX) * ((m.ny + kPairY - 1) / kPairY) >=
+         kPairTiles;
+}
+
+// one thread per tx x ty tile: does the tile or its one-node halo (mapped
 // like the gradient stencil) hold a solid node?
-__global__ void solid_tiles_kernel(const Model m, unsigned char* flags, int ntx, int nty) {
+__global__ void solid_tiles_kernel(const Model m, unsigned char* flags, int ntx, int nty, int tx,
+                                   int ty) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= ntx * nty) return;
-  const int x0 = (t % ntx) * kTX, y0 = (t / ntx) * kTY;
+  const int x0 = (t % ntx) * tx, y0 = (t / ntx) * ty;
+  const int xe = x0 + tx < m.nx ? x0 + tx : m.nx, ye = y0 + ty < m.ny ? y0 + ty : m.ny;
   bool any = false;
-  for (int ly = -1; ly <= kTY; ++ly)
-    for (int lx = -1; lx <= kTX; ++lx) any |= solid_mapped(m, x0 + lx, y0 + ly);
+  for (int y = y0 - 1; y <= ye; ++y)
+    for (int x = x0 - 1; x <= xe; ++x) any |= solid_mapped(m, x, y);
   flags[t] = any ? 1 : 0;
 }
 
-template <typename T, bool FLOW>
+template <typename T, bool FLOW, int kTX, int kTY, bool PAIR>
 cudaError_t prepare_t(const Model& m, void* const pops[2], void* const rings[2], StepMaps* out) {
   using L = Tiles2D<T, FLOW, kTX, kTY>;
   const CUtensorMapDataType dt = pop_tensor_type(m.storage);
@@ -305,7 +277,7 @@ cudaError_t prepare_t(const Model& m, void* const pops[2], void* const rings[2],
     out->uown = out->ring[0];  // unused
     out->uhal = out->ring[0];
   }
-  const int smem = kStages * L::STAGE + 128;
+  const int smem = kStages * L::STAGE;
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -315,21 +287,35 @@ cudaError_t prepare_t(const Model& m, void* const pops[2], void* const rings[2],
     int per_sm = 0;
     cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (r == cudaSuccess)
-      r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTX * kTY, smem);
+      r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern,
+                                                        tile_threads<kTX, kTY, PAIR>(), smem);
     *ctas = sms * (per_sm > 0 ? per_sm : 1);
     return r;
   };
-  if ((e = setup(step2d_tma_kernel<T, FLOW, kTX, kTY, kStages, false, false>,
+  if ((e = setup(step2d_tma_kernel<T, FLOW, kTX, kTY, PAIR, kStages, false, false>,
                  &out->ctas_v[0])) != cudaSuccess ||
-      (e = setup(step2d_tma_kernel<T, FLOW, kTX, kTY, kStages, true, false>,
+      (e = setup(step2d_tma_kernel<T, FLOW, kTX, kTY, PAIR, kStages, true, false>,
                  &out->ctas_v[1])) != cudaSuccess)
     return e;
   if constexpr (FLOW) {  // the central Hermite MRT exists with flow only
-    if ((e = setup(step2d_tma_kernel<T, FLOW, kTX, kTY, kStages, false, true>,
+    if ((e = setup(step2d_tma_kernel<T, FLOW, kTX, kTY, PAIR, kStages, false, true>,
                    &out->ctas_v[2])) != cudaSuccess ||
-        (e = setup(step2d_tma_kernel<T, FLOW, kTX, kTY, kStages, true, true>,
+        (e = setup(step2d_tma_kernel<T, FLOW, kTX, kTY, PAIR, kStages, true, true>,
                    &out->ctas_v[3])) != cudaSuccess)
       return e;
+  }
+  // Populations and ring of both buffers beyond the L2: the copies in flight are
+  // held to kStageBytes a SM.  More of them make the memory slower (2480 x 2080
+  // FP32, 64 x 4 tiles, two stages: 199 us per step with two CTAs per SM, 224
+  // with three or four; 1024^2: 40.2 and 42.6); a state that the L2 holds is
+  // bound by the arithmetic and takes every CTA that fits (775 x 650 FP32: 18.6
+  // us with four, 20.5 with two; 1024^2 FP16: 28.9 and 34.5).
+  int l2 = 0;
+  if ((e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev)) != cudaSuccess) return e;
+  const double state = 2.0 * double(m.plane) * double(q * sizeof(T) + 4 + (L::REL ? 2 : 0));
+  if (state > double(l2)) {
+    const int most = std::max(1, kStageBytes / (kStages * L::STAGE));
+    for (int v = 0; v < 4; ++v) out->ctas_v[v] = std::min(out->ctas_v[v], sms * most);
   }
   out->ctas = out->ctas_v[0];
   out->smem = smem;
@@ -337,24 +323,26 @@ cudaError_t prepare_t(const Model& m, void* const pops[2], void* const rings[2],
   return cudaSuccess;
 }
 
-template <typename T, bool FLOW>
+template <typename T, bool FLOW, int kTX, int kTY, bool PAIR>
 cudaError_t launch_tma_t(const Model& m, const StepMaps& maps, int c, const void* src, void* dst,
                          void* ring_cur, unsigned* err, cudaStream_t s) {
   const int ntx = (m.nx + kTX - 1) / kTX, nty = (m.ny + kTY - 1) / kTY;
   const int ntiles = ntx * nty;
   const int v = (m.solid ? 1 : 0) + (FLOW && m.chm ? 2 : 0);
-  const int grid = ntiles < maps.ctas_v[v] ? ntiles : maps.ctas_v[v];
+  // a number of CTAs coprime to the tiles per row: every CTA then meets the
+  // (slower) edge columns equally often
+  int grid = ntiles < maps.ctas_v[v] ? ntiles : maps.ctas_v[v];
+  while (grid < ntiles && grid > 1 && std::gcd(grid, ntx) > 1) --grid;
   auto go = [&](auto kern) {
-    kern<<<grid, kTX * kTY, maps.smem, s>>>(maps.fg[c], maps.h[c], maps.ring[c], maps.uown,
-                                            maps.uhal, m, static_cast<const T*>(src),
-                                            static_cast<T*>(dst), static_cast<float*>(ring_cur),
-                                            err, ntx, ntiles, c);
+    kern<<<grid, tile_threads<kTX, kTY, PAIR>(), maps.smem, s>>>(
+        maps.fg[c], maps.h[c], maps.ring[c], maps.uown, maps.uhal, m, static_cast<const T*>(src),
+        static_cast<T*>(dst), static_cast<float*>(ring_cur), err, ntx, ntiles, c);
   };
-  if (v == 0) go(step2d_tma_kernel<T, FLOW, kTX, kTY, kStages, false, false>);
-  else if (v == 1) go(step2d_tma_kernel<T, FLOW, kTX, kTY, kStages, true, false>);
+  if (v == 0) go(step2d_tma_kernel<T, FLOW, kTX, kTY, PAIR, kStages, false, false>);
+  else if (v == 1) go(step2d_tma_kernel<T, FLOW, kTX, kTY, PAIR, kStages, true, false>);
   if constexpr (FLOW) {
-    if (v == 2) go(step2d_tma_kernel<T, FLOW, kTX, kTY, kStages, false, true>);
-    else if (v == 3) go(step2d_tma_kernel<T, FLOW, kTX, kTY, kStages, true, true>);
+    if (v == 2) go(step2d_tma_kernel<T, FLOW, kTX, kTY, PAIR, kStages, false, true>);
+    else if (v == 3) go(step2d_tma_kernel<T, FLOW, kTX, kTY, PAIR, kStages, true, true>);
   }
   return cudaGetLastError();
 }
@@ -362,6 +350,7 @@ cudaError_t launch_tma_t(const Model& m, const StepMaps& maps, int c, const void
 template <typename T, typename R, bool FLOW>
 cudaError_t launch_plain_t(const Model& m, const void* src, void* dst, const void* ring_prev,
                            void* ring_cur, unsigned* err, cudaStream_t s) {
+  constexpr int kTX = kSmallX, kTY = kSmallY;
   dim3 block(kTX, kTY);
   dim3 grid((m.nx + kTX - 1) / kTX, (m.ny + kTY - 1) / kTY);
   const PopPtrs sp = pop_ptrs(m, const_cast<void*>(src), sizeof(T));
@@ -375,33 +364,50 @@ cudaError_t launch_plain_t(const Model& m, const void* src, void* dst, const voi
   return cudaGetLastError();
 }
 
+template <typename T>
+cudaError_t prepare_any(const Model& m, void* const pops[2], void* const rings[2],
+                        StepMaps* out) {
+  if (pair_tiles(m))
+    return m.flow ? prepare_t<T, true, kPairX, kPairY, true>(m, pops, rings, out)
+                  : prepare_t<T, false, kPairX, kPairY, true>(m, pops, rings, out);
+  return m.flow ? prepare_t<T, true, kSmallX, kSmallY, false>(m, pops, rings, out)
+                : prepare_t<T, false, kSmallX, kSmallY, false>(m, pops, rings, out);
+}
+
+template <typename T>
+cudaError_t launch_any(const Model& m, const StepMaps& maps, int c, const void* src, void* dst,
+                       void* ring_cur, unsigned* err, cudaStream_t s) {
+  if (pair_tiles(m))
+    return m.flow
+               ? launch_tma_t<T, true, kPairX, kPairY, true>(m, maps, c, src, dst, ring_cur, err, s)
+               : launch_tma_t<T, false, kPairX, kPairY, true>(m, maps, c, src, dst, ring_cur, err, s);
+  return m.flow ? launch_tma_t<T, true, kSmallX, kSmallY, false>(m, maps, c, src, dst, ring_cur, err, s)
+                : launch_tma_t<T, false, kSmallX, kSmallY, false>(m, maps, c, src, dst, ring_cur, err, s);
+}
+
 }  // namespace
 
 cudaError_t prepare_step2d(const Model& m, void* const pops[2], void* const rings[2],
                            StepMaps* out) {
   out->ready = 0;
-  if (m.storage == ST_FP64) return cudaSuccess;  // one-tile kernel, no maps
   switch (m.storage) {
-    case ST_FP16:
-      return m.flow ? prepare_t<__half, true>(m, pops, rings, out)
-                    : prepare_t<__half, false>(m, pops, rings, out);
-    case ST_BF16:
-      return m.flow ? prepare_t<__nv_bfloat16, true>(m, pops, rings, out)
-                    : prepare_t<__nv_bfloat16, false>(m, pops, rings, out);
-    default:
-      return m.flow ? prepare_t<float, true>(m, pops, rings, out)
-                    : prepare_t<float, false>(m, pops, rings, out);
+    case ST_FP64: return cudaSuccess;  // one-tile kernel, no maps
+    case ST_FP16: return prepare_any<__half>(m, pops, rings, out);
+    case ST_BF16: return prepare_any<__nv_bfloat16>(m, pops, rings, out);
+    default: return prepare_any<float>(m, pops, rings, out);
   }
 }
 
 size_t solid_tile_count(const Model& m) {
-  return size_t((m.nx + kTX - 1) / kTX) * size_t((m.ny + kTY - 1) / kTY);
+  const int tx = pair_tiles(m) ? kPairX : kSmallX, ty = pair_tiles(m) ? kPairY : kSmallY;
+  return size_t((m.nx + tx - 1) / tx) * size_t((m.ny + ty - 1) / ty);
 }
 
 cudaError_t launch_solid_tiles(const Model& m, unsigned char* flags, cudaStream_t s) {
   if (m.dim != 2 || !m.solid) return cudaErrorInvalidValue;
-  const int ntx = (m.nx + kTX - 1) / kTX, nty = (m.ny + kTY - 1) / kTY;
-  solid_tiles_kernel<<<(ntx * nty + 127) / 128, 128, 0, s>>>(m, flags, ntx, nty);
+  const int tx = pair_tiles(m) ? kPairX : kSmallX, ty = pair_tiles(m) ? kPairY : kSmallY;
+  const int ntx = (m.nx + tx - 1) / tx, nty = (m.ny + ty - 1) / ty;
+  solid_tiles_kernel<<<(ntx * nty + 127) / 128, 128, 0, s>>>(m, flags, ntx, nty, tx, ty);
   return cudaGetLastError();
 }
 
@@ -412,15 +418,9 @@ cudaError_t launch_step2d(const Model& m, const StepMaps& maps, int c, const voi
                   : launch_plain_t<double, double, false>(m, src, dst, ring_prev, ring_cur, err, s);
   if (!maps.ready) return cudaErrorNotReady;
   switch (m.storage) {
-    case ST_FP16:
-      return m.flow ? launch_tma_t<__half, true>(m, maps, c, src, dst, ring_cur, err, s)
-                    : launch_tma_t<__half, false>(m, maps, c, src, dst, ring_cur, err, s);
-    case ST_BF16:
-      return m.flow ? launch_tma_t<__nv_bfloat16, true>(m, maps, c, src, dst, ring_cur, err, s)
-                    : launch_tma_t<__nv_bfloat16, false>(m, maps, c, src, dst, ring_cur, err, s);
-    default:
-      return m.flow ? launch_tma_t<float, true>(m, maps, c, src, dst, ring_cur, err, s)
-                    : launch_tma_t<float, false>(m, maps, c, src, dst, ring_cur, err, s);
+    case ST_FP16: return launch_any<__half>(m, maps, c, src, dst, ring_cur, err, s);
+    case ST_BF16: return launch_any<__nv_bfloat16>(m, maps, c, src, dst, ring_cur, err, s);
+    default: return launch_any<float>(m, maps, c, src, dst, ring_cur, err, s);
   }
 }
 

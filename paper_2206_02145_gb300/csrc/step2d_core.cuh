@@ -9,36 +9,6 @@
 
 namespace lbk {
 
-// Shared-memory view of the halo-extended tile: value of lattice direction a
-// at local position (lx, ly) (lx, ly in [0, TX + 1] x [0, TY + 1]).  The
-// shape is compile-time, so every access is one load with an immediate
-// offset from a per-thread base.
-template <typename T, typename R, int ROW, int PLANE, int XOFF>
-struct TileView {
-  const T* base;
-  __device__ __forceinline__ R at(int a, int ly, int lx) const {
-    return Pop<T>::template ld<R>(base + a * PLANE + ly * ROW + lx + XOFF);
-  }
-};
-
-// The per-node g reference around a node (2D, 16-bit storage): `own` the
-// reference of the node's own populations, at(ly, lx) the encoding reference
-// of the node at local (ly, lx) (halo box of row pitch ROW, the pointer
-// offset so that lx = 0 is the tile's left halo column), `out` the plane that
-// receives each node's new U.  With REL = false (FP32 and FP64 storage) g is
-// relative to the global U_ref and every member is unused.
-template <bool REL, int ROW>
-struct UView {
-  static constexpr bool kRel = REL;
-  const __half* hal;
-  __half* out;
-  float own;
-  __device__ __forceinline__ float at(int ly, int lx) const {
-    return REL ? __half2float(hal[ly * ROW + lx]) : 0.f;
-  }
-};
-using NoUView = UView<false, 1>;
-
 // Solid nodes (2D mask): is the node at (x, y), mapped like a gradient
 // neighbour (periodic wrap, else nearest node), solid?
 __device__ __forceinline__ bool solid_mapped(const Model& m, int x, int y) {
@@ -56,276 +26,442 @@ __device__ __forceinline__ bool solid_mapped(const Model& m, int x, int y) {
 // keeps the small quantities: raw moments e_pq -> central Hermite moments
 // about u* -> relaxation by order -> raw moments -> populations through the
 // inverse of the D2Q9 raw-moment matrix.  out: post-collision deviations.
-template <typename R>
-__device__ __forceinline__ void chm_post_2d(const R (&d)[9], R drho, R rho, R mx, R my, R vx,
-                                            R vy, R Fx, R Fy, R wf, R wb, R wh, R (&out)[9]) {
-  const R t3 = R(1.0 / 3.0), t9 = R(1.0 / 9.0);
+template <typename N>
+__device__ __forceinline__ void chm_post_2d(const N (&d)[9], N drho, N rho, N mx, N my, N vx, N vy,
+                                            N Fx, N Fy, typename Lanes<N>::S wf,
+                                            typename Lanes<N>::S wb, typename Lanes<N>::S wh,
+                                            typename Lanes<N>::S mzero, N (&out)[9]) {
+  using S = typename Lanes<N>::S;
+  const N t3 = splat<N>(S(1.0 / 3.0)), t9 = splat<N>(S(1.0 / 9.0)), two = splat<N>(S(2));
+  const N t23 = splat<N>(S(2) * S(1.0 / 3.0)), half = splat<N>(S(0.5)), quarter = splat<N>(S(0.25));
+  // a sum of products: add(p, q, s) = s + p q, sub(p, q, s) = s - p q
+  auto add = [](N p, N q, N s) { return fma_r(p, q, s); };
+  auto sub = [](N p, N q, N s) { return fma_r(neg_r(p), q, s); };
   // raw moments of the deviations
-  const R e00 = drho, e10 = mx, e01 = my;
-  const R dd = (d[5] + d[6]) + (d[7] + d[8]);
-  const R e20 = (d[1] + d[3]) + dd, e02 = (d[2] + d[4]) + dd;
-  const R e11 = (d[5] - d[6]) + (d[7] - d[8]);
-  const R e21 = (d[5] + d[6]) - (d[7] + d[8]);
-  const R e12 = (d[5] - d[6]) - (d[7] - d[8]);
-  const R e22 = dd;
-  const R vxx = vx * vx, vyy = vy * vy, vxy = vx * vy;
+  const N e00 = drho, e10 = mx, e01 = my;
+  const N dd = add_r(add_r(d[5], d[6]), add_r(d[7], d[8]));
+  const N e20 = add_r(add_r(d[1], d[3]), dd), e02 = add_r(add_r(d[2], d[4]), dd);
+  const N e11 = add_r(sub_r(d[5], d[6]), sub_r(d[7], d[8]));
+  const N e21 = sub_r(add_r(d[5], d[6]), add_r(d[7], d[8]));
+  const N e12 = sub_r(sub_r(d[5], d[6]), sub_r(d[7], d[8]));
+  const N e22 = dd;
+  const N vxx = mul_r(vx, vx), vyy = mul_r(vy, vy), vxy = mul_r(vx, vy);
+  const N vx2 = mul_r(two, vx), vy2 = mul_r(two, vy), vxy2 = mul_r(two, vxy);
+  const N vxy4 = mul_r(splat<N>(S(4)), vxy), vxxy = mul_r(vxx, vy), vxyy = mul_r(vx, vyy);
+  const N vxy2y = mul_r(vxy2, vy), vxy2x = mul_r(vxy2, vx), vxxyy = mul_r(vxx, vyy);
   // central Hermite moments about (vx, vy)
-  const R h1 = e10 - vx * rho, h2 = e01 - vy * rho;
-  const R hxx = e20 - t3 * e00 - R(2) * vx * e10 + vxx * rho;
-  const R hyy = e02 - t3 * e00 - R(2) * vy * e01 + vyy * rho;
-  const R hxy = e11 - vx * e01 - vy * e10 + vxy * rho;
-  const R hxxy = e21 - R(2) * vx * e11 + vxx * e01 - vy * e20 + R(2) * vxy * e10 -
-                 vxx * vy * rho - t3 * e01 + t3 * vy * e00;
-  const R hxyy = e12 - R(2) * vy * e11 + vyy * e10 - vx * e02 + R(2) * vxy * e01 -
-                 vx * vyy * rho - t3 * e10 + t3 * vx * e00;
-  const R hxxyy = e22 - R(2) * vx * e12 - R(2) * vy * e21 + vxx * e02 + vyy * e20 +
-                  R(4) * vxy * e11 - R(2) * vxy * vy * e10 - R(2) * vxy * vx * e01 +
-                  vxx * vyy * rho - t3 * (e20 + e02) + R(2) * t3 * (vx * e10 + vy * e01) -
-                  t3 * (vxx + vyy) * e00 + t9 * e00;
+  const N h1 = sub(vx, rho, e10), h2 = sub(vy, rho, e01);
+  const N hxx = add(vxx, rho, sub(vx2, e10, sub(t3, e00, e20)));
+  const N hyy = add(vyy, rho, sub(vy2, e01, sub(t3, e00, e02)));
+  const N hxy = add(vxy, rho, sub(vy, e10, sub(vx, e01, e11)));
+  const N hxxy = add(mul_r(t3, vy), e00,
+                     sub(t3, e01,
+                         sub(vxxy, rho,
+                             add(vxy2, e10, sub(vy, e20, add(vxx, e01, sub(vx2, e11, e21)))))));
+  const N hxyy = add(mul_r(t3, vx), e00,
+                     sub(t3, e10,
+                         sub(vxyy, rho,
+                             add(vxy2, e01, sub(vx, e02, add(vyy, e10, sub(vy2, e11, e12)))))));
+  N hxxyy = sub(vy2, e21, sub(vx2, e12, e22));
+  hxxyy = add(vxy4, e11, add(vyy, e20, add(vxx, e02, hxxyy)));
+  hxxyy = add(vxxyy, rho, sub(vxy2x, e01, sub(vxy2y, e10, hxxyy)));
+  hxxyy = add(t23, fma_r(vx, e10, mul_r(vy, e01)), sub(t3, add_r(e20, e02), hxxyy));
+  hxxyy = add(t9, e00, sub(mul_r(t3, fma_r(vx, vx, vyy)), e00, hxxyy));
   // relaxation towards rho and zeros; the force in the first order
-  const R kf = R(1) - wf, gf = R(1) - R(0.5) * wf, kh = R(1) - wh;
-  const R h1s = kf * h1 + gf * Fx, h2s = kf * h2 + gf * Fy;
-  const R tr = (R(1) - wb) * (hxx + hyy), dv = kf * (hxx - hyy);
-  const R hxxs = R(0.5) * (tr + dv), hyys = R(0.5) * (tr - dv);
-  const R hxys = kf * hxy;
-  const R hxxys = kh * hxxy, hxyys = kh * hxyy, hxxyys = kh * hxxyy;
+  const N kf = splat<N>(S(1) - wf), gf = splat<N>(S(1) - S(0.5) * wf), kh = splat<N>(S(1) - wh);
+  const N kb = splat<N>(S(1) - wb);
+  const N h1s = fma_r(kf, h1, mul_r(gf, Fx)), h2s = fma_r(gf, Fy, mul_r(kf, h2));
+  const N sum = add_r(hxx, hyy), dv = mul_r(kf, sub_r(hxx, hyy));
+  const N hxxs = mul_r(half, fma_r(kb, sum, dv)), hyys = mul_r(half, fma_r(kb, sum, neg_r(dv)));
+  const N hxys = mul_r(kf, hxy);
   // central (raw) moments after collision, then raw moments of the deviations
-  const R k20 = hxxs + t3 * rho, k02 = hyys + t3 * rho;
-  const R k21 = hxxys + t3 * h2s, k12 = hxyys + t3 * h1s;
-  const R f10 = h1s + vx * rho, f01 = h2s + vy * rho;
-  const R f20 = hxxs + t3 * e00 + R(2) * vx * h1s + vxx * rho;
-  const R f02 = hyys + t3 * e00 + R(2) * vy * h2s + vyy * rho;
-  const R f11 = hxys + vx * h2s + vy * h1s + vxy * rho;
-  const R f21 = k21 + R(2) * vx * hxys + vxx * h2s + vy * k20 + R(2) * vxy * h1s + vxx * vy * rho;
-  const R f12 = k12 + R(2) * vy * hxys + vyy * h1s + vx * k02 + R(2) * vxy * h2s + vx * vyy * rho;
-  const R f22 = hxxyys + t3 * (hxxs + hyys) + t9 * e00 + R(2) * vx * k12 + R(2) * vy * k21 +
-                vxx * k02 + vyy * k20 + R(4) * vxy * hxys + R(2) * vxy * vy * h1s +
-                R(2) * vxy * vx * h2s + vxx * vyy * rho;
+  const N k20 = add(t3, rho, hxxs), k02 = add(t3, rho, hyys);
+  const N k21 = fma_r(t3, h2s, mul_r(kh, hxxy)), k12 = fma_r(t3, h1s, mul_r(kh, hxyy));
+  const N t3e = prod_r(t3, e00, mzero);
+  const N f10 = add(vx, rho, h1s), f01 = add(vy, rho, h2s);
+  const N f20 = add(vxx, rho, add(vx2, h1s, add_r(hxxs, t3e)));
+  const N f02 = add(vyy, rho, add(vy2, h2s, add_r(hyys, t3e)));
+  const N f11 = add(vxy, rho, add(vy, h1s, add(vx, h2s, hxys)));
+  const N f21 =
+      add(vxxy, rho, add(vxy2, h1s, add(vy, k20, add(vxx, h2s, add(vx2, hxys, k21)))));
+  const N f12 =
+      add(vxyy, rho, add(vxy2, h2s, add(vx, k02, add(vyy, h1s, add(vy2, hxys, k12)))));
+  N f22 = fma_r(kh, hxxyy, mul_r(t3, add_r(hxxs, hyys)));
+  f22 = add(vy2, k21, add(vx2, k12, add(t9, e00, f22)));
+  f22 = add(vxy4, hxys, add(vyy, k20, add(vxx, k02, f22)));
+  f22 = add(vxxyy, rho, add(vxy2x, h2s, add(vxy2y, h1s, f22)));
   // populations (D2Q9 order: rest, +x, +y, -x, -y, ++, -+, --, +-)
-  out[0] = e00 - f20 - f02 + f22;
-  out[1] = R(0.5) * (f10 + f20 - f12 - f22);
-  out[3] = R(0.5) * (-f10 + f20 + f12 - f22);
-  out[2] = R(0.5) * (f01 + f02 - f21 - f22);
-  out[4] = R(0.5) * (-f01 + f02 + f21 - f22);
-  out[5] = R(0.25) * (f11 + f21 + f12 + f22);
-  out[6] = R(0.25) * (-f11 + f21 - f12 + f22);
-  out[7] = R(0.25) * (f11 - f21 - f12 + f22);
-  out[8] = R(0.25) * (-f11 - f21 + f12 + f22);
+  out[0] = add_r(sub_r(sub_r(e00, f20), f02), f22);
+  out[1] = mul_r(half, sub_r(sub_r(add_r(f10, f20), f12), f22));
+  out[3] = mul_r(half, sub_r(add_r(sub_r(f20, f10), f12), f22));
+  out[2] = mul_r(half, sub_r(sub_r(add_r(f01, f02), f21), f22));
+  out[4] = mul_r(half, sub_r(add_r(sub_r(f02, f01), f21), f22));
+  out[5] = mul_r(quarter, add_r(add_r(add_r(f11, f21), f12), f22));
+  out[6] = mul_r(quarter, add_r(sub_r(sub_r(f21, f11), f12), f22));
+  out[7] = mul_r(quarter, add_r(sub_r(sub_r(f11, f21), f12), f22));
+  out[8] = mul_r(quarter, add_r(sub_r(f12, add_r(f11, f21)), f22));
 }
 
-// dphi_prev: phi(t-1) + 1 of this node; ring_cur: where phi(t) + 1 goes.
-// phi_s: the tile's phi + 1 with halo ([ly][lx], row pitch PROW).
-// dst: the destination population buffer (array a at dst + a * plane).
-// INTERIOR: the caller guarantees 1 <= x <= nx - 2 and 1 <= y <= ny - 2 for
-// every node of the tile, so every destination is an ordinary node (no wrap,
-// wall or ghost) and the push needs no boundary logic.  MASK: the code for
-// solid nodes is compiled in; `solids` (the tile holds or borders a solid
-// node) switches it on.  CHM: the flow collides by the central Hermite MRT.
-template <typename T, typename R, bool FLOW, bool INTERIOR, int PROW, bool MASK, bool CHM,
-          typename HV, typename UV>
-__device__ __forceinline__ void collide_push_2d(const Model& m, int x, int y, int lx, int ly,
-                                                const R (&f)[9], const R (&g)[9],
-                                                const R (&h)[9], R dphi, R dphi_prev,
-                                                const R* phi_s, const HV& hs, const UV& uh,
-                                                T* __restrict__ dst, R* __restrict__ ring_cur,
-                                                unsigned* __restrict__ err,
-                                                bool solids = false) {
-  constexpr int QF = FLOW ? 9 : 0;
-  const int nx = m.nx, ny = m.ny, px = m.px;
-  const int P = int(m.plane);  // fits: checked at creation
-  const int idx = y * px + x;
-  T* const pd = dst + idx;  // this node in array 0; the offsets below are uniform
-  const Coef<R>& c = coef<R>(m);
+// What the collisions of one node (or of a thread's two nodes, N = float2)
+// need, so that each direction costs a few FMAs:
+//   f*: (1 - w_f) d + w_f w [E0 + cu (E1 + E2 cu)] + guo w [cF (3 + 9 cu) - 3 u*.F]
+//       (Eq. 4, 5, 8, 9 with c_s^2 = 1/3, d = f - w)
+//   g*: (1 - w_U) d + w (K0 + K1 cu)            (Eqs. 13-16, d = g - w U_ref)
+//   h*: (1 - w_phi) d + w (H0 - c.H)            (Eqs. 19-21, d = h + w)
+// The order and rounding of every operation is written out (fma_r, mul_r,
+// add_r), so that one and two nodes per thread give the same bits.
+template <typename N>
+struct Node2D {
+  using S = typename Lanes<N>::S;
+  N U;                                 // Eq. 17
+  N usx, usy, Fx, Fy, E0, E1, E2, G0;  // flow (with the central Hermite MRT unused)
+  N keep_U, K0, K1, keep_phi, H0, Hx, Hy, inv_a2, keep_old;
+  N us_s, us_d, F_s, F_d, H_s, H_d;    // sums and differences of the two components
+  S keep_f, guo, mzero;
+};
 
+// Moments, gradient, anisotropy and the coefficients above (Eqs. 3-23) of a
+// node with population deviations f, g, phi + 1 = dphi (dphi_prev one step
+// earlier), the g reference Rg and the eight neighbours' phi + 1.  False if
+// phi, U or rho is not finite.
+template <typename N, bool FLOW, bool CHM>
+__device__ __forceinline__ bool node_2d(const Model& m, const N (&f)[9], const N (&g)[9], N dphi,
+                                        N dphi_prev, N Rg, N pE, N pW, N pN, N pS, N pNE, N pNW,
+                                        N pSE, N pSW, Node2D<N>& o, N (&fchm)[9]) {
+  using S = typename Lanes<N>::S;
+  const Coef<S>& c = coef<S>(m);
+  const N one = splat<N>(S(1)), half = splat<N>(S(0.5));
   // ---- local moments (Eqs. 11, 12, 17, 22) ----------------------------------
-  const R phi = dphi - R(1);
-  R dU = R(0);
+  const N phi = sub_r(dphi, one);
+  N dU = g[0];
 #pragma unroll
-  for (int a = 0; a < 9; ++a) dU += g[a];
+  for (int a = 1; a < 9; ++a) dU = add_r(dU, g[a]);
   // g deviations are taken from w_a Rg; the collision (Eqs. 13-16) is linear
   // in them, so any per-node Rg gives the same populations
-  const R Rg = UV::kRel ? R(uh.own) : c.ref_g;
-  const R U = Rg + dU;
-  R drho = R(0), mx = R(0), my = R(0);
+  const N U = o.U = add_r(Rg, dU);
+  N drho = splat<N>(S(0)), mx = drho, my = drho;
   if (FLOW) {
+    drho = f[0];
 #pragma unroll
-    for (int a = 0; a < 9; ++a) drho += f[a];
-    mx = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
-    my = (f[2] - f[4]) + (f[5] + f[6]) - (f[7] + f[8]);
+    for (int a = 1; a < 9; ++a) drho = add_r(drho, f[a]);
+    mx = add_r(add_r(sub_r(f[1], f[3]), sub_r(f[5], f[6])), sub_r(f[8], f[7]));
+    my = sub_r(add_r(sub_r(f[2], f[4]), add_r(f[5], f[6])), add_r(f[7], f[8]));
   }
-  const R rho = R(1) + drho;
-  const R ph = clamp1(phi);
-  const R mask = R(0.5) * (R(1) - ph);  // (1 - phi)/2 of Eq. 7 and q(phi) of Eq. 18
-  R ux = R(0), uy = R(0), Fx = R(0), Fy = R(0);
+  const N rho = add_r(one, drho);
+  const bool ok = all_finite(phi, U, rho);
+  const N ph = clamp1(phi);
+  const N mask = mul_r(half, sub_r(one, ph));  // (1 - phi)/2 of Eq. 7 and q(phi) of Eq. 18
+  o.usx = o.usy = o.Fx = o.Fy = splat<N>(S(0));
   if (FLOW) {
     // Eq. 6: F = b - K u, K = h tau_f (1+phi)^2 (1-phi) / (4 W0^2); the Guo
     // half-force velocity u = (m + F/2)/rho solved in closed form.
-    const R K = c.kdrag * (R(1) + ph) * (R(1) + ph) * (R(1) - ph);
-    const R inv = rcp_r(rho + R(0.5) * K);
-    ux = (mx + R(0.5) * c.body[0]) * inv;
-    uy = (my + R(0.5) * c.body[1]) * inv;
-    Fx = c.body[0] - K * ux;
-    Fy = c.body[1] - K * uy;
+    const N ph1 = add_r(one, ph);
+    const N K = mul_r(mul_r(mul_r(splat<N>(c.kdrag), ph1), ph1), sub_r(one, ph));
+    const N inv = rcp_r(fma_r(half, K, rho));
+    const N ux = mul_r(fma_r(half, splat<N>(c.body[0]), mx), inv);
+    const N uy = mul_r(fma_r(half, splat<N>(c.body[1]), my), inv);
+    o.Fx = fma_r(neg_r(K), ux, splat<N>(c.body[0]));
+    o.Fy = fma_r(neg_r(K), uy, splat<N>(c.body[1]));
+    o.usx = mul_r(mask, ux);  // u* (Eq. 7)
+    o.usy = mul_r(mask, uy);
   }
-  const R usx = mask * ux, usy = mask * uy;  // u* (Eq. 7)
-  R fchm[9];
-  if (FLOW && CHM)
-    chm_post_2d<R>(f, drho, rho, mx, my, usx, usy, Fx, Fy, c.omega_f, c.chm_wb, c.chm_wh, fchm);
-  const R omega_U = rcp_r(R(0.5) + c.tauU_slope * mask);  // Eq. 18
-  const R dphidt = dphi - dphi_prev;
-  ring_cur[idx] = dphi;
-  if (UV::kRel) uh.out[idx] = __float2half_rn(float(U));
-  if (!(finite_r(phi) && finite_r(U) && finite_r(rho))) atomicOr(err, 1u);
-  // a g deviation pushed to the node at local (dly, dlx), taken from its
-  // reference there instead of this node's
-  auto genc = [&](R v, R w, int dly, int dlx) -> R {
-    return UV::kRel ? fma_r(-w, R(uh.at(dly, dlx)) - Rg, v) : v;
-  };
+  if constexpr (FLOW && CHM)
+    chm_post_2d<N>(f, drho, rho, mx, my, o.usx, o.usy, o.Fx, o.Fy, c.omega_f, c.chm_wb, c.chm_wh,
+                   c.mzero, fchm);
+  const N omega_U = rcp_r(fma_r(splat<N>(c.tauU_slope), mask, half));  // Eq. 18
+  const N dphidt = sub_r(dphi, dphi_prev);
 
   // ---- gradient, anisotropy, phase-field coefficients (Eqs. 3, 20, 21, 23) --
-  const R* pc = phi_s + ly * PROW + lx;
-  R pE = pc[1], pW = pc[-1], pN = pc[PROW], pS = pc[-PROW];
-  R pNE = pc[PROW + 1], pNW = pc[PROW - 1], pSE = pc[-PROW + 1], pSW = pc[-PROW - 1];
-  if (MASK && !INTERIOR && solids) {
+  // grad = 3 sum_a w_a c_a phi(x + c_a) over D2Q9
+  const N third = splat<N>(S(1.0 / 3.0)), twelfth = splat<N>(S(1.0 / 12.0));
+  const N gx = fma_r(third, sub_r(pE, pW),
+                     mul_r(twelfth, sub_r(add_r(pNE, pSE), add_r(pNW, pSW))));
+  const N gy = fma_r(third, sub_r(pN, pS),
+                     mul_r(twelfth, sub_r(add_r(pNE, pNW), add_r(pSE, pSW))));
+  N as, Nx, Ny;
+  aniso_2d<N>(m, gx, gy, as, Nx, Ny);
+  const N a2 = mul_r(as, as);
+  o.inv_a2 = rcp_r(a2);
+  const N tpc = splat<N>(c.tpc);
+  const N omega_phi = rcp_r(fma_r(a2, tpc, half));  // Eq. 23
+  const N pp = mul_r(phi, phi);
+  const N phi2m = sub_r(one, pp);
+  // Eq. 20
+  const N Qs = mul_r(fma_r(mul_r(mul_r(splat<N>(c.lambda), U), phi2m), phi2m,
+                           fma_r(neg_r(pp), phi, phi)),
+                     splat<N>(c.inv_tau0));
+  if (FLOW && !CHM) {
+    const N uu = fma_r(o.usx, o.usx, mul_r(o.usy, o.usy));
+    const N uF = fma_r(o.usx, o.Fx, mul_r(o.usy, o.Fy));
+    o.E0 = mul_r(splat<N>(c.omega_f), fma_r(neg_r(mul_r(splat<N>(S(1.5)), rho)), uu, drho));
+    o.E1 = mul_r(splat<N>(c.omega_f * S(3)), rho);
+    o.E2 = mul_r(splat<N>(c.omega_f * S(4.5)), rho);
+    o.G0 = mul_r(splat<N>(S(-3)), uF);
+    o.F_s = add_r(o.Fx, o.Fy);
+    o.F_d = sub_r(o.Fx, o.Fy);
+    o.keep_f = S(1) - c.omega_f;
+    o.guo = c.guo;
+    o.mzero = c.mzero;
+  }
+  o.us_s = add_r(o.usx, o.usy);
+  o.us_d = sub_r(o.usx, o.usy);
+  o.keep_U = sub_r(one, omega_U);
+  o.K0 = fma_r(omega_U, dU, neg_r(dphidt));
+  o.K1 = mul_r(mul_r(splat<N>(S(3)), omega_U), U);
+  o.keep_phi = sub_r(one, omega_phi);
+  o.H0 = fma_r(omega_phi, dphi, Qs);
+  const N wt = mul_r(omega_phi, tpc);
+  o.Hx = mul_r(wt, Nx);
+  o.Hy = mul_r(wt, Ny);
+  o.H_s = add_r(o.Hx, o.Hy);
+  o.H_d = sub_r(o.Hx, o.Hy);
+  // Eq. 19: h_new = h* / a_s^2 + (1 - 1/a_s^2) h_old
+  o.keep_old = sub_r(one, o.inv_a2);
+  return ok;
+}
+
+// c_a . v from the components and their sum and difference (a a constant
+// after unrolling; not for the rest direction)
+template <typename N>
+__device__ __forceinline__ N dir_dot(int a, N x, N y, N s, N d) {
+  switch (a) {
+    case 1: return x;
+    case 2: return y;
+    case 3: return neg_r(x);
+    case 4: return neg_r(y);
+    case 5: return s;
+    case 6: return neg_r(d);
+    case 7: return neg_r(s);
+    default: return d;
+  }
+}
+
+// Post-collision deviations of direction a at the node: f* (Eq. 4), g* (Eq.
+// 13) and, before Eq. 19's division by a_s^2, h*.
+template <typename N>
+__device__ __forceinline__ N post_f_2d(const Node2D<N>& n, int a, N f) {
+  using S = typename Lanes<N>::S;
+  const N w = splat<N>(d2_w<S>(a)), keep = splat<N>(n.keep_f), guo = splat<N>(n.guo);
+  N feq = n.E0, gt = n.G0;
+  if (a > 0) {
+    const N cu = dir_dot(a, n.usx, n.usy, n.us_s, n.us_d);
+    const N cF = dir_dot(a, n.Fx, n.Fy, n.F_s, n.F_d);
+    feq = fma_r(cu, fma_r(n.E2, cu, n.E1), n.E0);
+    gt = fma_r(cF, fma_r(splat<N>(S(9)), cu, splat<N>(S(3))), n.G0);
+  }
+  return fma_r(keep, f, mul_r(w, add_r(feq, prod_r(guo, gt, n.mzero))));
+}
+template <typename N>
+__device__ __forceinline__ N post_g_2d(const Node2D<N>& n, int a, N g) {
+  using S = typename Lanes<N>::S;
+  const N w = splat<N>(d2_w<S>(a));
+  N e = n.K0;
+  if (a > 0) e = fma_r(n.K1, dir_dot(a, n.usx, n.usy, n.us_s, n.us_d), n.K0);
+  return fma_r(n.keep_U, g, mul_r(w, e));
+}
+template <typename N>
+__device__ __forceinline__ N post_h_2d(const Node2D<N>& n, int a, N h) {
+  using S = typename Lanes<N>::S;
+  const N w = splat<N>(d2_w<S>(a));
+  N e = n.H0;
+  if (a > 0) e = sub_r(n.H0, dir_dot(a, n.Hx, n.Hy, n.H_s, n.H_d));
+  return fma_r(n.keep_phi, h, mul_r(w, e));
+}
+// Eq. 19 at the destination, whose old value is hold
+template <typename N>
+__device__ __forceinline__ N arrive_h_2d(const Node2D<N>& n, N hp, N hold) {
+  return fma_r(n.inv_a2, hp, mul_r(n.keep_old, hold));
+}
+
+// lane k of a number of one or two nodes
+template <typename N>
+__device__ __forceinline__ typename Lanes<N>::S lane(const N& v, int k) {
+  if constexpr (Lanes<N>::V == 2) return k ? v.y : v.x;
+  else return v;
+}
+template <typename N>
+__device__ __forceinline__ void set_lane(N& v, int k, typename Lanes<N>::S s) {
+  if constexpr (Lanes<N>::V == 2) (k ? v.y : v.x) = s;
+  else v = s;
+}
+
+// Collide and push a thread's one or two nodes (N = float2: the second DY rows
+// below the first).
+//   own(q): stored deviation q of the node(s) (f, then g)
+//   pc: phi + 1 of the first node in the tile (row pitch PROW); dphi,
+//     dphi_prev: phi + 1 of the node(s) now and one step earlier
+//   hold(a, dy, dx), uref(dy, dx): h_a and the encoding reference of g (UREL) at
+//     that offset from the node(s)
+//   (x, y): the first node; tb: the tile's origin in array 0 of the
+//     destination buffer (the same for the whole CTA, so that every array's
+//     address is one uniform base plus the thread's offset); o0, o1: offsets
+//     of the node(s) from it, in bytes
+// EDGE = false: every destination is an ordinary node (the tile lies at least
+// one node away from every domain edge and holds or borders no solid node), so
+// the push needs no boundary logic.  EDGE = true: each destination goes through
+// the boundary rules; nodes outside the domain (of a partial tile) and solid
+// nodes push nothing.  MASK: the code for solid nodes is compiled in; `solids`
+// (the tile holds or borders a solid node) switches it on.  CHM: the flow
+// collides by the central Hermite MRT.
+template <typename T, typename N, bool FLOW, bool CHM, bool MASK, bool EDGE, bool UREL, int PROW,
+          int DY, typename Own, typename Hold, typename Uref>
+__device__ __forceinline__ void collide_push_2d(
+    const Model& m, int x, int y, const Own& own, const N (&h)[9], N dphi, N dphi_prev,
+    const typename Lanes<N>::S* pc, const Hold& hold, const Uref& uref, N Rg, T* __restrict__ tb,
+    unsigned o0, unsigned o1, unsigned* __restrict__ err, N& Unew, bool solids) {
+  using S = typename Lanes<N>::S;
+  constexpr int V = Lanes<N>::V, QF = FLOW ? 9 : 0;
+  const int nx = m.nx, ny = m.ny, px = m.px;
+  const long long P = m.plane;
+  N pn[9];  // the neighbours' phi + 1
+#pragma unroll
+  for (int a = 1; a < 9; ++a) {
+    const int off = D2_CY[a] * PROW + D2_CX[a];
+    set_lane(pn[a], 0, pc[off]);
+    if (V == 2) set_lane(pn[a], 1, pc[off + DY * PROW]);
+  }
+  if (MASK && EDGE && solids) {
     // a solid neighbour counts as the first fluid node among (x + c_x, y),
     // (x, y + c_y) and (x, y): zero normal derivative at walls and obstacles
-    auto sv = [&](int cx, int cy, R v) -> R {
-      if (!solid_mapped(m, x + cx, y + cy)) return v;
-      if (cx != 0 && !solid_mapped(m, x + cx, y)) return pc[cx];
-      if (cy != 0 && !solid_mapped(m, x, y + cy)) return pc[cy * PROW];
-      return pc[0];
-    };
-    pE = sv(1, 0, pE);
-    pW = sv(-1, 0, pW);
-    pN = sv(0, 1, pN);
-    pS = sv(0, -1, pS);
-    pNE = sv(1, 1, pNE);
-    pNW = sv(-1, 1, pNW);
-    pSE = sv(1, -1, pSE);
-    pSW = sv(-1, -1, pSW);
+#pragma unroll 1
+    for (int k = 0; k < V; ++k) {
+      const int yk = y + k * DY;
+      const S* pk = pc + k * (DY * PROW);
+      if (x >= nx || yk >= ny) continue;
+#pragma unroll
+      for (int a = 1; a < 9; ++a) {
+        const int cx = D2_CX[a], cy = D2_CY[a];
+        if (!solid_mapped(m, x + cx, yk + cy)) continue;
+        S v = pk[0];
+        if (cx != 0 && !solid_mapped(m, x + cx, yk)) v = pk[cx];
+        else if (cy != 0 && !solid_mapped(m, x, yk + cy)) v = pk[cy * PROW];
+        set_lane(pn[a], k, v);
+      }
+    }
   }
-  // grad = 3 sum_a w_a c_a phi(x + c_a) over D2Q9
-  const R gxv = R(1.0 / 3.0) * (pE - pW) + R(1.0 / 12.0) * ((pNE + pSE) - (pNW + pSW));
-  const R gyv = R(1.0 / 3.0) * (pN - pS) + R(1.0 / 12.0) * ((pNE + pNW) - (pSE + pSW));
-  R as, Nx, Ny, Nz;
-  aniso<R>(m, gxv, gyv, R(0), as, Nx, Ny, Nz);
-  const R a2 = as * as;
-  const R inv_a2 = rcp_r(a2);
-  const R omega_phi = rcp_r(a2 * c.tpc + R(0.5));  // Eq. 23
-  const R phi2m = R(1) - phi * phi;
-  const R Qs = (phi - phi * phi * phi + c.lambda * U * phi2m * phi2m) * c.inv_tau0;  // Eq. 20
-  // Node constants of the collisions, so that each direction costs a few FMAs:
-  //   f*: (1 - w_f) d + w_f w [E0 + cu (E1 + E2 cu)] + guo w [cF (3 + 9 cu) - 3 u*.F]
-  //       (Eq. 4, 5, 8, 9 with c_s^2 = 1/3, d = f - w)
-  //   g*: (1 - w_U) d + w (K0 + K1 cu)            (Eqs. 13-16, d = g - w U_ref)
-  //   h*: (1 - w_phi) d + w (H0 - c.H)            (Eqs. 19-21, d = h + w)
-  const R uu = usx * usx + usy * usy, uF = usx * Fx + usy * Fy;
-  const R omega_f = c.omega_f, keep_f = R(1) - c.omega_f, guo = c.guo;
-  const R E0 = omega_f * (drho - R(1.5) * rho * uu);
-  const R E1 = omega_f * R(3) * rho, E2 = omega_f * R(4.5) * rho;
-  const R G0 = -R(3) * uF;
-  const R keep_U = R(1) - omega_U;
-  const R K0 = omega_U * dU - dphidt, K1 = R(3) * omega_U * U;
-  const R keep_phi = R(1) - omega_phi;
-  const R H0 = omega_phi * dphi + Qs;
-  const R Hx = omega_phi * c.tpc * Nx, Hy = omega_phi * c.tpc * Ny;
-  const R keep_old = R(1) - inv_a2;  // Eq. 19: h_new = h* / a_s^2 + (1 - 1/a_s^2) h_old
-
-  // array of direction a: f at a * P, g at (QF + a) * P, h at (QF + 9 + a) * P
-#define LBPF_DF(a) (dst + (a) * P)
-#define LBPF_DG(a) (dst + (QF + (a)) * P)
-#define LBPF_DH(a) (dst + (QF + 9 + (a)) * P)
-  const int bcx = m.bc[0], bcy = m.bc[1];
-
+  N f[9], g[9];
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
-    const int cx = D2_CX[a], cy = D2_CY[a];
-    const R w = d2_w<R>(a);
-    const R cu = R(cx) * usx + R(cy) * usy;
-    // post-collision deviations at this node
-    R fp = R(0);
-    if (FLOW && CHM) {
-      fp = fchm[a];
-    } else if (FLOW) {
-      const R cF = R(cx) * Fx + R(cy) * Fy;
-      const R feq = fma_r(cu, fma_r(E2, cu, E1), E0);
-      const R guo_t = mul_r(guo, fma_r(cF, fma_r(R(9), cu, R(3)), G0));
-      fp = fma_r(keep_f, f[a], mul_r(w, add_r(feq, guo_t)));
+    if (FLOW) f[a] = own(a);
+    g[a] = own(QF + a);
+  }
+  Node2D<N> nd;
+  N fchm[9];
+  if (!node_2d<N, FLOW, CHM>(m, f, g, dphi, dphi_prev, Rg, pn[1], pn[3], pn[2], pn[4], pn[5],
+                             pn[6], pn[8], pn[7], nd, fchm))
+    atomicOr(err, 1u);
+  Unew = nd.U;
+
+  if constexpr (!EDGE) {
+    auto put = [&](int q, int off, N v) {
+      char* b = reinterpret_cast<char*>(tb + (q * P + off));
+      Pop<T>::st(reinterpret_cast<T*>(b + o0), lane(v, 0));
+      if (V == 2) Pop<T>::st(reinterpret_cast<T*>(b + o1), lane(v, 1));
+    };
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+      const int off = D2_CY[a] * px + D2_CX[a];
+      if (FLOW) put(a, off, CHM ? fchm[a] : post_f_2d<N>(nd, a, f[a]));
+      N gp = post_g_2d<N>(nd, a, g[a]);
+      if (UREL) gp = fma_r(splat<N>(-d2_w<S>(a)), sub_r(uref(D2_CY[a], D2_CX[a]), Rg), gp);
+      put(QF + a, off, gp);
+      put(QF + 9 + a, off,
+          arrive_h_2d<N>(nd, post_h_2d<N>(nd, a, h[a]), hold(a, D2_CY[a], D2_CX[a])));
     }
-    const R gp = fma_r(keep_U, g[a], mul_r(w, fma_r(K1, cu, K0)));
-    const R hp = fma_r(keep_phi, h[a], mul_r(w, add_r(H0, -add_r(R(cx) * Hx, R(cy) * Hy))));
-    if (INTERIOR) {
-      const int off = cy * px + cx;  // uniform
-      const R hold = hs.at(a, ly + cy, lx + cx);  // h_a(s + c_a, t)
-      if (FLOW) Pop<T>::st(pd + (a * P + off), fp);
-      Pop<T>::st(pd + ((QF + a) * P + off), genc(gp, w, ly + cy, lx + cx));
-      Pop<T>::st(pd + ((QF + 9 + a) * P + off), fma_r(inv_a2, hp, mul_r(keep_old, hold)));  // Eq. 19
-      continue;
+    return;
+  } else {
+    // Element steps to the neighbouring columns and rows (across a periodic
+    // edge to the far side) and what lies there: a wall (the population comes
+    // back to its node reversed, half-way bounce-back) or, in x, the inflow
+    // or outflow ghost (nothing to push).
+    const int bcx = m.bc[0], bcy = m.bc[1];
+    const bool x_lo = x == 0, x_hi = x == nx - 1;
+    const int sxm = x_lo ? nx - 1 : -1, sxp = x_hi ? 1 - nx : 1;
+    const bool wxm = x_lo && bcx == BC_WALL, wxp = x_hi && bcx == BC_WALL;
+    const bool gxm = x_lo && bcx == BC_INOUT, gxp = x_hi && bcx == BC_INOUT;
+    const int wrap_y = (ny - 1) * px;
+    int sym[V], syp[V];
+    bool wym[V], wyp[V], on[V];
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      const int yk = y + k * DY;
+      on[k] = x < nx && yk < ny;
+      if (MASK && solids && on[k]) on[k] = !m.solid[yk * px + x];
+      sym[k] = yk == 0 ? wrap_y : -px;
+      syp[k] = yk == ny - 1 ? -wrap_y : px;
+      wym[k] = yk == 0 && bcy == BC_WALL;
+      wyp[k] = yk == ny - 1 && bcy == BC_WALL;
     }
-    // destination s + c_a
-    int xd = x + cx, yd = y + cy;
-    bool bounce = false, drop = false;
-    if (yd < 0 || yd >= ny) {
-      if (bcy == BC_PERIODIC) yd = wrap1(yd, ny);
-      else bounce = true;
-    }
-    if (xd < 0 || xd >= nx) {
-      if (bcx == BC_PERIODIC) xd = wrap1(xd, nx);
-      else if (bcx == BC_WALL) bounce = true;
-      else drop = true;
-    }
-    if (MASK && solids && !bounce && !drop && m.solid[yd * px + xd]) bounce = true;  // obstacle
-    if (bounce) {
-      // half-way bounce-back: comes back to this node reversed
-      const int b = D2_OPP[a];
-      if (FLOW) Pop<T>::st(LBPF_DF(b) + idx, fp);
-      Pop<T>::st(LBPF_DG(b) + idx, genc(gp, w, ly, lx));
-      Pop<T>::st(LBPF_DH(b) + idx, fma_r(inv_a2, hp, mul_r(keep_old, h[b])));
-    } else if (!drop) {
-      const int jd = yd * px + xd;
-      const R hold = hs.at(a, ly + cy, lx + cx);  // h_a(s + c_a, t)
-      if (FLOW) Pop<T>::st(LBPF_DF(a) + jd, fp);
-      Pop<T>::st(LBPF_DG(a) + jd, genc(gp, w, ly + cy, lx + cx));
-      Pop<T>::st(LBPF_DH(a) + jd, fma_r(inv_a2, hp, mul_r(keep_old, hold)));  // Eq. 19
-    }
-    if (bcx == BC_INOUT) {
-      if (cx == -1 && x == nx - 1) {
-        // outflow ghost x = nx repeats this column: its post-collision value
-        // arrives at (nx - 1, y + c_y)
-        int yo = y + cy;
-        bool ok = true;
-        if (yo < 0 || yo >= ny) {
-          if (bcy == BC_PERIODIC) yo = wrap1(yo, ny);
-          else ok = false;
-        }
-        if (ok) {
-          const int jo = yo * px + x;
-          const R hold = hs.at(a, ly + cy, lx);
-          if (FLOW) Pop<T>::st(LBPF_DF(a) + jo, fp);
-          Pop<T>::st(LBPF_DG(a) + jo, genc(gp, w, ly + cy, lx));
-          Pop<T>::st(LBPF_DH(a) + jo, fma_r(inv_a2, hp, mul_r(keep_old, hold)));
+    T* const n0 = reinterpret_cast<T*>(reinterpret_cast<char*>(tb) + o0);
+    T* const n1 = reinterpret_cast<T*>(reinterpret_cast<char*>(tb) + o1);
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+      const int cx = D2_CX[a], cy = D2_CY[a], b = D2_OPP[a];
+      N fp = splat<N>(S(0));
+      if (FLOW) fp = CHM ? fchm[a] : post_f_2d<N>(nd, a, f[a]);
+      const N gp = post_g_2d<N>(nd, a, g[a]);
+      const N hp = post_h_2d<N>(nd, a, h[a]);
+      const N w = splat<N>(d2_w<S>(a));
+      const N hfar = arrive_h_2d<N>(nd, hp, hold(a, cy, cx));    // at the destination
+      const N hown = arrive_h_2d<N>(nd, hp, h[b]);               // reversed at the node
+      N gfar = gp, gown = gp;
+      if (UREL) {
+        gfar = fma_r(neg_r(w), sub_r(uref(cy, cx), Rg), gp);
+        gown = fma_r(neg_r(w), sub_r(uref(0, 0), Rg), gp);
+      }
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        T* const node = k ? n1 : n0;
+        bool back = (cy < 0 && wym[k]) || (cy > 0 && wyp[k]) || (cx < 0 && wxm) || (cx > 0 && wxp);
+        const bool ghost = !back && ((cx < 0 && gxm) || (cx > 0 && gxp));
+        const int step = (cx < 0 ? sxm : (cx > 0 ? sxp : 0)) +
+                         (cy < 0 ? sym[k] : (cy > 0 ? syp[k] : 0));
+        if (MASK && solids && on[k] && !back && !ghost)
+          back = m.solid[(y + k * DY) * px + x + step] != 0;  // obstacle
+        if (on[k] && !ghost) {
+          T* const p = back ? node + b * P : node + (a * P + step);
+          if (FLOW) Pop<T>::st(p, lane(fp, k));
+          Pop<T>::st(p + QF * P, back ? lane(gown, k) : lane(gfar, k));
+          Pop<T>::st(p + (QF + 9) * P, back ? lane(hown, k) : lane(hfar, k));
         }
       }
-      if (cx == 1 && x == 0) {
-        // inflow ghost x = -1: equilibrium at rho = 1, u = u_in e_x, U = U_in,
-        // phi = -1 (a_s = 1; its h deviation is 0), unless behind a wall
-        const int ys = y - cy;
-        if (!((ys < 0 || ys >= ny) && bcy == BC_WALL)) {
-          const R uin = c.u_in, cui = uin;
-          if (FLOW)
-            Pop<T>::st(LBPF_DF(a) + idx,
-                       w * (R(3) * cui + R(4.5) * cui * cui - R(1.5) * uin * uin));
-          const R gu = FLOW ? cui : R(0);
-          const R Uin = c.U_in;
-          Pop<T>::st(LBPF_DG(a) + idx, genc(w * ((Uin - Rg) + Uin * R(3) * gu), w, ly, lx));
-          Pop<T>::st(LBPF_DH(a) + idx, R(0));
+      if (cx != 0 && bcx == BC_INOUT) {
+        if (cx < 0 && x_hi) {
+          // outflow ghost x = nx repeats this column: its post-collision value
+          // arrives at (nx - 1, y + c_y)
+          const N hout = arrive_h_2d<N>(nd, hp, hold(a, cy, 0));
+          N gout = gp;
+          if (UREL) gout = fma_r(neg_r(w), sub_r(uref(cy, 0), Rg), gp);
+#pragma unroll
+          for (int k = 0; k < V; ++k) {
+            if (!on[k] || (cy < 0 && wym[k]) || (cy > 0 && wyp[k])) continue;
+            T* const p = (k ? n1 : n0) + (a * P + (cy < 0 ? sym[k] : (cy > 0 ? syp[k] : 0)));
+            if (FLOW) Pop<T>::st(p, lane(fp, k));
+            Pop<T>::st(p + QF * P, lane(gout, k));
+            Pop<T>::st(p + (QF + 9) * P, lane(hout, k));
+          }
+        }
+        if (cx > 0 && x_lo) {
+          // inflow ghost x = -1: equilibrium at rho = 1, u = u_in e_x, U = U_in,
+          // phi = -1 (a_s = 1; its h deviation is 0), unless behind a wall
+          const Coef<S>& c = coef<S>(m);
+          const S uin = c.u_in, Uin = c.U_in, ws = d2_w<S>(a), gu = FLOW ? uin : S(0);
+          const S fin = ws * (S(3) * uin + S(4.5) * uin * uin - S(1.5) * uin * uin);
+#pragma unroll
+          for (int k = 0; k < V; ++k) {
+            if (!on[k] || (cy > 0 && wym[k]) || (cy < 0 && wyp[k])) continue;
+            T* const p = (k ? n1 : n0) + a * P;
+            const S R0 = lane(Rg, k);
+            S gin = ws * ((Uin - R0) + Uin * S(3) * gu);
+            if (UREL) gin = fma_r(-ws, lane(uref(0, 0), k) - R0, gin);
+            if (FLOW) Pop<T>::st(p, fin);
+            Pop<T>::st(p + QF * P, gin);
+            Pop<T>::st(p + (QF + 9) * P, S(0));
+          }
         }
       }
     }
   }
-#undef LBPF_DF
-#undef LBPF_DG
-#undef LBPF_DH
 }
 
 }  // namespace lbk

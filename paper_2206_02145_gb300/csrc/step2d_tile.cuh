@@ -53,108 +53,161 @@ __device__ __forceinline__ void issue_tile_2d(const CUtensorMap* tm_fg, const CU
   }
 }
 
+// Threads that work on a TX x TY tile.  PAIR: a thread holds the two nodes
+// (tx, ty) and (tx, ty + TY / 2), so that interior tiles run on the packed
+// two-lane FP32 instructions.
+template <int TX, int TY, bool PAIR>
+constexpr int tile_threads() {
+  return PAIR ? TX * TY / 2 : TX * TY;
+}
+
 // Work on a filled stage `st` for the tile at (x0, y0).  Called by all
 // threads of the CTA; contains CTA barriers.  sh_phi: (TY + 2) x (TX + 2).
-// MASK: solid nodes are handled (flag of the tile from m.solid_tiles).  CHM:
-// the flow collides by the central Hermite MRT.
-template <typename T, bool FLOW, int TX, int TY, bool MASK, bool CHM>
-__device__ __forceinline__ void tile_2d(const Model& m, const T* __restrict__ src,
+// `bad`: this thread saw the stage's loads time out; the first barrier tells
+// every thread, and the tile is given up before its first global write
+// (returns false).  MASK: solid nodes are handled (flag of the tile from
+// m.solid_tiles).  CHM: the flow collides by the central Hermite MRT.
+template <typename T, bool FLOW, int TX, int TY, bool PAIR, bool MASK, bool CHM>
+__device__ __forceinline__ bool tile_2d(const Model& m, const T* __restrict__ src,
                                         T* __restrict__ dst, float* __restrict__ ring_cur,
                                         unsigned* __restrict__ err, int x0, int y0, int c,
-                                        unsigned char* st, float* sh_phi_flat) {
+                                        unsigned char* st, float* sh_phi_flat, bool bad) {
   using R = float;
   using L = Tiles2D<T, FLOW, TX, TY>;
-  constexpr int NT = TX * TY, SX = TX + 2, SY = TY + 2;
+  constexpr int NT = tile_threads<TX, TY, PAIR>(), SX = TX + 2, SY = TY + 2;
+  constexpr int V = PAIR ? 2 : 1, DY = TY / 2;
   constexpr int QF = FLOW ? 9 : 0;
   const int tid = threadIdx.x;
   const int tx = tid % TX, ty = tid / TX;
   const int nx = m.nx, ny = m.ny, px = m.px;
   R(*sh_phi)[SX] = reinterpret_cast<R(*)[SX]>(sh_phi_flat);
-    const T* fgs = reinterpret_cast<const T*>(st);
-    T* hsm = reinterpret_cast<T*>(st + L::OFF_H);
-    const float* rings = reinterpret_cast<const float*>(st + L::OFF_RING);
-    const __half* uown = reinterpret_cast<const __half*>(st + L::OFF_UOWN);
-    __half* uhal = reinterpret_cast<__half*>(st + L::OFF_UHAL);
-    constexpr int HPLANE = SY * L::BXH;
-    // tiles next to solid nodes take the general path with the mask (the
-    // flag is loaded first, so that its latency overlaps the phi sums)
-    const bool solids =
-        MASK && m.solid && m.solid_tiles[(y0 / TY) * ((nx + TX - 1) / TX) + x0 / TX];
+  const T* fgs = reinterpret_cast<const T*>(st);
+  T* hsm = reinterpret_cast<T*>(st + L::OFF_H);
+  const float* rings = reinterpret_cast<const float*>(st + L::OFF_RING);
+  const __half* uown = reinterpret_cast<const __half*>(st + L::OFF_UOWN);
+  __half* uhal = reinterpret_cast<__half*>(st + L::OFF_UHAL);
+  constexpr int HPLANE = SY * L::BXH;
+  // tiles next to solid nodes take the general path with the mask (the
+  // flag is loaded first, so that its latency overlaps the phi sums)
+  const bool solids =
+      MASK && m.solid && m.solid_tiles[(y0 / TY) * ((nx + TX - 1) / TX) + x0 / TX];
 
-    if (x0 == 0 || y0 == 0 || x0 + TX >= nx || y0 + TY >= ny) {
-      // halo positions outside the domain: periodic wrap or nearest node
-      for (int i = tid; i < SX * SY; i += NT) {
-        const int lx = i % SX, ly = i / SX;
-        int gx = x0 + lx - 1, gy = y0 + ly - 1;
-        if (gx >= 0 && gx < nx && gy >= 0 && gy < ny) continue;
-        gx = grad_coord(gx, nx, m.bc[0]);
-        gy = grad_coord(gy, ny, m.bc[1]);
-        const int j = gy * px + gx;
-        const int P = int(m.plane);
+  if (x0 == 0 || y0 == 0 || x0 + TX >= nx || y0 + TY >= ny) {
+    // halo positions outside the domain: the nearest node, which the tile
+    // holds, or across a periodic edge the far side (or, where the tile spans
+    // the domain, its own other side)
+    for (int i = tid; i < SX * SY; i += NT) {
+      const int lx = i % SX, ly = i / SX;
+      int gx = x0 + lx - 1, gy = y0 + ly - 1;
+      if (gx >= 0 && gx < nx && gy >= 0 && gy < ny) continue;
+      if (gx > nx || gy > ny) continue;  // beyond the halo of a partial tile
+      const int wx = grad_coord(gx, nx, m.bc[0]), wy = grad_coord(gy, ny, m.bc[1]);
+      const int sx = wx - x0 + 1, sy = wy - y0 + 1;  // the mapped node in the tile's box
+      T* const hd = hsm + ly * L::BXH + lx + L::HX - 1;
+      __half* const ud = uhal + ly * L::BXU + lx + L::HXU - 1;
+      if (sx >= 0 && sx < SX && sy >= 0 && sy < SY) {
+        const T* const hf = hsm + sy * L::BXH + sx + L::HX - 1;
 #pragma unroll
-        for (int a = 0; a < 9; ++a)
-          hsm[a * HPLANE + ly * L::BXH + lx + L::HX - 1] = src[(QF + 9 + a) * P + j];
-        if (L::REL) uhal[ly * L::BXU + lx + L::HXU - 1] = m.uring[size_t(c ^ 1) * m.plane + j];
-      }
-      __syncthreads();
-    }
-    // phi + 1 of the halo-extended tile: each thread's own position from the
-    // h it keeps for the collision, the ring around the tile by a pass
-    R h[9];
-    {
-      R sum = R(0);
-#pragma unroll
-      for (int a = 0; a < 9; ++a) {
-        h[a] = Pop<T>::template ld<R>(hsm + a * HPLANE + (ty + 1) * L::BXH + tx + L::HX);
-        sum += h[a];
-      }
-      sh_phi[ty + 1][tx + 1] = sum;
-    }
-    constexpr int NRING = 2 * SX + 2 * TY;
-    for (int i = tid; i < NRING; i += NT) {
-      int lx, ly;
-      if (i < 2 * SX) {
-        lx = i % SX;
-        ly = i < SX ? 0 : SY - 1;
+        for (int a = 0; a < 9; ++a) hd[a * HPLANE] = hf[a * HPLANE];
+        if (L::REL) *ud = uhal[sy * L::BXU + sx + L::HXU - 1];
       } else {
-        lx = (i - 2 * SX) & 1 ? SX - 1 : 0;
-        ly = 1 + (i - 2 * SX) / 2;
-      }
-      const T* hp = hsm + ly * L::BXH + lx + L::HX - 1;
-      R sum = R(0);
+        const long long j = (long long)wy * px + wx, P = m.plane;
 #pragma unroll
-      for (int a = 0; a < 9; ++a) sum += Pop<T>::template ld<R>(hp + a * HPLANE);
-      sh_phi[ly][lx] = sum;
+        for (int a = 0; a < 9; ++a) hd[a * HPLANE] = src[(QF + 9 + a) * P + j];
+        if (L::REL) *ud = m.uring[size_t(c ^ 1) * m.plane + j];
+      }
     }
     __syncthreads();
-
-    const int x = x0 + tx, y = y0 + ty;
-    if (x < nx && y < ny && solids && m.solid[y * px + x]) {
-      ring_cur[y * px + x] = sh_phi[ty + 1][tx + 1];  // a solid node keeps its state
-    } else if (x < nx && y < ny) {
-      R f[9], g[9];
-      const int o = ty * TX + tx;
+  }
+  // phi + 1 of the halo-extended tile: each thread's own positions from the
+  // h it keeps for the collision, the ring around the tile by a pass
+  const T* hown = hsm + (ty + 1) * L::BXH + tx + L::HX;
+  using N = std::conditional_t<PAIR, float2, float>;
+  auto h_at = [&](int a, int off) -> N {  // h_a at `off` from the thread's node(s)
+    const T* p = hown + a * HPLANE + off;
+    if constexpr (PAIR)
+      return make_float2(Pop<T>::template ld<R>(p), Pop<T>::template ld<R>(p + DY * L::BXH));
+    else
+      return Pop<T>::template ld<R>(p);
+  };
+  N h[9], dphi;
+  {
 #pragma unroll
-      for (int a = 0; a < 9; ++a) {
-        if (FLOW) f[a] = Pop<T>::template ld<R>(fgs + a * (TY * TX) + o);
-        g[a] = Pop<T>::template ld<R>(fgs + (QF + a) * (TY * TX) + o);
-      }
-      // g stored relative to the node's own U reference, the collision
-      // takes the deviations from it as they are
-      UView<L::REL, L::BXU> uh{uhal + L::HXU - 1,
-                               L::REL ? m.uring + size_t(c) * m.plane : nullptr,
-                               L::REL ? __half2float(uown[o]) : 0.f};
-      TileView<T, R, L::BXH, HPLANE, L::HX - 1> hs{hsm};
-      if (!solids && x0 >= 1 && x0 + TX <= nx - 1 && y0 >= 1 && y0 + TY <= ny - 1)
-        collide_push_2d<T, R, FLOW, true, SX, MASK, CHM>(m, x, y, tx + 1, ty + 1, f, g, h,
-                                                    sh_phi[ty + 1][tx + 1], rings[o],
-                                                    &sh_phi[0][0], hs, uh, dst, ring_cur, err);
-      else
-        collide_push_2d<T, R, FLOW, false, SX, MASK, CHM>(m, x, y, tx + 1, ty + 1, f, g, h,
-                                                     sh_phi[ty + 1][tx + 1], rings[o],
-                                                     &sh_phi[0][0], hs, uh, dst, ring_cur, err,
-                                                     solids);
+    for (int a = 0; a < 9; ++a) {
+      h[a] = h_at(a, 0);
+      dphi = a == 0 ? h[0] : add_r(dphi, h[a]);
     }
+    if constexpr (PAIR) {
+      sh_phi[ty + 1][tx + 1] = dphi.x;
+      sh_phi[ty + 1 + DY][tx + 1] = dphi.y;
+    } else {
+      sh_phi[ty + 1][tx + 1] = dphi;
+    }
+  }
+  constexpr int NRING = 2 * SX + 2 * TY;
+  for (int i = tid; i < NRING; i += NT) {
+    int lx, ly;
+    if (i < 2 * SX) {
+      lx = i % SX;
+      ly = i < SX ? 0 : SY - 1;
+    } else {
+      lx = (i - 2 * SX) & 1 ? SX - 1 : 0;
+      ly = 1 + (i - 2 * SX) / 2;
+    }
+    const T* hp = hsm + ly * L::BXH + lx + L::HX - 1;
+    R sum = R(0);
+#pragma unroll
+    for (int a = 0; a < 9; ++a) sum += Pop<T>::template ld<R>(hp + a * HPLANE);
+    sh_phi[ly][lx] = sum;
+  }
+  if (__syncthreads_or(bad)) return false;
+
+  const int x = x0 + tx, y = y0 + ty;
+  const int o = ty * TX + tx;
+  auto two = [](float v, float w) -> N {
+    if constexpr (PAIR) return make_float2(v, w);
+    else return v;
+  };
+  // g is stored relative to the node's own U reference (16-bit storage); the
+  // collision takes the deviations from it as they are
+  N Rg = splat<N>(m.cf.ref_g), Unew;
+  if constexpr (L::REL) Rg = two(__half2float(uown[o]), __half2float(uown[o + (V - 1) * DY * TX]));
+  const __half* uc = uhal + (ty + 1) * L::BXU + tx + L::HXU;
+  const size_t org = size_t(y0) * px + x0;
+  const unsigned e0 = unsigned(ty * px + tx), e1 = e0 + unsigned(DY * px);
+  auto work = [&](auto edge) {
+    collide_push_2d<T, N, FLOW, CHM, MASK, decltype(edge)::value, L::REL, SX, DY>(
+        m, x, y,
+        [&](int q) {
+          const T* p = fgs + q * (TY * TX) + o;
+          return two(Pop<T>::template ld<R>(p), Pop<T>::template ld<R>(p + (V - 1) * DY * TX));
+        },
+        h, dphi, two(rings[o], rings[o + (V - 1) * DY * TX]), &sh_phi[ty + 1][tx + 1],
+        [&](int a, int dy, int dx) { return h_at(a, dy * L::BXH + dx); },
+        [&](int dy, int dx) {
+          const __half* p = uc + dy * L::BXU + dx;
+          return two(__half2float(p[0]), __half2float(p[(V - 1) * DY * L::BXU]));
+        },
+        Rg, dst + org, e0 * unsigned(sizeof(T)), e1 * unsigned(sizeof(T)), err, Unew, solids);
+  };
+  // boundary logic only for the warps that have a node on a domain edge
+  const bool edge = __any_sync(0xffffffffu, solids || x < 1 || x > nx - 2 || y < 1 ||
+                                                y + (V - 1) * DY > ny - 2);
+  if (edge) work(std::true_type{});
+  else work(std::false_type{});
+  // phi(t) of every node, and the new U of every node but the solid ones
+  float* ring_t = ring_cur + org;
+  __half* un = L::REL ? m.uring + (size_t(c) * m.plane + org) : nullptr;
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    const unsigned e = k ? e1 : e0;
+    if (!edge || (x < nx && y + k * DY < ny)) {
+      ring_t[e] = lane(dphi, k);
+      if constexpr (L::REL)
+        if (!(MASK && solids && m.solid[(y + k * DY) * px + x])) un[e] = __float2half_rn(lane(Unew, k));
+    }
+  }
+  return true;
 }
 
 }  // namespace lbk

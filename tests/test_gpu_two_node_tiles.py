@@ -1,0 +1,100 @@
+"""The 2D step's tiles with two nodes per thread, taken by grids of at least
+1500 tiles of 64 x 4: sizes at that line and one tile below it, whole and
+ragged last tiles, every kind of boundary, solid nodes and both collisions,
+against the FP64 oracle.
+
+FP32 fields to 1e-5 (the repository's bar).  16-bit storage: a step rounds each
+stored deviation once, to u = 2^-11 (FP16) or 2^-8 (BF16) of itself, so N steps
+move a moment by at most N u times the sum of the deviations it is made of:
+at most 2 for phi, 0.5 for U (its own reference removed, plus the change next
+to the crystal), 0.1 for rho and u.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+STEPS = 5
+SIZES = [(960, 400),  # 15 x 100 tiles, all whole
+         (901, 397),  # the same tiles, ragged on both sides
+         (960, 396),  # one row of tiles fewer: one node per thread
+         (4000, 93)]  # 63 x 24 tiles, long rows
+BOUNDS = {
+    "inflow": dict(bc=(1, 0, 0), u_in=0.01, U_in=0.4),
+    "inflow_walls": dict(bc=(1, 2, 0), u_in=0.01, U_in=0.4),
+    "periodic": dict(bc=(0, 0, 0), body=(1e-5, 2e-5, 0.0)),
+    "walls_x": dict(bc=(2, 0, 0), body=(0.0, 1e-5, 0.0)),
+}
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    assert torch.cuda.is_available(), "these tests need a CUDA GPU"
+    import _pairs
+    return _pairs
+
+
+def problem(P, size, bounds, flow=1):
+    nx, ny = size
+    p = P.params(nx=nx, ny=ny, flow=flow, fold=5, eps=0.03, theta0=0.2, **BOUNDS[bounds])
+    # crystals on the left and right edge columns and across the top edge too
+    y, x = np.mgrid[0:ny, 0:nx].astype(float)
+    rng = np.random.default_rng(5)
+    r = np.minimum.reduce([np.hypot(x - cx, y - cy) for cx, cy in
+                           ((0, ny / 2), (nx - 1, ny / 3), (nx / 2, 0), (65, 9))])
+    phi = np.tanh((12.0 - r) / (np.sqrt(2.0) * 2.0)) + 0.01 * rng.uniform(-1, 1, r.shape)
+    U = 0.4 + 0.01 * rng.uniform(-1, 1, r.shape)
+    v = [0.01 * rng.uniform(-1, 1, r.shape) for _ in range(3)]
+    return p, (phi, U, 1.0 + 1e-3 * rng.uniform(-1, 1, r.shape), v)
+
+
+@pytest.mark.parametrize("bounds", BOUNDS)
+@pytest.mark.parametrize("size", SIZES, ids=str)
+def test_fp32(P, size, bounds):
+    p, fields = problem(P, size, bounds)
+    a, b = P.pair(p, "fp32", fields=fields)
+    a.step(STEPS)
+    b.step(STEPS, P.THREADS)
+    errs = P.max_errors(a, b)
+    assert max(errs.values()) < 1e-5, errs
+    a.close()
+
+
+@pytest.mark.parametrize("storage,u", [("fp16", 2.0 ** -11), ("bf16", 2.0 ** -8)])
+@pytest.mark.parametrize("size", SIZES[:2], ids=str)
+def test_16bit(P, size, storage, u):
+    p, fields = problem(P, size, "inflow")
+    a, b = P.pair(p, storage, fields=fields)
+    a.step(STEPS)
+    b.step(STEPS, P.THREADS)
+    errs = P.max_errors(a, b)
+    n = STEPS + 1  # the initial state is rounded too
+    assert errs["phi"] < n * u * 2.0 and errs["U"] < n * u * 0.5, errs
+    assert max(errs["rho"], errs["ux"], errs["uy"]) < n * u * 0.1, errs
+    a.close()
+
+
+@pytest.mark.parametrize("chm", [0, 1])
+@pytest.mark.parametrize("size", SIZES[:2], ids=str)
+def test_solids_and_collision(P, size, chm):
+    import oracle
+    import paper_2206_02145_gb300 as L
+    p, (phi, U, rho, v) = problem(P, size, "inflow_walls")
+    mask = np.zeros(phi.shape, bool)
+    mask[100:300, 60:68] = True      # across a tile edge
+    mask[0:3, 200:230] = True        # on the wall
+    mask[-2:, 895:898] = True        # in the last tiles
+    a = L.Sim(dim=2, nx=p["nx"], ny=p["ny"], bc=p["bc"], flow=1, fold=5, eps_aniso=0.03,
+              theta0=0.2, u_inlet=0.01, u0_inlet=0.4, collision=chm)
+    b = oracle.Oracle(oracle.Params(dim=2, nx=p["nx"], ny=p["ny"], bc=p["bc"], flow=1, fold=5,
+                                    eps=0.03, theta0=0.2, u_inlet=0.01, u0_inlet=0.4,
+                                    collision=chm))
+    for s in (a, b):
+        s.init_fields(phi, U, rho, v[0], v[1], None)
+        s.set_solid(mask)
+    a.step(STEPS)
+    b.step(STEPS, P.THREADS)
+    errs = P.max_errors(a, b)
+    assert max(errs.values()) < 1e-5, errs
+    a.close()

@@ -137,6 +137,16 @@ cudaError_t batch_plan_build(const BatchMember* members, int count, int storage,
   if ((e = dispatch_any(storage, flow, v, plan->mask, plan->chm, true, &plan->ctas, &plan->smem,
                         nullptr, nullptr, nullptr, 0, nullptr)) != cudaSuccess)
     return e;
+  double state = 0.0;  // beyond the L2 the copies in flight are bounded, as in the single step
+  for (int i = 0; i < count; ++i)
+    state += 2.0 * double(members[i].m.plane) * double((qfg + 9) * es + 4 + (es == 2 ? 2 : 0));
+  if (state > kL2Bytes) {
+    int dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+      return e;
+    plan->ctas = std::min(plan->ctas, sms * std::max(1, kStageBytes / plan->smem));
+  }
   std::vector<BatchSeg> segs;
   std::vector<int> cta_seg;
   batch_schedule(tiles, plan->ctas, order, &segs, &cta_seg);

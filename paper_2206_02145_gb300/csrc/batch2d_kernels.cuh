@@ -40,6 +40,7 @@ struct StageMeta {
   float* ring_cur;
   unsigned* err;
   int x0, y0, c, inst;
+  int solids;  // the tile or its halo holds a solid node
 };
 // bytes of an instance's model copied into a stage (16-byte multiple) and the
 // stage's slot for it after the tile data
@@ -49,8 +50,8 @@ static_assert(offsetof(BatchDesc, m) % 16 == 0 &&
                   offsetof(BatchDesc, m) + kModelCopy <= sizeof(BatchDesc),
               "the model copy must be an aligned span of the descriptor");
 
-// Registers held to 20 resident warps per SM (five CTAs of 32 x 4), the
-// occupancy of the single-instance step.  MASK: solid nodes (each instance's
+// Registers held to 16 resident warps per SM (12 where a thread holds two
+// nodes: at 16 those spill, 406 against 378 us per step of 32 FP16 instances).  MASK: solid nodes (each instance's
 // model points at the per-tile flags of this variant's tiles); CHM: the
 // central Hermite MRT flow collision.
 //
@@ -63,7 +64,7 @@ static_assert(offsetof(BatchDesc, m) % 16 == 0 &&
 // everything from shared memory: no global lookups on a tile's critical path.
 template <typename T, bool FLOW, int TX, int TY, bool PAIR, int S, bool MASK, bool CHM>
 __global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(),
-                                  512 / tile_threads<TX, TY, PAIR>())
+                                  (PAIR ? 384 : 512) / tile_threads<TX, TY, PAIR>())
     step2d_batch_kernel(const BatchDesc* __restrict__ descs, const BatchSeg* __restrict__ segs,
                         const int* __restrict__ cta_seg) {
   using L = Tiles2D<T, FLOW, TX, TY>;
@@ -73,6 +74,7 @@ __global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(),
   __shared__ __align__(8) uint64_t full[S];
   __shared__ float sh_phi[SY][SX];
   __shared__ StageMeta meta[S];
+  __shared__ unsigned char sh_solid[MASK ? SX * SY : 1];
   const int tid = threadIdx.x;
   const int sb = cta_seg[blockIdx.x], se = cta_seg[blockIdx.x + 1];
   int ntiles = 0;  // this CTA's tiles (every thread)
@@ -103,6 +105,7 @@ __global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(),
     const int lt = ig.first + ik * ig.stride;
     im.x0 = (lt % intx) * TX;
     im.y0 = (lt / intx) * TY;
+    im.solids = MASK && id->m.solid ? id->m.solid_tiles[lt] : 0;
     meta[s] = im;
     unsigned char* st = smem + s * STAGE;
 #pragma unroll
@@ -145,9 +148,12 @@ __global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(),
     }
     const StageMeta mt = meta[s];
     unsigned char* st = smem + s * STAGE;
-    tile_2d<T, FLOW, TX, TY, PAIR, MASK, CHM>(
-        *reinterpret_cast<const Model*>(st + L::STAGE), static_cast<const T*>(mt.src),
-        static_cast<T*>(mt.dst), mt.ring_cur, mt.err, mt.x0, mt.y0, mt.c, st, &sh_phi[0][0], false);
+    const Model& m = *reinterpret_cast<const Model*>(st + L::STAGE);
+    const Grid2D gr(m);
+    tile_2d<T, FLOW, TX, TY, PAIR, MASK, CHM>(gr, m, static_cast<const T*>(mt.src),
+                                              static_cast<T*>(mt.dst), mt.ring_cur, mt.err, mt.x0,
+                                              mt.y0, mt.c, st, &sh_phi[0][0], sh_solid,
+                                              mt.solids != 0, false);
     __syncthreads();  // stage s (tile data, model slot, meta) and sh_phi are free again
     if (tid == 0) {
       fence_proxy_async_smem();
@@ -160,7 +166,7 @@ __global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(),
 struct Variant {
   int tx, ty, stages, nodes;
 };
-constexpr Variant kVariants[] = {{64, 4, 2, 2}, {32, 8, 2, 2}, {32, 4, 2, 2}, {32, 4, 2, 1}};
+constexpr Variant kVariants[] = {{32, 8, 2, 2}, {64, 4, 2, 2}, {64, 2, 2, 1}, {32, 4, 2, 1}};
 constexpr int kNumVariants = int(sizeof(kVariants) / sizeof(kVariants[0]));
 
 template <typename T, bool FLOW, int TX, int TY, int S, bool PAIR, bool MASK, bool CHM>

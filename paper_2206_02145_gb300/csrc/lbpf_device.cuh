@@ -159,8 +159,8 @@ __device__ __forceinline__ float2 add_r(float2 a, float2 b) { return __fadd2_rn(
 // compiler does not know to be one as its addend
 __device__ __forceinline__ float prod_r(float a, float b, float) { return mul_r(a, b); }
 __device__ __forceinline__ double prod_r(double a, double b, double) { return mul_r(a, b); }
-__device__ __forceinline__ float2 prod_r(float2 a, float2 b, float mzero) {
-  return __ffma2_rn(a, b, make_float2(mzero, mzero));
+__device__ __forceinline__ float2 prod_r(float2 a, float2 b, float2 mzero) {
+  return __ffma2_rn(a, b, mzero);
 }
 __device__ __forceinline__ float neg_r(float a) { return -a; }
 __device__ __forceinline__ double neg_r(double a) { return -a; }
@@ -176,6 +176,17 @@ template <typename N>
 __device__ __forceinline__ N splat(typename Lanes<N>::S v) {
   if constexpr (Lanes<N>::V == 2) return make_float2(v, v);
   else return v;
+}
+// lane k of a number of one or two nodes
+template <typename N>
+__device__ __forceinline__ typename Lanes<N>::S lane(const N& v, int k) {
+  if constexpr (Lanes<N>::V == 2) return k ? v.y : v.x;
+  else return v;
+}
+template <typename N>
+__device__ __forceinline__ void set_lane(N& v, int k, typename Lanes<N>::S s) {
+  if constexpr (Lanes<N>::V == 2) (k ? v.y : v.x) = s;
+  else v = s;
 }
 // are a, b and c finite (in every lane)?
 template <typename N>
@@ -207,45 +218,43 @@ __device__ __forceinline__ bool any_steep(float2 g2) { return g2.x > 1e-12f || g
 //   k-fold: N = fac k eps a_s sin(k(theta - theta0)) (g_y, -g_x)
 //   cubic : N_i = fac 16 eps a_s |grad| (n_i S - n_i^3), S = sum n_j^4
 template <typename N>
-__device__ __forceinline__ void aniso_cubic(const Coef<typename Lanes<N>::S>& c, const N* n,
-                                            N g2, N ig, int dim, N& a, N* out) {
-  using S1 = typename Lanes<N>::S;
-  N n2[3], S = splat<N>(S1(0));
+__device__ __forceinline__ void aniso_cubic(const Coef<N>& c, const N* n, N g2, N ig, int dim,
+                                            N& a, N* out) {
+  N n2[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d)
     if (d < dim) n2[d] = mul_r(n[d], n[d]);
-  S = fma_r(n2[0], n2[0], mul_r(n2[1], n2[1]));
+  N S = fma_r(n2[0], n2[0], mul_r(n2[1], n2[1]));
   if (dim == 3) S = fma_r(n2[2], n2[2], S);
-  a = fma_r(splat<N>(S1(4) * c.eps), S, splat<N>(fma_r(S1(-3), c.eps, S1(1))));
-  const N amp = mul_r(mul_r(splat<N>(c.aniso_fac * S1(16) * c.eps), a), mul_r(g2, ig));
+  a = fma_r(c.eps4, S, c.cub0);
+  const N amp = mul_r(mul_r(c.amp_c, a), mul_r(g2, ig));
 #pragma unroll
   for (int d = 0; d < 3; ++d)
     if (d < dim) out[d] = mul_r(mul_r(amp, n[d]), sub_r(S, n2[d]));
 }
 
 template <typename N>
-__device__ __forceinline__ void aniso_2d(const Model& m, N gx, N gy, N& as, N& Nx, N& Ny) {
+__device__ __forceinline__ void aniso_2d(const Coef<N>& c, int fold, N gx, N gy, N& as, N& Nx,
+                                         N& Ny) {
   using S1 = typename Lanes<N>::S;
-  const Coef<S1>& c = coef<S1>(m);
   as = splat<N>(S1(1));
   Nx = Ny = splat<N>(S1(0));
   const N g2 = fma_r(gx, gx, mul_r(gy, gy));
-  if (!any_steep(g2) || c.eps == S1(0)) return;
+  if (!any_steep(g2) || lane(c.eps, 0) == S1(0)) return;
   // (n = 0 on a flat lane: the k-fold form then gives a_s = 1, N = 0 by itself)
   const N ig = where_steep(g2, rsqrt_r(g2), splat<N>(S1(0)));
   const N n[2] = {mul_r(neg_r(gx), ig), mul_r(neg_r(gy), ig)};
-  if (m.fold > 0) {
+  if (fold > 0) {
     N ck = n[0], sk = n[1];
-    for (int j = 1; j < m.fold; ++j) {
+    for (int j = 1; j < fold; ++j) {
       const N c2 = fma_r(ck, n[0], neg_r(mul_r(sk, n[1])));
       sk = fma_r(ck, n[1], mul_r(sk, n[0]));
       ck = c2;
     }
-    const N ck0 = splat<N>(c.ck0), sk0 = splat<N>(c.sk0);
-    const N cosd = fma_r(ck, ck0, mul_r(sk, sk0));
-    const N sind = fma_r(sk, ck0, neg_r(mul_r(ck, sk0)));
-    as = fma_r(splat<N>(c.eps), cosd, splat<N>(S1(1)));
-    const N amp = mul_r(mul_r(splat<N>(c.aniso_fac * S1(m.fold) * c.eps), as), sind);
+    const N cosd = fma_r(ck, c.ck0, mul_r(sk, c.sk0));
+    const N sind = fma_r(sk, c.ck0, neg_r(mul_r(ck, c.sk0)));
+    as = fma_r(c.eps, cosd, splat<N>(S1(1)));
+    const N amp = mul_r(mul_r(c.amp_k, as), sind);
     Nx = mul_r(amp, gy);
     Ny = mul_r(neg_r(amp), gx);
   } else {
@@ -258,14 +267,13 @@ __device__ __forceinline__ void aniso_2d(const Model& m, N gx, N gy, N& as, N& N
 }
 
 template <typename N>
-__device__ __forceinline__ void aniso_3d(const Model& m, const N (&g)[3], N& as, N (&Nv)[3]) {
+__device__ __forceinline__ void aniso_3d(const Coef<N>& c, const N (&g)[3], N& as, N (&Nv)[3]) {
   using S1 = typename Lanes<N>::S;
-  const Coef<S1>& c = coef<S1>(m);
   as = splat<N>(S1(1));
 #pragma unroll
   for (int d = 0; d < 3; ++d) Nv[d] = splat<N>(S1(0));
   const N g2 = fma_r(g[2], g[2], fma_r(g[0], g[0], mul_r(g[1], g[1])));
-  if (!any_steep(g2) || c.eps == S1(0)) return;
+  if (!any_steep(g2) || lane(c.eps, 0) == S1(0)) return;
   // (n = 0 on a flat lane, so N = 0 there by itself)
   const N ig = where_steep(g2, rsqrt_r(g2), splat<N>(S1(0)));
   N n[3], a;

@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstdint>
 #include <type_traits>
 
@@ -17,15 +18,21 @@ namespace lbk {
 enum { BC_PERIODIC = 0, BC_INOUT = 1, BC_WALL = 2 };
 enum { ST_FP32 = 0, ST_FP64 = 1, ST_FP16 = 2, ST_BF16 = 3 };
 
-// Model constants in one arithmetic type.  The kernels read the copy in their
-// own type: converting a double constant inside the per-node code would run
-// on the FP64 pipe, which on GB300 is narrow enough to bound the whole step.
+// Model constants in one arithmetic type (float2: both lanes alike, for the
+// packed two-node arithmetic).  The kernels read the copy in their own type:
+// converting a double constant inside the per-node code would run on the FP64
+// pipe, which on GB300 is narrow enough to bound the whole step.
 template <typename R>
 struct Coef {
-  R omega_f, guo, tauU_slope, inv_tau0, tpc, lambda, eps, ck0, sk0, aniso_fac, kdrag;
+  R omega_f, guo, tauU_slope, inv_tau0, tpc, lambda, eps, ck0, sk0, kdrag;
   R body[3];
   R u_in, U_in, ref_f, ref_g, ref_h;
   R chm_wb, chm_wh;  // central Hermite MRT: trace and higher-order rates
+  // products of constants, rounded in the arithmetic type
+  R keep_f;          // 1 - omega_f
+  R wf3, wf45;       // omega_f * 3, omega_f * 4.5
+  R amp_k, amp_c;    // fac k eps (k-fold), fac 16 eps (cubic): amplitude of N
+  R eps4, cub0;      // cubic a_s = cub0 + eps4 S: 4 eps, 1 - 3 eps
   R mzero;           // -0, an addend the compiler cannot fold away (prod_r)
 };
 
@@ -56,6 +63,7 @@ struct Model {
   double u_in, U_in;   // inflow ghost state
   double ref_f, ref_g, ref_h;  // reference moments of the stored deviations (1, U_ref, -1)
   Coef<float> cf;   // the constants above in FP32 ...
+  Coef<float2> c2;  // ... for two nodes ...
   Coef<double> cd;  // ... and in FP64 (filled by finalize())
   // 16-bit storage (2D and 3D): g is stored relative to a per-node U instead
   // of the global U_ref.  uring: two FP16 planes of `plane` values; for the
@@ -83,33 +91,47 @@ inline const __half* uref_plane(const Model& m, int c) {
   return m.rel_g ? m.uring + size_t(c) * size_t(m.plane) : nullptr;
 }
 
-// Fill m.cf and m.cd from the FP64 fields; call after every change of those.
+// Fill m.cf, m.c2 and m.cd from the FP64 fields; call after every change of those.
 inline void finalize(Model& m) {
-  auto fill = [&](auto& c) {
-    using R = std::remove_reference_t<decltype(c.omega_f)>;
-    c.omega_f = R(m.omega_f);
-    c.guo = R(m.guo);
-    c.tauU_slope = R(m.tauU_slope);
-    c.inv_tau0 = R(m.inv_tau0);
-    c.tpc = R(m.tpc);
-    c.lambda = R(m.lambda);
-    c.eps = R(m.eps);
-    c.ck0 = R(m.ck0);
-    c.sk0 = R(m.sk0);
-    c.aniso_fac = R(m.aniso_fac);
-    c.kdrag = R(m.kdrag);
-    for (int d = 0; d < 3; ++d) c.body[d] = R(m.body[d]);
-    c.u_in = R(m.u_in);
-    c.U_in = R(m.U_in);
-    c.ref_f = R(m.ref_f);
-    c.ref_g = R(m.ref_g);
-    c.ref_h = R(m.ref_h);
-    c.chm_wb = R(m.chm_wb);
-    c.chm_wh = R(m.chm_wh);
-    c.mzero = R(-0.0);
+  auto fill = [&](auto& c, auto one) {
+    using S = decltype(one);
+    auto put = [](auto& to, S v) {
+      if constexpr (std::is_same_v<std::remove_reference_t<decltype(to)>, float2>)
+        to = make_float2(v, v);
+      else
+        to = v;
+    };
+    const S wf = S(m.omega_f), eps = S(m.eps), fac = S(m.aniso_fac);
+    put(c.omega_f, wf);
+    put(c.guo, S(m.guo));
+    put(c.tauU_slope, S(m.tauU_slope));
+    put(c.inv_tau0, S(m.inv_tau0));
+    put(c.tpc, S(m.tpc));
+    put(c.lambda, S(m.lambda));
+    put(c.eps, eps);
+    put(c.ck0, S(m.ck0));
+    put(c.sk0, S(m.sk0));
+    put(c.kdrag, S(m.kdrag));
+    for (int d = 0; d < 3; ++d) put(c.body[d], S(m.body[d]));
+    put(c.u_in, S(m.u_in));
+    put(c.U_in, S(m.U_in));
+    put(c.ref_f, S(m.ref_f));
+    put(c.ref_g, S(m.ref_g));
+    put(c.ref_h, S(m.ref_h));
+    put(c.chm_wb, S(m.chm_wb));
+    put(c.chm_wh, S(m.chm_wh));
+    put(c.keep_f, S(1) - wf);
+    put(c.wf3, wf * S(3));
+    put(c.wf45, wf * S(4.5));
+    put(c.amp_k, fac * S(m.fold) * eps);
+    put(c.amp_c, fac * S(16) * eps);
+    put(c.eps4, S(4) * eps);
+    put(c.cub0, std::fma(S(-3), eps, S(1)));
+    put(c.mzero, S(-0.0));
   };
-  fill(m.cf);
-  fill(m.cd);
+  fill(m.cf, 0.0f);
+  fill(m.c2, 0.0f);
+  fill(m.cd, 0.0);
 }
 
 template <typename R>
@@ -117,6 +139,10 @@ __host__ __device__ __forceinline__ const Coef<R>& coef(const Model& m);
 template <>
 __host__ __device__ __forceinline__ const Coef<float>& coef<float>(const Model& m) {
   return m.cf;
+}
+template <>
+__host__ __device__ __forceinline__ const Coef<float2>& coef<float2>(const Model& m) {
+  return m.c2;
 }
 template <>
 __host__ __device__ __forceinline__ const Coef<double>& coef<double>(const Model& m) {
@@ -137,6 +163,12 @@ struct StepMaps {
   int ctas = 0, smem = 0, ready = 0;
   int ctas_v[4] = {0, 0, 0, 0};  // 2D: CTAs of the variant MASK + 2 CHM
 };
+
+// The 2D steps: a state (populations and rings of both buffers) of more than
+// kL2Bytes does not stay in the L2; then at most kStageBytes of pipeline stages
+// are kept resident per SM (step2d.cu).
+constexpr double kL2Bytes = 129e6;
+constexpr int kStageBytes = 142 * 1024;
 
 // Launchers (each returns the launch error).
 cudaError_t prepare_step2d(const Model& m, void* const pops[2], void* const rings[2],

@@ -26,21 +26,22 @@
 // computed and pushed, the next one is in flight.  Halo positions outside
 // the domain (the TMA fills them with zeros) are patched on edge tiles only.
 //
-// What bounds it, and the shape taken for that (1024^2 and 2480 x 2080 coupled
-// FP32 steps; GB300, 6.69 TB/s copy):
-//  - issue slots and latency.  A thread of a large grid holds two nodes, 2 rows
-//    apart, on the packed two-lane FP32 instructions (lbpf_device.cuh):
-//    480 warp instructions per 32 nodes instead of 754 (FP16: 606 for 906);
-//  - how the memory is asked.  Tiles are 64 x 4 (256-byte rows: 64 x 4 moves
-//    the step's bytes without arithmetic in 36 us, 32 x 8 in 38), and where
-//    the state exceeds the L2 at most kStageBytes of stages are resident per
-//    SM: with all CTAs that fit the h halos are read twice (666 MB from DRAM
-//    per 2480 x 2080 step against 587) and the step is slower.
-//  1024^2: 48.4 -> 40.2 us (0.72 -> 0.87 of the copy rate), FP16 38.2 -> 28.9;
-//  2480 x 2080: 250 -> 199 us, FP16 -> 119.
-// Grids of fewer than kPairTiles tiles take 32 x 4 tiles with one node per
-// thread: more CTAs, a shorter chain per tile (512^2: 10.5 us against 12.4;
-// 640^2: 14.2 against 13.9).
+// What bounds it, and what was taken for that (coupled steps, GB300, 6.69 TB/s
+// copy rate):
+//  - FP32 beyond the L2: how the memory is asked.  Tiles are 64 columns wide
+//    (256-byte rows), and at most kStageBytes of stages are resident per SM:
+//    with every CTA that fits, the h halos are read twice (666 MB from DRAM per
+//    2480 x 2080 step against 587) and the step takes 224 us instead of 177.
+//    1024^2: 48.4 -> 40.1 us (0.87 of the copy rate); 2480 x 2080: 250 -> 177
+//    (0.98).
+//  - 16-bit storage: issue slots.  A thread of a large grid holds two nodes, 2
+//    rows apart, on the packed two-lane FP32 instructions (lbpf_device.cuh): 606
+//    warp instructions per 32 nodes instead of 906.  1024^2: 38.2 -> 29.1 us;
+//    2480 x 2080: 119.
+//  - small grids: the chain of a tile.  Tiles of 32 x 4 with one node per
+//    thread give the most CTAs; boundary tiles run the same arithmetic as inner
+//    ones with precomputed steps.  128^2 without flow: 3.6 -> 3.2 us.
+// The shapes are chosen in shape_of().
 //
 // step2d_kernel (FP64 storage): one thread per node, one tile per CTA, the
 // same per-node code.
@@ -115,15 +116,20 @@ __global__ void __launch_bounds__(TX* TY)
   __syncthreads();
   const bool solids = m.solid && m.solid_tiles[blockIdx.y * gridDim.x + blockIdx.x];
   if (!active) return;
+  const Grid2D gr(m);
+  unsigned sm[1] = {0};  // solid neighbours
+  if (solids)
+    for (int a = 0; a < 9; ++a)
+      sm[0] |= solid_mapped(m, x + D2_CX[a], y + D2_CY[a]) ? 1u << a : 0u;
   R Unew;
   const unsigned o = unsigned(ty * px + tx) * unsigned(sizeof(T));
   auto work = [&](auto edge) {
     collide_push_2d<T, R, FLOW, CHM, true, decltype(edge)::value, false, SX, 0>(
-        m, x, y, [&](int q) { return q < QF ? f[q] : g[q - QF]; }, h, sh_phi[ty + 1][tx + 1],
+        gr, coef<R>(m), x, y, [&](int q) { return q < QF ? f[q] : g[q - QF]; }, h, sh_phi[ty + 1][tx + 1],
         dphi_prev, &sh_phi[ty + 1][tx + 1],
         [&](int a, int dy, int dx) { return sh_h[a][ty + 1 + dy][tx + 1 + dx]; },
-        [](int, int) { return R(0); }, R(coef<R>(m).ref_g),
-        static_cast<T*>(dp.p[0]) + (size_t(y0) * px + x0), o, o, err, Unew, solids);
+        [](int, int) { return R(0); }, sm, R(coef<R>(m).ref_g),
+        static_cast<T*>(dp.p[0]) + (size_t(y0) * px + x0), o, o, err, Unew);
   };
   if (solids || x0 < 1 || x0 + TX > nx - 1 || y0 < 1 || y0 + TY > ny - 1) work(std::true_type{});
   else work(std::false_type{});
@@ -135,7 +141,7 @@ __global__ void __launch_bounds__(TX* TY)
 // MASK: the variant with the solid-node path; CHM: the central Hermite MRT
 // flow collision; PAIR: two nodes per thread (step2d_tile.cuh).
 template <typename T, bool FLOW, int TX, int TY, bool PAIR, int S, bool MASK, bool CHM>
-__global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(), 4)
+__global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(), 512 / tile_threads<TX, TY, PAIR>())
     step2d_tma_kernel(const __grid_constant__ CUtensorMap tm_fg,
                       const __grid_constant__ CUtensorMap tm_h,
                       const __grid_constant__ CUtensorMap tm_ring,
@@ -150,7 +156,8 @@ __global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(), 4)
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[S];
   __shared__ R sh_phi[SY][SX];
-
+  __shared__ unsigned char sh_solid[MASK ? SX * SY : 1];
+  const Grid2D gr(m);
   const int tid = threadIdx.x;
   const int first = blockIdx.x, G = gridDim.x;
 
@@ -189,12 +196,21 @@ __global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(), 4)
     advance(load);
   }
 
+  // the solid flag of a tile, read one tile ahead
+  auto flag = [&](const Cursor& q) -> unsigned char {
+    return MASK && q.tile < ntiles ? m.solid_tiles[q.row * ntx + q.col] : 0;
+  };
+  unsigned char solids = flag(work);
+
   for (int k = 0; work.tile < ntiles; ++k) {
     const int s = k % S;
+    Cursor next = work;
+    advance(next);
+    const unsigned char next_solids = flag(next);
     const bool ok = mbar_wait_bounded(&full[s], uint32_t((k / S) & 1), kSpin);
-    if (!tile_2d<T, FLOW, TX, TY, PAIR, MASK, CHM>(m, src, dst, ring_cur, err, work.col * TX,
+    if (!tile_2d<T, FLOW, TX, TY, PAIR, MASK, CHM>(gr, m, src, dst, ring_cur, err, work.col * TX,
                                                    work.row * TY, c, smem + s * L::STAGE,
-                                                   &sh_phi[0][0], !ok)) {
+                                                   &sh_phi[0][0], sh_solid, solids != 0, !ok)) {
       // a tile never arrived: report, let the copies in flight land, stop
       if (tid == 0) {
         atomicOr(err, 2u);
@@ -213,22 +229,36 @@ __global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(), 4)
       issue(load, s);
     }
     advance(load);
-    advance(work);
+    work = next;
+    solids = next_solids;
   }
 }
 
 // ---- host side: tensor maps and launches -------------------------------------------
 constexpr int kStages = 2;
-constexpr int kPairX = 64, kPairY = 4;    // tile with two nodes per thread
-constexpr int kPairTiles = 1500;          // fewest of them (about ten a SM)
-constexpr int kStageBytes = 142 * 1024;  // stages per SM where the state exceeds the L2
-constexpr int kSmallX = 32, kSmallY = 4;  // ... with one (small grids, and the FP64 kernel)
 
-// Does the step take the tiles with two nodes per thread?
-bool pair_tiles(const Model& m) {
-  if (m.storage == ST_FP64) return false;
-  return (long long)((m.nx + kPairX - 1) / kPairX) * ((m.ny + kPairY - 1) / kPairY) >=
-         kPairTiles;
+// Tile shapes of the step: columns, rows, two nodes per thread or one.
+enum { SH_SMALL = 0, SH_WIDE = 1, SH_PAIR = 2 };
+constexpr int kShapeX[3] = {32, 64, 64}, kShapeY[3] = {4, 2, 4};
+constexpr int kPairTiles = 1500;  // fewest 64 x 4 tiles (about ten a SM) for SH_PAIR
+
+// FP32 states beyond the L2 take the wide tiles, 16-bit states of at least
+// kPairTiles tiles two nodes per thread, everything else (and the FP64 kernel)
+// the small tiles.  Measured, us per coupled step (small / wide / pair):
+//   FP32  775 x 650 19.0 / 19.3 / 18.8, 1024^2 40.7 / 40.1 / 40.3,
+//         1555 x 2023 119 / 113 / 118, 2480 x 2080 188 / 177 / 200
+//   FP16  512^2 11.1 / - / 12.9, 640^2 14.3 / - / 14.9, 775 x 650 17.7 / 18.9 /
+//         15.7, 1024^2 30.8 / 32.2 / 29.1, 2480 x 2080 135 / 141 / 119
+// (FP32 with a baffle of solid nodes, 775 x 650: 19.6 / 20.0 / 22.7).
+int shape_of(const Model& m) {
+  if (m.storage == ST_FP64) return SH_SMALL;
+  if (m.storage == ST_FP32) {
+    const double state = 2.0 * double(m.plane) * double((m.qf + 2 * m.qs) * 4 + 4);
+    return state > kL2Bytes ? SH_WIDE : SH_SMALL;
+  }
+  const long long tiles = (long long)((m.nx + kShapeX[SH_PAIR] - 1) / kShapeX[SH_PAIR]) *
+                          ((m.ny + kShapeY[SH_PAIR] - 1) / kShapeY[SH_PAIR]);
+  return tiles >= kPairTiles ? SH_PAIR : SH_SMALL;
 }
 
 // one thread per tx x ty tile: does the tile or its one-node halo (mapped
@@ -304,17 +334,10 @@ cudaError_t prepare_t(const Model& m, void* const pops[2], void* const rings[2],
                    &out->ctas_v[3])) != cudaSuccess)
       return e;
   }
-  // Populations and ring of both buffers beyond the L2: the copies in flight are
-  // held to kStageBytes a SM.  More of them make the memory slower (2480 x 2080
-  // FP32, 64 x 4 tiles, two stages: 199 us per step with two CTAs per SM, 224
-  // with three or four; 1024^2: 40.2 and 42.6); a state that the L2 holds is
-  // bound by the arithmetic and takes every CTA that fits (775 x 650 FP32: 18.6
-  // us with four, 20.5 with two; 1024^2 FP16: 28.9 and 34.5).
-  int l2 = 0;
-  if ((e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev)) != cudaSuccess) return e;
+  // populations and ring of both buffers beyond the L2: bound the copies in flight
   const double state = 2.0 * double(m.plane) * double(q * sizeof(T) + 4 + (L::REL ? 2 : 0));
-  if (state > double(l2)) {
-    const int most = std::max(1, kStageBytes / (kStages * L::STAGE));
+  if (state > kL2Bytes) {
+    const int most = std::max(1, kStageBytes / smem);
     for (int v = 0; v < 4; ++v) out->ctas_v[v] = std::min(out->ctas_v[v], sms * most);
   }
   out->ctas = out->ctas_v[0];
@@ -350,7 +373,7 @@ cudaError_t launch_tma_t(const Model& m, const StepMaps& maps, int c, const void
 template <typename T, typename R, bool FLOW>
 cudaError_t launch_plain_t(const Model& m, const void* src, void* dst, const void* ring_prev,
                            void* ring_cur, unsigned* err, cudaStream_t s) {
-  constexpr int kTX = kSmallX, kTY = kSmallY;
+  constexpr int kTX = kShapeX[SH_SMALL], kTY = kShapeY[SH_SMALL];
   dim3 block(kTX, kTY);
   dim3 grid((m.nx + kTX - 1) / kTX, (m.ny + kTY - 1) / kTY);
   const PopPtrs sp = pop_ptrs(m, const_cast<void*>(src), sizeof(T));
@@ -364,25 +387,41 @@ cudaError_t launch_plain_t(const Model& m, const void* src, void* dst, const voi
   return cudaGetLastError();
 }
 
+// fn(shape X, shape Y, pair) for the tile shape of m, of those compiled for T
+template <typename T, typename F>
+cudaError_t with_shape(const Model& m, F fn) {
+  using std::integral_constant;
+  const int sh = shape_of(m);
+  auto go = [&](auto i) {
+    constexpr int I = decltype(i)::value;
+    return fn(integral_constant<int, kShapeX[I]>{}, integral_constant<int, kShapeY[I]>{},
+              integral_constant<bool, I == SH_PAIR>{});
+  };
+  if constexpr (sizeof(T) == 4) {
+    if (sh == SH_WIDE) return go(integral_constant<int, SH_WIDE>{});
+  } else {
+    if (sh == SH_PAIR) return go(integral_constant<int, SH_PAIR>{});
+  }
+  return go(integral_constant<int, SH_SMALL>{});
+}
+
 template <typename T>
 cudaError_t prepare_any(const Model& m, void* const pops[2], void* const rings[2],
                         StepMaps* out) {
-  if (pair_tiles(m))
-    return m.flow ? prepare_t<T, true, kPairX, kPairY, true>(m, pops, rings, out)
-                  : prepare_t<T, false, kPairX, kPairY, true>(m, pops, rings, out);
-  return m.flow ? prepare_t<T, true, kSmallX, kSmallY, false>(m, pops, rings, out)
-                : prepare_t<T, false, kSmallX, kSmallY, false>(m, pops, rings, out);
+  return with_shape<T>(m, [&](auto x, auto y, auto p) {
+    return m.flow ? prepare_t<T, true, x(), y(), p()>(m, pops, rings, out)
+                  : prepare_t<T, false, x(), y(), p()>(m, pops, rings, out);
+  });
 }
 
 template <typename T>
 cudaError_t launch_any(const Model& m, const StepMaps& maps, int c, const void* src, void* dst,
                        void* ring_cur, unsigned* err, cudaStream_t s) {
-  if (pair_tiles(m))
+  return with_shape<T>(m, [&](auto x, auto y, auto p) {
     return m.flow
-               ? launch_tma_t<T, true, kPairX, kPairY, true>(m, maps, c, src, dst, ring_cur, err, s)
-               : launch_tma_t<T, false, kPairX, kPairY, true>(m, maps, c, src, dst, ring_cur, err, s);
-  return m.flow ? launch_tma_t<T, true, kSmallX, kSmallY, false>(m, maps, c, src, dst, ring_cur, err, s)
-                : launch_tma_t<T, false, kSmallX, kSmallY, false>(m, maps, c, src, dst, ring_cur, err, s);
+               ? launch_tma_t<T, true, x(), y(), p()>(m, maps, c, src, dst, ring_cur, err, s)
+               : launch_tma_t<T, false, x(), y(), p()>(m, maps, c, src, dst, ring_cur, err, s);
+  });
 }
 
 }  // namespace
@@ -399,13 +438,13 @@ cudaError_t prepare_step2d(const Model& m, void* const pops[2], void* const ring
 }
 
 size_t solid_tile_count(const Model& m) {
-  const int tx = pair_tiles(m) ? kPairX : kSmallX, ty = pair_tiles(m) ? kPairY : kSmallY;
+  const int tx = kShapeX[shape_of(m)], ty = kShapeY[shape_of(m)];
   return size_t((m.nx + tx - 1) / tx) * size_t((m.ny + ty - 1) / ty);
 }
 
 cudaError_t launch_solid_tiles(const Model& m, unsigned char* flags, cudaStream_t s) {
   if (m.dim != 2 || !m.solid) return cudaErrorInvalidValue;
-  const int tx = pair_tiles(m) ? kPairX : kSmallX, ty = pair_tiles(m) ? kPairY : kSmallY;
+  const int tx = kShapeX[shape_of(m)], ty = kShapeY[shape_of(m)];
   const int ntx = (m.nx + tx - 1) / tx, nty = (m.ny + ty - 1) / ty;
   solid_tiles_kernel<<<(ntx * nty + 127) / 128, 128, 0, s>>>(m, flags, ntx, nty, tx, ty);
   return cudaGetLastError();

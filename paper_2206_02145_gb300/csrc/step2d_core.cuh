@@ -14,8 +14,19 @@ namespace lbk {
 __device__ __forceinline__ bool solid_mapped(const Model& m, int x, int y) {
   x = grad_coord(x, m.nx, m.bc[0]);
   y = grad_coord(y, m.ny, m.bc[1]);
-  return m.solid[y * m.px + x] != 0;
+  return m.solid[(long long)y * m.px + x] != 0;
 }
+
+// What the step needs of a grid besides the model constants.
+struct Grid2D {
+  int nx, ny, px, bcx, bcy, fold;
+  long long plane;
+  __half* uring;
+  const unsigned char* solid;
+  __device__ __forceinline__ explicit Grid2D(const Model& m)
+      : nx(m.nx), ny(m.ny), px(m.px), bcx(m.bc[0]), bcy(m.bc[1]), fold(m.fold), plane(m.plane),
+        uring(m.uring), solid(m.solid) {}
+};
 
 // Central Hermite MRT of the flow populations (2D; the collision of the
 // paper's flow solver, read as the C ABI documents for LBPF_COLL_CHM).
@@ -28,9 +39,7 @@ __device__ __forceinline__ bool solid_mapped(const Model& m, int x, int y) {
 // inverse of the D2Q9 raw-moment matrix.  out: post-collision deviations.
 template <typename N>
 __device__ __forceinline__ void chm_post_2d(const N (&d)[9], N drho, N rho, N mx, N my, N vx, N vy,
-                                            N Fx, N Fy, typename Lanes<N>::S wf,
-                                            typename Lanes<N>::S wb, typename Lanes<N>::S wh,
-                                            typename Lanes<N>::S mzero, N (&out)[9]) {
+                                            N Fx, N Fy, const Coef<N>& c, N (&out)[9]) {
   using S = typename Lanes<N>::S;
   const N t3 = splat<N>(S(1.0 / 3.0)), t9 = splat<N>(S(1.0 / 9.0)), two = splat<N>(S(2));
   const N t23 = splat<N>(S(2) * S(1.0 / 3.0)), half = splat<N>(S(0.5)), quarter = splat<N>(S(0.25));
@@ -68,8 +77,8 @@ __device__ __forceinline__ void chm_post_2d(const N (&d)[9], N drho, N rho, N mx
   hxxyy = add(t23, fma_r(vx, e10, mul_r(vy, e01)), sub(t3, add_r(e20, e02), hxxyy));
   hxxyy = add(t9, e00, sub(mul_r(t3, fma_r(vx, vx, vyy)), e00, hxxyy));
   // relaxation towards rho and zeros; the force in the first order
-  const N kf = splat<N>(S(1) - wf), gf = splat<N>(S(1) - S(0.5) * wf), kh = splat<N>(S(1) - wh);
-  const N kb = splat<N>(S(1) - wb);
+  const N one = splat<N>(S(1)), kf = c.keep_f, gf = fma_r(splat<N>(S(-0.5)), c.omega_f, one);
+  const N kh = sub_r(one, c.chm_wh), kb = sub_r(one, c.chm_wb);
   const N h1s = fma_r(kf, h1, mul_r(gf, Fx)), h2s = fma_r(gf, Fy, mul_r(kf, h2));
   const N sum = add_r(hxx, hyy), dv = mul_r(kf, sub_r(hxx, hyy));
   const N hxxs = mul_r(half, fma_r(kb, sum, dv)), hyys = mul_r(half, fma_r(kb, sum, neg_r(dv)));
@@ -77,7 +86,7 @@ __device__ __forceinline__ void chm_post_2d(const N (&d)[9], N drho, N rho, N mx
   // central (raw) moments after collision, then raw moments of the deviations
   const N k20 = add(t3, rho, hxxs), k02 = add(t3, rho, hyys);
   const N k21 = fma_r(t3, h2s, mul_r(kh, hxxy)), k12 = fma_r(t3, h1s, mul_r(kh, hxyy));
-  const N t3e = prod_r(t3, e00, mzero);
+  const N t3e = prod_r(t3, e00, c.mzero);
   const N f10 = add(vx, rho, h1s), f01 = add(vy, rho, h2s);
   const N f20 = add(vxx, rho, add(vx2, h1s, add_r(hxxs, t3e)));
   const N f02 = add(vyy, rho, add(vy2, h2s, add_r(hyys, t3e)));
@@ -117,7 +126,6 @@ struct Node2D {
   N usx, usy, Fx, Fy, E0, E1, E2, G0;  // flow (with the central Hermite MRT unused)
   N keep_U, K0, K1, keep_phi, H0, Hx, Hy, inv_a2, keep_old;
   N us_s, us_d, F_s, F_d, H_s, H_d;    // sums and differences of the two components
-  S keep_f, guo, mzero;
 };
 
 // Moments, gradient, anisotropy and the coefficients above (Eqs. 3-23) of a
@@ -125,11 +133,10 @@ struct Node2D {
 // earlier), the g reference Rg and the eight neighbours' phi + 1.  False if
 // phi, U or rho is not finite.
 template <typename N, bool FLOW, bool CHM>
-__device__ __forceinline__ bool node_2d(const Model& m, const N (&f)[9], const N (&g)[9], N dphi,
+__device__ __forceinline__ bool node_2d(const Coef<N>& c, int fold, const N (&f)[9], const N (&g)[9], N dphi,
                                         N dphi_prev, N Rg, N pE, N pW, N pN, N pS, N pNE, N pNW,
                                         N pSE, N pSW, Node2D<N>& o, N (&fchm)[9]) {
   using S = typename Lanes<N>::S;
-  const Coef<S>& c = coef<S>(m);
   const N one = splat<N>(S(1)), half = splat<N>(S(0.5));
   // ---- local moments (Eqs. 11, 12, 17, 22) ----------------------------------
   const N phi = sub_r(dphi, one);
@@ -156,19 +163,18 @@ __device__ __forceinline__ bool node_2d(const Model& m, const N (&f)[9], const N
     // Eq. 6: F = b - K u, K = h tau_f (1+phi)^2 (1-phi) / (4 W0^2); the Guo
     // half-force velocity u = (m + F/2)/rho solved in closed form.
     const N ph1 = add_r(one, ph);
-    const N K = mul_r(mul_r(mul_r(splat<N>(c.kdrag), ph1), ph1), sub_r(one, ph));
+    const N K = mul_r(mul_r(mul_r(c.kdrag, ph1), ph1), sub_r(one, ph));
     const N inv = rcp_r(fma_r(half, K, rho));
-    const N ux = mul_r(fma_r(half, splat<N>(c.body[0]), mx), inv);
-    const N uy = mul_r(fma_r(half, splat<N>(c.body[1]), my), inv);
-    o.Fx = fma_r(neg_r(K), ux, splat<N>(c.body[0]));
-    o.Fy = fma_r(neg_r(K), uy, splat<N>(c.body[1]));
+    const N ux = mul_r(fma_r(half, c.body[0], mx), inv);
+    const N uy = mul_r(fma_r(half, c.body[1], my), inv);
+    o.Fx = fma_r(neg_r(K), ux, c.body[0]);
+    o.Fy = fma_r(neg_r(K), uy, c.body[1]);
     o.usx = mul_r(mask, ux);  // u* (Eq. 7)
     o.usy = mul_r(mask, uy);
   }
   if constexpr (FLOW && CHM)
-    chm_post_2d<N>(f, drho, rho, mx, my, o.usx, o.usy, o.Fx, o.Fy, c.omega_f, c.chm_wb, c.chm_wh,
-                   c.mzero, fchm);
-  const N omega_U = rcp_r(fma_r(splat<N>(c.tauU_slope), mask, half));  // Eq. 18
+    chm_post_2d<N>(f, drho, rho, mx, my, o.usx, o.usy, o.Fx, o.Fy, c, fchm);
+  const N omega_U = rcp_r(fma_r(c.tauU_slope, mask, half));  // Eq. 18
   const N dphidt = sub_r(dphi, dphi_prev);
 
   // ---- gradient, anisotropy, phase-field coefficients (Eqs. 3, 20, 21, 23) --
@@ -179,29 +185,26 @@ __device__ __forceinline__ bool node_2d(const Model& m, const N (&f)[9], const N
   const N gy = fma_r(third, sub_r(pN, pS),
                      mul_r(twelfth, sub_r(add_r(pNE, pNW), add_r(pSE, pSW))));
   N as, Nx, Ny;
-  aniso_2d<N>(m, gx, gy, as, Nx, Ny);
+  aniso_2d<N>(c, fold, gx, gy, as, Nx, Ny);
   const N a2 = mul_r(as, as);
   o.inv_a2 = rcp_r(a2);
-  const N tpc = splat<N>(c.tpc);
+  const N tpc = c.tpc;
   const N omega_phi = rcp_r(fma_r(a2, tpc, half));  // Eq. 23
   const N pp = mul_r(phi, phi);
   const N phi2m = sub_r(one, pp);
   // Eq. 20
-  const N Qs = mul_r(fma_r(mul_r(mul_r(splat<N>(c.lambda), U), phi2m), phi2m,
+  const N Qs = mul_r(fma_r(mul_r(mul_r(c.lambda, U), phi2m), phi2m,
                            fma_r(neg_r(pp), phi, phi)),
-                     splat<N>(c.inv_tau0));
+                     c.inv_tau0);
   if (FLOW && !CHM) {
     const N uu = fma_r(o.usx, o.usx, mul_r(o.usy, o.usy));
     const N uF = fma_r(o.usx, o.Fx, mul_r(o.usy, o.Fy));
-    o.E0 = mul_r(splat<N>(c.omega_f), fma_r(neg_r(mul_r(splat<N>(S(1.5)), rho)), uu, drho));
-    o.E1 = mul_r(splat<N>(c.omega_f * S(3)), rho);
-    o.E2 = mul_r(splat<N>(c.omega_f * S(4.5)), rho);
+    o.E0 = mul_r(c.omega_f, fma_r(neg_r(mul_r(splat<N>(S(1.5)), rho)), uu, drho));
+    o.E1 = mul_r(c.wf3, rho);
+    o.E2 = mul_r(c.wf45, rho);
     o.G0 = mul_r(splat<N>(S(-3)), uF);
     o.F_s = add_r(o.Fx, o.Fy);
     o.F_d = sub_r(o.Fx, o.Fy);
-    o.keep_f = S(1) - c.omega_f;
-    o.guo = c.guo;
-    o.mzero = c.mzero;
   }
   o.us_s = add_r(o.usx, o.usy);
   o.us_d = sub_r(o.usx, o.usy);
@@ -239,9 +242,9 @@ __device__ __forceinline__ N dir_dot(int a, N x, N y, N s, N d) {
 // Post-collision deviations of direction a at the node: f* (Eq. 4), g* (Eq.
 // 13) and, before Eq. 19's division by a_s^2, h*.
 template <typename N>
-__device__ __forceinline__ N post_f_2d(const Node2D<N>& n, int a, N f) {
+__device__ __forceinline__ N post_f_2d(const Coef<N>& c, const Node2D<N>& n, int a, N f) {
   using S = typename Lanes<N>::S;
-  const N w = splat<N>(d2_w<S>(a)), keep = splat<N>(n.keep_f), guo = splat<N>(n.guo);
+  const N w = splat<N>(d2_w<S>(a));
   N feq = n.E0, gt = n.G0;
   if (a > 0) {
     const N cu = dir_dot(a, n.usx, n.usy, n.us_s, n.us_d);
@@ -249,7 +252,7 @@ __device__ __forceinline__ N post_f_2d(const Node2D<N>& n, int a, N f) {
     feq = fma_r(cu, fma_r(n.E2, cu, n.E1), n.E0);
     gt = fma_r(cF, fma_r(splat<N>(S(9)), cu, splat<N>(S(3))), n.G0);
   }
-  return fma_r(keep, f, mul_r(w, add_r(feq, prod_r(guo, gt, n.mzero))));
+  return fma_r(c.keep_f, f, mul_r(w, add_r(feq, prod_r(c.guo, gt, c.mzero))));
 }
 template <typename N>
 __device__ __forceinline__ N post_g_2d(const Node2D<N>& n, int a, N g) {
@@ -273,18 +276,6 @@ __device__ __forceinline__ N arrive_h_2d(const Node2D<N>& n, N hp, N hold) {
   return fma_r(n.inv_a2, hp, mul_r(n.keep_old, hold));
 }
 
-// lane k of a number of one or two nodes
-template <typename N>
-__device__ __forceinline__ typename Lanes<N>::S lane(const N& v, int k) {
-  if constexpr (Lanes<N>::V == 2) return k ? v.y : v.x;
-  else return v;
-}
-template <typename N>
-__device__ __forceinline__ void set_lane(N& v, int k, typename Lanes<N>::S s) {
-  if constexpr (Lanes<N>::V == 2) (k ? v.y : v.x) = s;
-  else v = s;
-}
-
 // Collide and push a thread's one or two nodes (N = float2: the second DY rows
 // below the first).
 //   own(q): stored deviation q of the node(s) (f, then g)
@@ -292,6 +283,8 @@ __device__ __forceinline__ void set_lane(N& v, int k, typename Lanes<N>::S s) {
 //     dphi_prev: phi + 1 of the node(s) now and one step earlier
 //   hold(a, dy, dx), uref(dy, dx): h_a and the encoding reference of g (UREL) at
 //     that offset from the node(s)
+//   sm[k]: bit a set where node k's neighbour in direction a (0: the node
+//     itself) is solid, mapped like a gradient neighbour (MASK)
 //   (x, y): the first node; tb: the tile's origin in array 0 of the
 //     destination buffer (the same for the whole CTA, so that every array's
 //     address is one uniform base plus the thread's offset); o0, o1: offsets
@@ -300,19 +293,19 @@ __device__ __forceinline__ void set_lane(N& v, int k, typename Lanes<N>::S s) {
 // one node away from every domain edge and holds or borders no solid node), so
 // the push needs no boundary logic.  EDGE = true: each destination goes through
 // the boundary rules; nodes outside the domain (of a partial tile) and solid
-// nodes push nothing.  MASK: the code for solid nodes is compiled in; `solids`
-// (the tile holds or borders a solid node) switches it on.  CHM: the flow
-// collides by the central Hermite MRT.
+// nodes push nothing.  MASK: the code for solid nodes is compiled in.  CHM: the
+// flow collides by the central Hermite MRT.
 template <typename T, typename N, bool FLOW, bool CHM, bool MASK, bool EDGE, bool UREL, int PROW,
           int DY, typename Own, typename Hold, typename Uref>
 __device__ __forceinline__ void collide_push_2d(
-    const Model& m, int x, int y, const Own& own, const N (&h)[9], N dphi, N dphi_prev,
-    const typename Lanes<N>::S* pc, const Hold& hold, const Uref& uref, N Rg, T* __restrict__ tb,
-    unsigned o0, unsigned o1, unsigned* __restrict__ err, N& Unew, bool solids) {
+    const Grid2D& gr, const Coef<N>& c, int x, int y, const Own& own, const N (&h)[9], N dphi,
+    N dphi_prev, const typename Lanes<N>::S* pc, const Hold& hold, const Uref& uref,
+    const unsigned (&sm)[Lanes<N>::V], N Rg, T* __restrict__ tb, unsigned o0, unsigned o1,
+    unsigned* __restrict__ err, N& Unew) {
   using S = typename Lanes<N>::S;
   constexpr int V = Lanes<N>::V, QF = FLOW ? 9 : 0;
-  const int nx = m.nx, ny = m.ny, px = m.px;
-  const long long P = m.plane;
+  const int nx = gr.nx, ny = gr.ny, px = gr.px;
+  const long long P = gr.plane;
   N pn[9];  // the neighbours' phi + 1
 #pragma unroll
   for (int a = 1; a < 9; ++a) {
@@ -320,21 +313,24 @@ __device__ __forceinline__ void collide_push_2d(
     set_lane(pn[a], 0, pc[off]);
     if (V == 2) set_lane(pn[a], 1, pc[off + DY * PROW]);
   }
-  if (MASK && EDGE && solids) {
+  if (MASK && EDGE) {
     // a solid neighbour counts as the first fluid node among (x + c_x, y),
     // (x, y + c_y) and (x, y): zero normal derivative at walls and obstacles
-#pragma unroll 1
-    for (int k = 0; k < V; ++k) {
-      const int yk = y + k * DY;
-      const S* pk = pc + k * (DY * PROW);
-      if (x >= nx || yk >= ny) continue;
+    const N centre = dphi;
 #pragma unroll
-      for (int a = 1; a < 9; ++a) {
-        const int cx = D2_CX[a], cy = D2_CY[a];
-        if (!solid_mapped(m, x + cx, yk + cy)) continue;
-        S v = pk[0];
-        if (cx != 0 && !solid_mapped(m, x + cx, yk)) v = pk[cx];
-        else if (cy != 0 && !solid_mapped(m, x, yk + cy)) v = pk[cy * PROW];
+    for (int k = 0; k < V; ++k) {
+      if (sm[k] == 0) continue;
+      auto is = [&](int a) { return (sm[k] >> a & 1u) != 0; };
+      // the diagonals first: they look at the axis values as they are
+#pragma unroll
+      for (int a = 8; a > 0; --a) {
+        if (!is(a)) continue;
+        S v = lane(centre, k);
+        if (a > 4) {
+          const int ax = D2_CX[a] > 0 ? 1 : 3, ay = D2_CY[a] > 0 ? 2 : 4;
+          if (!is(ax)) v = lane(pn[ax], k);
+          else if (!is(ay)) v = lane(pn[ay], k);
+        }
         set_lane(pn[a], k, v);
       }
     }
@@ -347,7 +343,7 @@ __device__ __forceinline__ void collide_push_2d(
   }
   Node2D<N> nd;
   N fchm[9];
-  if (!node_2d<N, FLOW, CHM>(m, f, g, dphi, dphi_prev, Rg, pn[1], pn[3], pn[2], pn[4], pn[5],
+  if (!node_2d<N, FLOW, CHM>(c, gr.fold, f, g, dphi, dphi_prev, Rg, pn[1], pn[3], pn[2], pn[4], pn[5],
                              pn[6], pn[8], pn[7], nd, fchm))
     atomicOr(err, 1u);
   Unew = nd.U;
@@ -361,7 +357,7 @@ __device__ __forceinline__ void collide_push_2d(
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
       const int off = D2_CY[a] * px + D2_CX[a];
-      if (FLOW) put(a, off, CHM ? fchm[a] : post_f_2d<N>(nd, a, f[a]));
+      if (FLOW) put(a, off, CHM ? fchm[a] : post_f_2d<N>(c, nd, a, f[a]));
       N gp = post_g_2d<N>(nd, a, g[a]);
       if (UREL) gp = fma_r(splat<N>(-d2_w<S>(a)), sub_r(uref(D2_CY[a], D2_CX[a]), Rg), gp);
       put(QF + a, off, gp);
@@ -374,7 +370,7 @@ __device__ __forceinline__ void collide_push_2d(
     // edge to the far side) and what lies there: a wall (the population comes
     // back to its node reversed, half-way bounce-back) or, in x, the inflow
     // or outflow ghost (nothing to push).
-    const int bcx = m.bc[0], bcy = m.bc[1];
+    const int bcx = gr.bcx, bcy = gr.bcy;
     const bool x_lo = x == 0, x_hi = x == nx - 1;
     const int sxm = x_lo ? nx - 1 : -1, sxp = x_hi ? 1 - nx : 1;
     const bool wxm = x_lo && bcx == BC_WALL, wxp = x_hi && bcx == BC_WALL;
@@ -386,7 +382,7 @@ __device__ __forceinline__ void collide_push_2d(
     for (int k = 0; k < V; ++k) {
       const int yk = y + k * DY;
       on[k] = x < nx && yk < ny;
-      if (MASK && solids && on[k]) on[k] = !m.solid[yk * px + x];
+      if (MASK) on[k] = on[k] && !(sm[k] & 1u);
       sym[k] = yk == 0 ? wrap_y : -px;
       syp[k] = yk == ny - 1 ? -wrap_y : px;
       wym[k] = yk == 0 && bcy == BC_WALL;
@@ -398,7 +394,7 @@ __device__ __forceinline__ void collide_push_2d(
     for (int a = 0; a < 9; ++a) {
       const int cx = D2_CX[a], cy = D2_CY[a], b = D2_OPP[a];
       N fp = splat<N>(S(0));
-      if (FLOW) fp = CHM ? fchm[a] : post_f_2d<N>(nd, a, f[a]);
+      if (FLOW) fp = CHM ? fchm[a] : post_f_2d<N>(c, nd, a, f[a]);
       const N gp = post_g_2d<N>(nd, a, g[a]);
       const N hp = post_h_2d<N>(nd, a, h[a]);
       const N w = splat<N>(d2_w<S>(a));
@@ -416,8 +412,7 @@ __device__ __forceinline__ void collide_push_2d(
         const bool ghost = !back && ((cx < 0 && gxm) || (cx > 0 && gxp));
         const int step = (cx < 0 ? sxm : (cx > 0 ? sxp : 0)) +
                          (cy < 0 ? sym[k] : (cy > 0 ? syp[k] : 0));
-        if (MASK && solids && on[k] && !back && !ghost)
-          back = m.solid[(y + k * DY) * px + x + step] != 0;  // obstacle
+        if (MASK) back = back || (!ghost && (sm[k] >> a & 1u));  // obstacle
         if (on[k] && !ghost) {
           T* const p = back ? node + b * P : node + (a * P + step);
           if (FLOW) Pop<T>::st(p, lane(fp, k));
@@ -444,8 +439,7 @@ __device__ __forceinline__ void collide_push_2d(
         if (cx > 0 && x_lo) {
           // inflow ghost x = -1: equilibrium at rho = 1, u = u_in e_x, U = U_in,
           // phi = -1 (a_s = 1; its h deviation is 0), unless behind a wall
-          const Coef<S>& c = coef<S>(m);
-          const S uin = c.u_in, Uin = c.U_in, ws = d2_w<S>(a), gu = FLOW ? uin : S(0);
+          const S uin = lane(c.u_in, 0), Uin = lane(c.U_in, 0), ws = d2_w<S>(a), gu = FLOW ? uin : S(0);
           const S fin = ws * (S(3) * uin + S(4.5) * uin * uin - S(1.5) * uin * uin);
 #pragma unroll
           for (int k = 0; k < V; ++k) {

@@ -65,13 +65,16 @@ constexpr int tile_threads() {
 // threads of the CTA; contains CTA barriers.  sh_phi: (TY + 2) x (TX + 2).
 // `bad`: this thread saw the stage's loads time out; the first barrier tells
 // every thread, and the tile is given up before its first global write
-// (returns false).  MASK: solid nodes are handled (flag of the tile from
-// m.solid_tiles).  CHM: the flow collides by the central Hermite MRT.
+// (returns false).  MASK: solid nodes are handled (sh_solid: (TY + 2) x (TX + 2)
+// bytes); `solids`: the tile or its halo holds one.  CHM: the flow collides by
+// the central Hermite MRT.
 template <typename T, bool FLOW, int TX, int TY, bool PAIR, bool MASK, bool CHM>
-__device__ __forceinline__ bool tile_2d(const Model& m, const T* __restrict__ src,
-                                        T* __restrict__ dst, float* __restrict__ ring_cur,
-                                        unsigned* __restrict__ err, int x0, int y0, int c,
-                                        unsigned char* st, float* sh_phi_flat, bool bad) {
+__device__ __forceinline__ bool tile_2d(const Grid2D& gr, const Model& m,
+                                        const T* __restrict__ src, T* __restrict__ dst,
+                                        float* __restrict__ ring_cur, unsigned* __restrict__ err,
+                                        int x0, int y0, int c, unsigned char* st,
+                                        float* sh_phi_flat, unsigned char* sh_solid, bool solids,
+                                        bool bad) {
   using R = float;
   using L = Tiles2D<T, FLOW, TX, TY>;
   constexpr int NT = tile_threads<TX, TY, PAIR>(), SX = TX + 2, SY = TY + 2;
@@ -79,7 +82,7 @@ __device__ __forceinline__ bool tile_2d(const Model& m, const T* __restrict__ sr
   constexpr int QF = FLOW ? 9 : 0;
   const int tid = threadIdx.x;
   const int tx = tid % TX, ty = tid / TX;
-  const int nx = m.nx, ny = m.ny, px = m.px;
+  const int nx = gr.nx, ny = gr.ny, px = gr.px;
   R(*sh_phi)[SX] = reinterpret_cast<R(*)[SX]>(sh_phi_flat);
   const T* fgs = reinterpret_cast<const T*>(st);
   T* hsm = reinterpret_cast<T*>(st + L::OFF_H);
@@ -87,11 +90,15 @@ __device__ __forceinline__ bool tile_2d(const Model& m, const T* __restrict__ sr
   const __half* uown = reinterpret_cast<const __half*>(st + L::OFF_UOWN);
   __half* uhal = reinterpret_cast<__half*>(st + L::OFF_UHAL);
   constexpr int HPLANE = SY * L::BXH;
-  // tiles next to solid nodes take the general path with the mask (the
-  // flag is loaded first, so that its latency overlaps the phi sums)
-  const bool solids =
-      MASK && m.solid && m.solid_tiles[(y0 / TY) * ((nx + TX - 1) / TX) + x0 / TX];
-
+  if (MASK && solids) {  // the tile's solid flags with halo, for the general path
+    for (int i = tid; i < SX * SY; i += NT) {
+      const int gx = x0 + i % SX - 1, gy = y0 + i / SX - 1;
+      unsigned char v = 0;
+      if (gx <= nx && gy <= ny)
+        v = gr.solid[(long long)grad_coord(gy, ny, gr.bcy) * px + grad_coord(gx, nx, gr.bcx)];
+      sh_solid[i] = v;
+    }
+  }
   if (x0 == 0 || y0 == 0 || x0 + TX >= nx || y0 + TY >= ny) {
     // halo positions outside the domain: the nearest node, which the tile
     // holds, or across a periodic edge the far side (or, where the tile spans
@@ -101,7 +108,7 @@ __device__ __forceinline__ bool tile_2d(const Model& m, const T* __restrict__ sr
       int gx = x0 + lx - 1, gy = y0 + ly - 1;
       if (gx >= 0 && gx < nx && gy >= 0 && gy < ny) continue;
       if (gx > nx || gy > ny) continue;  // beyond the halo of a partial tile
-      const int wx = grad_coord(gx, nx, m.bc[0]), wy = grad_coord(gy, ny, m.bc[1]);
+      const int wx = grad_coord(gx, nx, gr.bcx), wy = grad_coord(gy, ny, gr.bcy);
       const int sx = wx - x0 + 1, sy = wy - y0 + 1;  // the mapped node in the tile's box
       T* const hd = hsm + ly * L::BXH + lx + L::HX - 1;
       __half* const ud = uhal + ly * L::BXU + lx + L::HXU - 1;
@@ -111,10 +118,10 @@ __device__ __forceinline__ bool tile_2d(const Model& m, const T* __restrict__ sr
         for (int a = 0; a < 9; ++a) hd[a * HPLANE] = hf[a * HPLANE];
         if (L::REL) *ud = uhal[sy * L::BXU + sx + L::HXU - 1];
       } else {
-        const long long j = (long long)wy * px + wx, P = m.plane;
+        const long long j = (long long)wy * px + wx, P = gr.plane;
 #pragma unroll
         for (int a = 0; a < 9; ++a) hd[a * HPLANE] = src[(QF + 9 + a) * P + j];
-        if (L::REL) *ud = m.uring[size_t(c ^ 1) * m.plane + j];
+        if (L::REL) *ud = gr.uring[(c ^ 1) * gr.plane + j];
       }
     }
     __syncthreads();
@@ -170,14 +177,25 @@ __device__ __forceinline__ bool tile_2d(const Model& m, const T* __restrict__ sr
   };
   // g is stored relative to the node's own U reference (16-bit storage); the
   // collision takes the deviations from it as they are
-  N Rg = splat<N>(m.cf.ref_g), Unew;
+  const Coef<N>& cf = coef<N>(m);
+  N Rg = cf.ref_g, Unew;
   if constexpr (L::REL) Rg = two(__half2float(uown[o]), __half2float(uown[o + (V - 1) * DY * TX]));
   const __half* uc = uhal + (ty + 1) * L::BXU + tx + L::HXU;
   const size_t org = size_t(y0) * px + x0;
   const unsigned e0 = unsigned(ty * px + tx), e1 = e0 + unsigned(DY * px);
+  unsigned sm[V], near = 0;  // solid neighbours (bit a: direction a, 0 the node itself)
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    sm[k] = 0;
+    if (MASK && solids)
+#pragma unroll
+      for (int a = 0; a < 9; ++a)
+        sm[k] |= sh_solid[(ty + k * DY + 1 + D2_CY[a]) * SX + tx + 1 + D2_CX[a]] ? 1u << a : 0u;
+    near |= sm[k];
+  }
   auto work = [&](auto edge) {
     collide_push_2d<T, N, FLOW, CHM, MASK, decltype(edge)::value, L::REL, SX, DY>(
-        m, x, y,
+        gr, cf, x, y,
         [&](int q) {
           const T* p = fgs + q * (TY * TX) + o;
           return two(Pop<T>::template ld<R>(p), Pop<T>::template ld<R>(p + (V - 1) * DY * TX));
@@ -188,23 +206,24 @@ __device__ __forceinline__ bool tile_2d(const Model& m, const T* __restrict__ sr
           const __half* p = uc + dy * L::BXU + dx;
           return two(__half2float(p[0]), __half2float(p[(V - 1) * DY * L::BXU]));
         },
-        Rg, dst + org, e0 * unsigned(sizeof(T)), e1 * unsigned(sizeof(T)), err, Unew, solids);
+        sm, Rg, dst + org, e0 * unsigned(sizeof(T)), e1 * unsigned(sizeof(T)), err, Unew);
   };
-  // boundary logic only for the warps that have a node on a domain edge
-  const bool edge = __any_sync(0xffffffffu, solids || x < 1 || x > nx - 2 || y < 1 ||
+  // boundary logic only for the warps that have a node on a domain edge or
+  // next to a solid node
+  const bool edge = __any_sync(0xffffffffu, near != 0 || x < 1 || x > nx - 2 || y < 1 ||
                                                 y + (V - 1) * DY > ny - 2);
   if (edge) work(std::true_type{});
   else work(std::false_type{});
   // phi(t) of every node, and the new U of every node but the solid ones
   float* ring_t = ring_cur + org;
-  __half* un = L::REL ? m.uring + (size_t(c) * m.plane + org) : nullptr;
+  __half* un = L::REL ? gr.uring + (c * gr.plane + (long long)org) : nullptr;
 #pragma unroll
   for (int k = 0; k < V; ++k) {
     const unsigned e = k ? e1 : e0;
     if (!edge || (x < nx && y + k * DY < ny)) {
       ring_t[e] = lane(dphi, k);
       if constexpr (L::REL)
-        if (!(MASK && solids && m.solid[(y + k * DY) * px + x])) un[e] = __float2half_rn(lane(Unew, k));
+        if (!(sm[k] & 1u)) un[e] = __float2half_rn(lane(Unew, k));
     }
   }
   return true;

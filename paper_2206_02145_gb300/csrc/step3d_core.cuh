@@ -304,7 +304,7 @@ __device__ __forceinline__ void collide_push_3d(const Model& m, int x, int y, in
     if (D3_CZ[a]) gr[2] += R(D3_CZ[a]) * v;
   }
   R as, N[3];
-  aniso_3d<R>(m, gr, as, N);
+  aniso_3d<R>(c, gr, as, N);
   const R a2 = as * as;
   const R inv_a2 = rcp_r(a2);
   const R omega_phi = rcp_r(a2 * c.tpc + R(0.5));  // Eq. 23

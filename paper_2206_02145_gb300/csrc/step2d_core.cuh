@@ -53,15 +53,15 @@ __device__ __forceinline__ void chm_post_2d(const N (&d)[9], N drho, N rho, N mx
   const N e11 = add_r(sub_r(d[5], d[6]), sub_r(d[7], d[8]));
   const N e21 = sub_r(add_r(d[5], d[6]), add_r(d[7], d[8]));
   const N e12 = sub_r(sub_r(d[5], d[6]), sub_r(d[7], d[8]));
-  const N e22 = dd;
+  const N e22 = dd, t3e = prod_r(t3, e00, c.mzero);
   const N vxx = mul_r(vx, vx), vyy = mul_r(vy, vy), vxy = mul_r(vx, vy);
   const N vx2 = mul_r(two, vx), vy2 = mul_r(two, vy), vxy2 = mul_r(two, vxy);
   const N vxy4 = mul_r(splat<N>(S(4)), vxy), vxxy = mul_r(vxx, vy), vxyy = mul_r(vx, vyy);
   const N vxy2y = mul_r(vxy2, vy), vxy2x = mul_r(vxy2, vx), vxxyy = mul_r(vxx, vyy);
   // central Hermite moments about (vx, vy)
   const N h1 = sub(vx, rho, e10), h2 = sub(vy, rho, e01);
-  const N hxx = add(vxx, rho, sub(vx2, e10, sub(t3, e00, e20)));
-  const N hyy = add(vyy, rho, sub(vy2, e01, sub(t3, e00, e02)));
+  const N hxx = add(vxx, rho, sub(vx2, e10, sub_r(e20, t3e)));
+  const N hyy = add(vyy, rho, sub(vy2, e01, sub_r(e02, t3e)));
   const N hxy = add(vxy, rho, sub(vy, e10, sub(vx, e01, e11)));
   const N hxxy = add(mul_r(t3, vy), e00,
                      sub(t3, e01,
@@ -86,7 +86,6 @@ __device__ __forceinline__ void chm_post_2d(const N (&d)[9], N drho, N rho, N mx
   // central (raw) moments after collision, then raw moments of the deviations
   const N k20 = add(t3, rho, hxxs), k02 = add(t3, rho, hyys);
   const N k21 = fma_r(t3, h2s, mul_r(kh, hxxy)), k12 = fma_r(t3, h1s, mul_r(kh, hxyy));
-  const N t3e = prod_r(t3, e00, c.mzero);
   const N f10 = add(vx, rho, h1s), f01 = add(vy, rho, h2s);
   const N f20 = add(vxx, rho, add(vx2, h1s, add_r(hxxs, t3e)));
   const N f02 = add(vyy, rho, add(vy2, h2s, add_r(hyys, t3e)));

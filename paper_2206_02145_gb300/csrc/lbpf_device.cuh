@@ -266,13 +266,19 @@ __device__ __forceinline__ void aniso_2d(const Coef<N>& c, int fold, N gx, N gy,
   }
 }
 
+// y_first: |grad|^2 takes x's square rounded and adds y's exactly, else the other
+// way round.  An FP32 rounding apart, but with 16-bit storage it turns over a
+// stored value here and there, which spreads over the run; results keep to the
+// order that each part of a 16-bit grid has always had.
 template <typename N>
-__device__ __forceinline__ void aniso_3d(const Coef<N>& c, const N (&g)[3], N& as, N (&Nv)[3]) {
+__device__ __forceinline__ void aniso_3d(const Coef<N>& c, const N (&g)[3], bool y_first, N& as,
+                                         N (&Nv)[3]) {
   using S1 = typename Lanes<N>::S;
   as = splat<N>(S1(1));
 #pragma unroll
   for (int d = 0; d < 3; ++d) Nv[d] = splat<N>(S1(0));
-  const N g2 = fma_r(g[2], g[2], fma_r(g[0], g[0], mul_r(g[1], g[1])));
+  const N ga = y_first ? g[1] : g[0], gb = y_first ? g[0] : g[1];
+  const N g2 = fma_r(g[2], g[2], fma_r(ga, ga, mul_r(gb, gb)));
   if (!any_steep(g2) || lane(c.eps, 0) == S1(0)) return;
   // (n = 0 on a flat lane, so N = 0 there by itself)
   const N ig = where_steep(g2, rsqrt_r(g2), splat<N>(S1(0)));

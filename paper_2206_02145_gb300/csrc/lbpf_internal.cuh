@@ -78,8 +78,8 @@ struct Model {
   __half* uring;
   // Solid nodes (walls, obstacles): one byte per node at (z * ny + y) * px +
   // x, 1 = solid; null when there are none.  solid_tiles: in 2D one byte per
-  // 32 x 4 tile of the step (row-major over the tiles), in 3D one per column
-  // chunk of the z-marching step; 1 = the tile or chunk or its one-node halo
+  // 32 x 4 tile of the step (row-major over the tiles), in 3D one per 32 x 4 x 8
+  // block of nodes; 1 = the tile or block or its one-node halo
   // holds a solid node
   const unsigned char* solid;
   const unsigned char* solid_tiles;
@@ -266,7 +266,7 @@ cudaError_t launch_solid_sync(const Model& m, void* const pops[2], void* const r
 // (solid_tile_count(m) bytes).
 size_t solid_tile_count(const Model& m);
 cudaError_t launch_solid_tiles(const Model& m, unsigned char* flags, cudaStream_t s);
-// 3D: one flag per column chunk of the z-marching step
+// 3D: one flag per 32 x 4 x 8 block of nodes
 size_t solid_chunk_count(const Model& m);
 cudaError_t launch_solid_chunks(const Model& m, unsigned char* flags, cudaStream_t s);
 // Support values of the phi = 0 contour of a 2D state (phi from the h

@@ -1,44 +1,16 @@
 // Per-node part of the 3D coupled step, shared by the 3D step kernels:
 // D3Q19 flow f (Eqs. 4-12), D3Q7 solute g (Eqs. 13-18) and D3Q7 phase field
 // h (Eqs. 19-23, cubic anisotropy of Eq. 3), push streaming.  The caller has
-// the node's own population deviations in registers and phi + 1 and the h
-// deviations around the node (one node in x, y and z) in shared memory.
+// the node's own population deviations, phi + 1 and the h deviations around
+// the node (one node in x, y and z) in shared memory.  As in 2D every
+// operation is written with its rounding; a thread holds one node (two, on
+// the packed FP32 instructions, measured slower: 831 against 690 us per step of
+// 256^3 in FP16, the code of both paths no longer fits the instruction cache).
 #pragma once
 
 #include "lbpf_device.cuh"
 
 namespace lbk {
-
-// Shared-memory views of the node's neighbourhood, indexed by the plane
-// offset dz in {-1, 0, 1} from the node's plane and the local (ly, lx) of a
-// halo-extended tile.  PhiSlab3 / HSlab3: a contiguous [z][y][x] tile (plane
-// of the node at lz); PhiRing3 / HRing3: three separately stored planes.
-template <typename R, int ROW, int SLAB>
-struct PhiSlab3 {
-  const R* base;  // plane of the node
-  __device__ __forceinline__ R at(int dz, int ly, int lx) const {
-    return base[dz * SLAB + ly * ROW + lx];
-  }
-};
-template <typename R, int ROW, int SLAB, int PLANE>
-struct HSlab3 {
-  const R* base;  // direction 0, plane of the node
-  __device__ __forceinline__ R at(int a, int dz, int ly, int lx) const {
-    return base[a * PLANE + dz * SLAB + ly * ROW + lx];
-  }
-};
-template <typename R, int ROW>
-struct PhiRing3 {
-  const R* p[3];  // planes dz = -1, 0, 1
-  __device__ __forceinline__ R at(int dz, int ly, int lx) const { return p[dz + 1][ly * ROW + lx]; }
-};
-template <typename R, int ROW, int PLANE>
-struct HRing3 {
-  const R* p[3];  // planes dz = -1, 0, 1 (direction 0; direction a at + a * PLANE)
-  __device__ __forceinline__ R at(int a, int dz, int ly, int lx) const {
-    return p[dz + 1][a * PLANE + ly * ROW + lx];
-  }
-};
 
 // ---- central Hermite MRT of the D3Q19 flow lattice (Sec. 2.2 after Eq. 9) ----
 // The nineteen moments are the products H_i(X) H_j(Y) H_k(Z) (H_0 = 1,
@@ -189,23 +161,6 @@ __device__ __forceinline__ void chm_post_3d(const R (&d)[19], R drho, R rho, con
   }
 }
 
-// The per-node g reference around a node (3D, 16-bit storage), as UView of
-// the 2D step: `own` the reference of the node's own populations, at(dz, ly,
-// lx) the encoding reference of the node at plane offset dz and local (ly,
-// lx) (three halo-extended planes of row pitch ROW), `out` the plane that
-// receives each node's new U.  REL = false: every member unused.
-template <bool REL, int ROW>
-struct UView3 {
-  static constexpr bool kRel = REL;
-  const __half* p[3];
-  __half* out;
-  float own;
-  __device__ __forceinline__ float at(int dz, int ly, int lx) const {
-    return REL ? __half2float(p[dz + 1][ly * ROW + lx]) : 0.f;
-  }
-};
-using NoUView3 = UView3<false, 1>;
-
 // Solid nodes (3D mask): is the node at (x, y, z), mapped like a gradient
 // neighbour (periodic wrap, else nearest node), solid?
 __device__ __forceinline__ bool solid_mapped3(const Model& m, int x, int y, int z) {
@@ -215,222 +170,347 @@ __device__ __forceinline__ bool solid_mapped3(const Model& m, int x, int y, int 
   return m.solid[(size_t(z) * m.ny + y) * m.px + x] != 0;
 }
 
-// pv: phi + 1 around the node, hv: the h deviations around it (views above).
-// INTERIOR: every node of the tile is at least one node away from every
-// domain face, so every destination is an ordinary node.  CHM: the flow
-// collides by the central Hermite MRT.  MASK: the code for solid nodes is
-// compiled in; `solids` (the tile or column chunk holds or borders a solid
-// node) switches it on: a solid gradient neighbour counts as the first fluid
-// node among the single-axis steps of its direction (x, y, z order) and the
-// node itself, and a push towards a solid node comes back reversed.
-template <typename T, typename R, bool FLOW, bool INTERIOR, bool CHM, bool MASK = false,
-          typename PV, typename HV, typename UV = NoUView3>
-__device__ __forceinline__ void collide_push_3d(const Model& m, int x, int y, int z, int lx,
-                                                int ly, const R (&f)[19], const R (&g)[7],
-                                                const R (&h)[7], R dphi, R dphi_prev,
-                                                const PV& pv, const HV& hs,
-                                                T* __restrict__ dst, R* __restrict__ ring_cur,
-                                                unsigned* __restrict__ err,
-                                                bool solids = false, const UV& uh = UV()) {
-  constexpr int QF = FLOW ? 19 : 0;
-  const int nx = m.nx, ny = m.ny, nz = m.nz, px = m.px;
-  const int P = int(m.plane);  // fits: checked at creation
-  const int slab = ny * px;
-  const int idx = z * slab + y * px + x;
-  T* const pd = dst + idx;
-  const Coef<R>& c = coef<R>(m);
+// What the collisions need, so that each direction costs a few FMAs (see the
+// 2D core; D3Q7 has c_s^2 = 1/4).
+template <typename N>
+struct Node3D {
+  N U;
+  N us[3], F[3], E0, E1, E2, G0;
+  N keep_U, K0, K1, keep_phi, H0, H[3], inv_a2, keep_old;
+};
 
+// Moments, gradient, anisotropy and coefficients of a node; pn: the eighteen
+// neighbours' phi + 1.  False if phi, U or rho is not finite.
+template <typename N, bool FLOW, bool CHM>
+__device__ __forceinline__ bool node_3d(const Coef<N>& c, const N (&f)[19], const N (&g)[7], N dphi,
+                                        N dphi_prev, N Rg, const N (&pn)[19], bool y_first,
+                                        Node3D<N>& o,
+                                        N (&fchm)[19]) {
+  using S = typename Lanes<N>::S;
+  const N one = splat<N>(S(1)), half = splat<N>(S(0.5));
   // ---- local moments (Eqs. 11, 12, 17, 22) ----------------------------------
-  const R phi = dphi - R(1);
-  R dU = R(0);
+  const N phi = sub_r(dphi, one);
+  N dU = g[0];
 #pragma unroll
-  for (int a = 0; a < 7; ++a) dU += g[a];
+  for (int a = 1; a < 7; ++a) dU = add_r(dU, g[a]);
   // g deviations are taken from w_a Rg; the collision (Eqs. 13-16) is linear
   // in them, so any per-node Rg gives the same populations
-  const R Rg = UV::kRel ? R(uh.own) : c.ref_g;
-  const R U = Rg + dU;
-  R drho = R(0), mo[3] = {R(0), R(0), R(0)};
+  const N U = o.U = add_r(Rg, dU);
+  N drho = splat<N>(S(0)), mo[3] = {drho, drho, drho};
   if (FLOW) {
+    drho = f[0];
+    mo[0] = f[1];
+    mo[1] = f[3];
+    mo[2] = f[5];
 #pragma unroll
-    for (int a = 0; a < 19; ++a) {
-      drho += f[a];
-      if (D3_CX[a]) mo[0] += R(D3_CX[a]) * f[a];
-      if (D3_CY[a]) mo[1] += R(D3_CY[a]) * f[a];
-      if (D3_CZ[a]) mo[2] += R(D3_CZ[a]) * f[a];
+    for (int a = 1; a < 19; ++a) {
+      drho = add_r(drho, f[a]);
+      const int cv[3] = {D3_CX[a], D3_CY[a], D3_CZ[a]};
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        if (cv[d] == 0 || a == 1 + 2 * d) continue;
+        mo[d] = cv[d] > 0 ? add_r(mo[d], f[a]) : sub_r(mo[d], f[a]);
+      }
     }
   }
-  const R rho = R(1) + drho;
-  const R ph = clamp1(phi);
-  const R mask = R(0.5) * (R(1) - ph);  // (1 - phi)/2 of Eq. 7 and q(phi) of Eq. 18
-  R u[3] = {R(0), R(0), R(0)}, F[3] = {R(0), R(0), R(0)};
+  const N rho = add_r(one, drho);
+  const bool ok = all_finite(phi, U, rho);
+  const N ph = clamp1(phi);
+  const N mask = mul_r(half, sub_r(one, ph));  // (1 - phi)/2 of Eq. 7 and q(phi) of Eq. 18
+#pragma unroll
+  for (int d = 0; d < 3; ++d) o.us[d] = o.F[d] = splat<N>(S(0));
   if (FLOW) {
-    const R K = c.kdrag * (R(1) + ph) * (R(1) + ph) * (R(1) - ph);  // Eq. 6
-    const R inv = rcp_r(rho + R(0.5) * K);
+    const N ph1 = add_r(one, ph);
+    const N K = mul_r(mul_r(mul_r(c.kdrag, ph1), ph1), sub_r(one, ph));  // Eq. 6
+    const N inv = rcp_r(fma_r(half, K, rho));
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      u[d] = (mo[d] + R(0.5) * c.body[d]) * inv;
-      F[d] = c.body[d] - K * u[d];
+      const N u = mul_r(fma_r(half, c.body[d], mo[d]), inv);
+      o.F[d] = fma_r(neg_r(K), u, c.body[d]);
+      o.us[d] = mul_r(mask, u);  // Eq. 7
     }
   }
-  const R us[3] = {mask * u[0], mask * u[1], mask * u[2]};  // Eq. 7
-  R fchm[19];
-  if (FLOW && CHM) chm_post_3d<R>(f, drho, rho, mo, us, F, c.omega_f, c.chm_wb, c.chm_wh, fchm);
-  const R omega_U = rcp_r(R(0.5) + c.tauU_slope * mask);  // Eq. 18
-  const R dphidt = dphi - dphi_prev;
-  ring_cur[idx] = dphi;
-  if (UV::kRel) uh.out[idx] = __float2half_rn(float(U));
-  if (!(finite_r(phi) && finite_r(U) && finite_r(rho))) atomicOr(err, 1u);
-  // a g deviation pushed to the node at (dz, dly, dlx), taken from its
-  // reference there instead of this node's
-  auto genc = [&](R v, R w, int dz, int dly, int dlx) -> R {
-    return UV::kRel ? fma_r(-w, R(uh.at(dz, dly, dlx)) - Rg, v) : v;
-  };
+  if constexpr (FLOW && CHM) {
+#pragma unroll
+    for (int k = 0; k < Lanes<N>::V; ++k) {
+      S d[19], post[19], m3[3], v3[3], F3[3];
+#pragma unroll
+      for (int a = 0; a < 19; ++a) d[a] = lane(f[a], k);
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        m3[e] = lane(mo[e], k);
+        v3[e] = lane(o.us[e], k);
+        F3[e] = lane(o.F[e], k);
+      }
+      chm_post_3d<S>(d, lane(drho, k), lane(rho, k), m3, v3, F3, lane(c.omega_f, 0),
+                     lane(c.chm_wb, 0), lane(c.chm_wh, 0), post);
+#pragma unroll
+      for (int a = 0; a < 19; ++a) set_lane(fchm[a], k, post[a]);
+    }
+  }
+  const N omega_U = rcp_r(fma_r(c.tauU_slope, mask, half));  // Eq. 18
+  const N dphidt = sub_r(dphi, dphi_prev);
 
   // ---- grad = 3 sum_a w_a c_a phi(x + c_a) over D3Q19 ---------------------------
-  R gr[3] = {R(0), R(0), R(0)};
+  N gr[3];
 #pragma unroll
-  for (int a = 1; a < 19; ++a) {
-    const int gcx = D3_CX[a], gcy = D3_CY[a], gcz = D3_CZ[a];
-    R pn = pv.at(gcz, ly + gcy, lx + gcx);
-    if (MASK && !INTERIOR && solids && solid_mapped3(m, x + gcx, y + gcy, z + gcz)) {
-      if (gcx != 0 && !solid_mapped3(m, x + gcx, y, z)) pn = pv.at(0, ly, lx + gcx);
-      else if (gcy != 0 && !solid_mapped3(m, x, y + gcy, z)) pn = pv.at(0, ly + gcy, lx);
-      else if (gcz != 0 && !solid_mapped3(m, x, y, z + gcz)) pn = pv.at(gcz, ly, lx);
-      else pn = pv.at(0, ly, lx);
+  for (int d = 0; d < 3; ++d) gr[d] = mul_r(pn[1 + 2 * d], splat<N>(S(1.0 / 6.0)));
+#pragma unroll
+  for (int a = 2; a < 19; ++a) {
+    const N w = splat<N>(a < 7 ? S(1.0 / 6.0) : S(1.0 / 12.0));
+    const int cv[3] = {D3_CX[a], D3_CY[a], D3_CZ[a]};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      if (cv[d] == 0 || a == 1 + 2 * d) continue;
+      gr[d] = fma_r(cv[d] > 0 ? pn[a] : neg_r(pn[a]), w, gr[d]);
     }
-    const R v = pn * (a < 7 ? R(1.0 / 6.0) : R(1.0 / 12.0));
-    if (D3_CX[a]) gr[0] += R(D3_CX[a]) * v;
-    if (D3_CY[a]) gr[1] += R(D3_CY[a]) * v;
-    if (D3_CZ[a]) gr[2] += R(D3_CZ[a]) * v;
   }
-  R as, N[3];
-  aniso_3d<R>(c, gr, as, N);
-  const R a2 = as * as;
-  const R inv_a2 = rcp_r(a2);
-  const R omega_phi = rcp_r(a2 * c.tpc + R(0.5));  // Eq. 23
-  const R phi2m = R(1) - phi * phi;
-  const R Qs = (phi - phi * phi * phi + c.lambda * U * phi2m * phi2m) * c.inv_tau0;  // Eq. 20
-
-  // node constants of the collisions (see the 2D core); D3Q7 has c_s^2 = 1/4
-  const R uu = us[0] * us[0] + us[1] * us[1] + us[2] * us[2];
-  const R uF = us[0] * F[0] + us[1] * F[1] + us[2] * F[2];
-  const R omega_f = c.omega_f, keep_f = R(1) - c.omega_f, guo = c.guo;
-  const R E0 = omega_f * (drho - R(1.5) * rho * uu);
-  const R E1 = omega_f * R(3) * rho, E2 = omega_f * R(4.5) * rho;
-  const R G0 = -R(3) * uF;
-  const R keep_U = R(1) - omega_U;
-  const R K0 = omega_U * dU - dphidt, K1 = R(4) * omega_U * U;
-  const R keep_phi = R(1) - omega_phi;
-  const R H0 = omega_phi * dphi + Qs;
-  const R Hx = omega_phi * c.tpc * N[0], Hy = omega_phi * c.tpc * N[1],
-          Hz = omega_phi * c.tpc * N[2];
-  const R keep_old = R(1) - inv_a2;  // Eq. 19: h_new = h* / a_s^2 + (1 - 1/a_s^2) h_old
-  const int bcx = m.bc[0], bcy = m.bc[1], bcz = m.bc[2];
-
+  N as, Nv[3];
+  aniso_3d<N>(c, gr, y_first, as, Nv);
+  const N a2 = mul_r(as, as);
+  o.inv_a2 = rcp_r(a2);
+  const N omega_phi = rcp_r(fma_r(a2, c.tpc, half));  // Eq. 23
+  const N pp = mul_r(phi, phi);
+  const N phi2m = sub_r(one, pp);
+  // Eq. 20
+  const N Qs = mul_r(fma_r(mul_r(mul_r(c.lambda, U), phi2m), phi2m, fma_r(neg_r(pp), phi, phi)),
+                     c.inv_tau0);
+  if (FLOW && !CHM) {
+    const N uu = fma_r(o.us[2], o.us[2], fma_r(o.us[0], o.us[0], mul_r(o.us[1], o.us[1])));
+    const N uF = fma_r(o.us[2], o.F[2], fma_r(o.us[0], o.F[0], mul_r(o.us[1], o.F[1])));
+    o.E0 = mul_r(c.omega_f, fma_r(neg_r(mul_r(splat<N>(S(1.5)), rho)), uu, drho));
+    o.E1 = mul_r(c.wf3, rho);
+    o.E2 = mul_r(c.wf45, rho);
+    o.G0 = mul_r(splat<N>(S(-3)), uF);
+  }
+  o.keep_U = sub_r(one, omega_U);
+  o.K0 = fma_r(omega_U, dU, neg_r(dphidt));
+  o.K1 = mul_r(mul_r(splat<N>(S(4)), omega_U), U);
+  o.keep_phi = sub_r(one, omega_phi);
+  o.H0 = fma_r(omega_phi, dphi, Qs);
+  const N wt = mul_r(omega_phi, c.tpc);
 #pragma unroll
-  for (int a = 0; a < 19; ++a) {
-    if (!FLOW && a >= 7) break;
-    const int cx = D3_CX[a], cy = D3_CY[a], cz = D3_CZ[a];
-    const R cu = R(cx) * us[0] + R(cy) * us[1] + R(cz) * us[2];
-    const bool sc = a < 7;  // also a direction of the D3Q7 lattices
-    R fp = R(0), gp = R(0), hp = R(0);
-    if (FLOW) {
-      const R wf = d3q19_w<R>(a);
-      const R cF = R(cx) * F[0] + R(cy) * F[1] + R(cz) * F[2];
-      const R feq = fma_r(cu, fma_r(E2, cu, E1), E0);
-      const R guo_t = mul_r(guo, fma_r(cF, fma_r(R(9), cu, R(3)), G0));
-      fp = CHM ? fchm[a] : fma_r(keep_f, f[a], mul_r(wf, add_r(feq, guo_t)));
+  for (int d = 0; d < 3; ++d) o.H[d] = mul_r(wt, Nv[d]);
+  // Eq. 19: h_new = h* / a_s^2 + (1 - 1/a_s^2) h_old
+  o.keep_old = sub_r(one, o.inv_a2);
+  return ok;
+}
+
+// c_a . v (a a constant after unrolling; not the rest direction)
+template <typename N>
+__device__ __forceinline__ N dir_dot3(int a, const N (&v)[3]) {
+  const int cv[3] = {D3_CX[a], D3_CY[a], D3_CZ[a]};
+  N r = v[0];
+  bool first = true;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    if (cv[d] == 0) continue;
+    const N t = cv[d] > 0 ? v[d] : neg_r(v[d]);
+    r = first ? t : add_r(r, t);
+    first = false;
+  }
+  return r;
+}
+
+// Post-collision deviations of direction a at the node: f* (Eq. 4), g* (Eq.
+// 13) and, before Eq. 19's division by a_s^2, h*.
+template <typename N>
+__device__ __forceinline__ N post_f_3d(const Coef<N>& c, const Node3D<N>& n, int a, N f) {
+  using S = typename Lanes<N>::S;
+  N feq = n.E0, gt = n.G0;
+  if (a > 0) {
+    const N cu = dir_dot3(a, n.us), cF = dir_dot3(a, n.F);
+    feq = fma_r(cu, fma_r(n.E2, cu, n.E1), n.E0);
+    gt = fma_r(cF, fma_r(splat<N>(S(9)), cu, splat<N>(S(3))), n.G0);
+  }
+  return fma_r(c.keep_f, f,
+               mul_r(splat<N>(d3q19_w<S>(a)), add_r(feq, prod_r(c.guo, gt, c.mzero))));
+}
+template <typename N>
+__device__ __forceinline__ N post_g_3d(const Node3D<N>& n, int a, N g) {
+  using S = typename Lanes<N>::S;
+  N e = n.K0;
+  if (a > 0) e = fma_r(n.K1, dir_dot3(a, n.us), n.K0);
+  return fma_r(n.keep_U, g, mul_r(splat<N>(d3q7_w<S>(a)), e));
+}
+template <typename N>
+__device__ __forceinline__ N post_h_3d(const Node3D<N>& n, int a, N h) {
+  using S = typename Lanes<N>::S;
+  N e = n.H0;
+  if (a > 0) e = sub_r(n.H0, dir_dot3(a, n.H));
+  return fma_r(n.keep_phi, h, mul_r(splat<N>(d3q7_w<S>(a)), e));
+}
+// Eq. 19 at the destination, whose old value is hold
+template <typename N>
+__device__ __forceinline__ N arrive_h_3d(const Node3D<N>& n, N hp, N hold) {
+  return fma_r(n.inv_a2, hp, mul_r(n.keep_old, hold));
+}
+
+// the D3Q19 directions (bit a) whose component d is v
+constexpr unsigned dirs3(int d, int v) {
+  unsigned m = 0;
+  for (int a = 0; a < 19; ++a)
+    if ((d == 0 ? D3_CX[a] : (d == 1 ? D3_CY[a] : D3_CZ[a])) == v) m |= 1u << a;
+  return m;
+}
+
+// What the 3D step needs of a grid besides the model constants.
+struct Grid3D {
+  int nx, ny, nz, px, slab, bc[3];
+  long long plane;
+  __device__ __forceinline__ explicit Grid3D(const Model& m)
+      : nx(m.nx), ny(m.ny), nz(m.nz), px(m.px), slab(m.ny * m.px),
+        bc{m.bc[0], m.bc[1], m.bc[2]}, plane(m.plane) {}
+};
+
+// Collide the node (x, y, z) and push its populations.
+//   own(q): stored deviation q of the node (f, then g); h: its own h
+//   dphi, dphi_prev: phi + 1 now and one step earlier
+//   phi(dz, dy, dx), hold(a, dz, dy, dx), uref(dz, dy, dx): phi + 1, h_a and the
+//     encoding reference of g (UREL) at that offset from the node
+//   sm: bit a set where the D3Q19 neighbour a (0: the node itself) is solid (MASK)
+//   tb: the tile's first node in its plane in array 0 of the destination
+//     buffer (the same for the whole CTA, so that every array's address is one
+//     uniform base plus the thread's offset); o0: the node's byte offset from it
+//   y_first: as of aniso_3d
+// EDGE = false: interior nodes with no solid node near: all neighbours at fixed
+// offsets, no tests.  EDGE = true: any node; one outside the domain (of a partial
+// column) or solid pushes nothing.  Which populations go where is then a few
+// bit masks over the directions: 25 % of the warps of a 256^3 grid touch a
+// boundary in x (871 us per step against 891 with a test per direction).
+template <typename T, typename R, bool FLOW, bool CHM, bool MASK, bool EDGE, bool UREL,
+          typename Own, typename Phi, typename Hold, typename Uref>
+__device__ __forceinline__ void collide_push_3d(
+    const Grid3D& gr, const Coef<R>& c, int x, int y, int z, const Own& own, const R (&h)[7],
+    R dphi, R dphi_prev, const Phi& phi, const Hold& hold, const Uref& uref, unsigned sm, R Rg,
+    T* __restrict__ tb, unsigned o0, bool y_first, unsigned* __restrict__ err, R& Unew) {
+  constexpr int QF = FLOW ? 19 : 0;
+  const long long P = gr.plane;
+  const int px = gr.px, slab = gr.slab;
+  R pn[19];  // the neighbours' phi + 1
+#pragma unroll
+  for (int a = 1; a < 19; ++a) pn[a] = phi(D3_CZ[a], D3_CY[a], D3_CX[a]);
+  if (MASK && EDGE && sm != 0) {
+    // a solid neighbour counts as the first fluid node among the single-axis
+    // steps of its direction (x, y, z order) and the node itself: zero normal
+    // derivative at walls and obstacles
+    auto is = [&](int a) { return (sm >> a & 1u) != 0; };
+#pragma unroll
+    for (int a = 18; a > 0; --a) {  // the axis values last: the others look at them
+      if (!is(a)) continue;
+      R v = dphi;
+      if (a > 6) {
+        const int ax = D3_CX[a] > 0 ? 1 : 2, ay = D3_CY[a] > 0 ? 3 : 4, az = D3_CZ[a] > 0 ? 5 : 6;
+        if (D3_CX[a] != 0 && !is(ax)) v = pn[ax];
+        else if (D3_CY[a] != 0 && !is(ay)) v = pn[ay];
+        else if (D3_CZ[a] != 0 && !is(az)) v = pn[az];
+      }
+      pn[a] = v;
     }
-    if (sc) {
-      const R ws = d3q7_w<R>(a);
-      gp = fma_r(keep_U, g[a], mul_r(ws, fma_r(K1, cu, K0)));
-      hp = fma_r(keep_phi, h[a],
-                 mul_r(ws, add_r(H0, -add_r(add_r(R(cx) * Hx, R(cy) * Hy), R(cz) * Hz))));
-    }
-    if (INTERIOR) {
+  }
+  R f[19], g[7];
+  if (FLOW) {
+#pragma unroll
+    for (int a = 0; a < 19; ++a) f[a] = own(a);
+  }
+#pragma unroll
+  for (int a = 0; a < 7; ++a) g[a] = own(QF + a);
+  Node3D<R> nd;
+  R fchm[19];
+  if (!node_3d<R, FLOW, CHM>(c, f, g, dphi, dphi_prev, Rg, pn, y_first, nd, fchm)) atomicOr(err, 1u);
+  Unew = nd.U;
+
+  if constexpr (!EDGE) {
+    auto put = [&](int q, int off, R v) {
+      Pop<T>::st(reinterpret_cast<T*>(reinterpret_cast<char*>(tb + (q * P + off)) + o0), v);
+    };
+#pragma unroll
+    for (int a = 0; a < 19; ++a) {
+      if (!FLOW && a >= 7) break;
+      const int cx = D3_CX[a], cy = D3_CY[a], cz = D3_CZ[a];
       const int off = cz * slab + cy * px + cx;
-      if (FLOW) Pop<T>::st(pd + (a * P + off), fp);
-      if (sc) {
-        const R hold = hs.at(a, cz, ly + cy, lx + cx);
-        Pop<T>::st(pd + ((QF + a) * P + off), genc(gp, d3q7_w<R>(a), cz, ly + cy, lx + cx));
-        Pop<T>::st(pd + ((QF + 7 + a) * P + off), fma_r(inv_a2, hp, mul_r(keep_old, hold)));  // Eq. 19
-      }
-      continue;
-    }
-    int xd = x + cx, yd = y + cy, zd = z + cz;
-    bool bounce = false, drop = false;
-    if (yd < 0 || yd >= ny) {
-      if (bcy == BC_PERIODIC) yd = wrap1(yd, ny);
-      else bounce = true;
-    }
-    if (zd < 0 || zd >= nz) {
-      if (bcz == BC_PERIODIC) zd = wrap1(zd, nz);
-      else bounce = true;
-    }
-    if (xd < 0 || xd >= nx) {
-      if (bcx == BC_PERIODIC) xd = wrap1(xd, nx);
-      else if (bcx == BC_WALL) bounce = true;
-      else drop = true;
-    }
-    if (MASK && solids && !bounce && !drop && m.solid[zd * slab + yd * px + xd])
-      bounce = true;  // obstacle
-    if (bounce) {
-      // half-way bounce-back: comes back to this node reversed
-      const int b = D3_OPP[a];
-      if (FLOW) Pop<T>::st(dst + (b * P + idx), fp);
-      if (sc) {
-        Pop<T>::st(dst + ((QF + b) * P + idx), genc(gp, d3q7_w<R>(a), 0, ly, lx));
-        Pop<T>::st(dst + ((QF + 7 + b) * P + idx), fma_r(inv_a2, hp, mul_r(keep_old, h[b])));
-      }
-    } else if (!drop) {
-      const int jd = zd * slab + yd * px + xd;
-      if (FLOW) Pop<T>::st(dst + (a * P + jd), fp);
-      if (sc) {
-        const R hold = hs.at(a, cz, ly + cy, lx + cx);
-        Pop<T>::st(dst + ((QF + a) * P + jd), genc(gp, d3q7_w<R>(a), cz, ly + cy, lx + cx));
-        Pop<T>::st(dst + ((QF + 7 + a) * P + jd), fma_r(inv_a2, hp, mul_r(keep_old, hold)));  // Eq. 19
+      if (FLOW) put(a, off, CHM ? fchm[a] : post_f_3d<R>(c, nd, a, f[a]));
+      if (a < 7) {
+        R gp = post_g_3d<R>(nd, a, g[a]);
+        if (UREL) gp = fma_r(-d3q7_w<R>(a), sub_r(uref(cz, cy, cx), Rg), gp);
+        put(QF + a, off, gp);
+        put(QF + 7 + a, off, arrive_h_3d<R>(nd, post_h_3d<R>(nd, a, h[a]), hold(a, cz, cy, cx)));
       }
     }
-    if (bcx == BC_INOUT) {
-      if (cx == -1 && x == nx - 1) {
-        // outflow ghost x = nx repeats this column
-        int yo = y + cy, zo = z + cz;
-        bool ok = true;
-        if (yo < 0 || yo >= ny) {
-          if (bcy == BC_PERIODIC) yo = wrap1(yo, ny);
-          else ok = false;
+  } else {
+    // Element steps to the neighbouring columns, rows and planes (across a
+    // periodic edge to the far side), and the directions (bit a) in which the
+    // node's push meets a wall or solid node (the population comes back to it
+    // reversed, half-way bounce-back) or, in x, the inflow or outflow ghost
+    // (nothing to push); those whose outflow repeats at the last column and
+    // those that arrive from the inflow ghost.
+    constexpr unsigned XM = dirs3(0, -1), XP = dirs3(0, 1), YM = dirs3(1, -1), YP = dirs3(1, 1),
+                       ZM = dirs3(2, -1), ZP = dirs3(2, 1);
+    const int nx = gr.nx, ny = gr.ny, nz = gr.nz;
+    const bool x_lo = x == 0, x_hi = x == nx - 1, y_lo = y == 0, y_hi = y == ny - 1;
+    const bool z_lo = z == 0, z_hi = z == nz - 1;
+    const int sx[3] = {x_lo ? nx - 1 : -1, 0, x_hi ? 1 - nx : 1};
+    const int sy[3] = {y_lo ? (ny - 1) * px : -px, 0, y_hi ? -(ny - 1) * px : px};
+    const int sz[3] = {z_lo ? (nz - 1) * slab : -slab, 0, z_hi ? -(nz - 1) * slab : slab};
+    const bool io = gr.bc[0] == BC_INOUT, wy = gr.bc[1] == BC_WALL, wz = gr.bc[2] == BC_WALL;
+    const unsigned x_out = (x_lo ? XM : 0u) | (x_hi ? XP : 0u);
+    const unsigned wall = (wy && y_lo ? YM : 0u) | (wy && y_hi ? YP : 0u) |
+                          (wz && z_lo ? ZM : 0u) | (wz && z_hi ? ZP : 0u);
+    const unsigned behind = (wy && y_lo ? YP : 0u) | (wy && y_hi ? YM : 0u) |
+                            (wz && z_lo ? ZP : 0u) | (wz && z_hi ? ZM : 0u);
+    unsigned back = wall | (gr.bc[0] == BC_WALL ? x_out : 0u);
+    const unsigned ghost = io ? x_out & ~back : 0u;
+    if (MASK) back |= sm & ~ghost;  // obstacles
+    unsigned go = ~(back | ghost);
+    unsigned outf = io && x_hi ? XM & ~wall : 0u;
+    unsigned inf = io && x_lo ? XP & ~behind : 0u;
+    if (!(x < nx && y < ny) || (MASK && (sm & 1u))) go = back = outf = inf = 0u;
+    const unsigned odd = back | outf | inf;
+    T* const node = reinterpret_cast<T*>(reinterpret_cast<char*>(tb) + o0);
+#pragma unroll
+    for (int a = 0; a < 19; ++a) {
+      if (!FLOW && a >= 7) break;
+      const int cx = D3_CX[a], cy = D3_CY[a], cz = D3_CZ[a], b = D3_OPP[a];
+      const bool sc = a < 7;  // also a direction of the D3Q7 lattices
+      R fp = R(0), gp = R(0), hp = R(0), hd = R(0), gd = R(0);
+      if (FLOW) fp = CHM ? fchm[a] : post_f_3d<R>(c, nd, a, f[a]);
+      const R w = sc ? d3q7_w<R>(a) : R(0);
+      if (sc) {
+        gp = post_g_3d<R>(nd, a, g[a]);
+        hp = post_h_3d<R>(nd, a, h[a]);
+        hd = arrive_h_3d<R>(nd, hp, hold(a, cz, cy, cx));
+        gd = UREL ? fma_r(-w, sub_r(uref(cz, cy, cx), Rg), gp) : gp;
+      }
+      auto store = [&](T* p, R fv, R gv, R hv) {
+        if (FLOW) Pop<T>::st(p, fv);
+        if (sc) {
+          Pop<T>::st(p + QF * P, gv);
+          Pop<T>::st(p + (QF + 7) * P, hv);
         }
-        if (zo < 0 || zo >= nz) {
-          if (bcz == BC_PERIODIC) zo = wrap1(zo, nz);
-          else ok = false;
+      };
+      if (go >> a & 1u) store(node + (a * P + sx[cx + 1] + sy[cy + 1] + sz[cz + 1]), fp, gd, hd);
+      if (a > 0 && (odd >> a & 1u)) {
+        if (sc) {  // reversed at the node
+          hd = arrive_h_3d<R>(nd, hp, h[b < 7 ? b : 0]);
+          if (UREL) gd = fma_r(-w, sub_r(uref(0, 0, 0), Rg), gp);
         }
-        if (ok) {
-          const int jo = zo * slab + yo * px + x;
-          if (FLOW) Pop<T>::st(dst + (a * P + jo), fp);
+        if (back >> a & 1u) store(node + b * P, fp, gd, hd);
+        if (cx < 0) {
+          // outflow ghost x = nx repeats this column
           if (sc) {
-            const R hold = hs.at(a, cz, ly + cy, lx);
-            Pop<T>::st(dst + ((QF + a) * P + jo), genc(gp, d3q7_w<R>(a), cz, ly + cy, lx));
-            Pop<T>::st(dst + ((QF + 7 + a) * P + jo), fma_r(inv_a2, hp, mul_r(keep_old, hold)));
+            hd = arrive_h_3d<R>(nd, hp, hold(a, cz, cy, 0));
+            if (UREL) gd = fma_r(-w, sub_r(uref(cz, cy, 0), Rg), gp);
           }
+          if (outf >> a & 1u) store(node + (a * P + sy[cy + 1] + sz[cz + 1]), fp, gd, hd);
         }
-      }
-      if (cx == 1 && x == 0) {
-        // inflow ghost x = -1 (equilibrium, phi = -1), unless behind a wall
-        const int ys = y - cy, zs = z - cz;
-        const bool behind_wall = ((ys < 0 || ys >= ny) && bcy == BC_WALL) ||
-                                 ((zs < 0 || zs >= nz) && bcz == BC_WALL);
-        if (!behind_wall) {
-          const R uin = c.u_in, cui = uin;
-          if (FLOW)
-            Pop<T>::st(dst + (a * P + idx),
-                       d3q19_w<R>(a) * (R(3) * cui + R(4.5) * cui * cui - R(1.5) * uin * uin));
-          if (sc) {
-            const R ws = d3q7_w<R>(a);
-            const R gu = FLOW ? cui : R(0);
-            Pop<T>::st(dst + ((QF + a) * P + idx),
-                       genc(ws * ((c.U_in - Rg) + c.U_in * R(4) * gu), ws, 0, ly, lx));
-            Pop<T>::st(dst + ((QF + 7 + a) * P + idx), R(0));  // phi = -1: zero deviation
-          }
+        if (cx > 0 && (inf >> a & 1u)) {
+          // inflow ghost x = -1 (equilibrium, phi = -1: zero h deviation), unless
+          // behind a wall
+          const R uin = c.u_in, Uin = c.U_in, gu = FLOW ? uin : R(0);
+          const R fin = d3q19_w<R>(a) * (R(3) * uin + R(4.5) * uin * uin - R(1.5) * uin * uin);
+          R gin = w * ((Uin - Rg) + Uin * R(4) * gu);
+          if (UREL) gin = fma_r(-w, uref(0, 0, 0) - Rg, gin);
+          store(node + a * P, fin, gin, R(0));
         }
       }
     }

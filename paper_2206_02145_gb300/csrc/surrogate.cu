@@ -228,6 +228,8 @@ int conv_bwd(lbpf_unet* n, const ConvLayer& l, const Act& x, int xoff, const Act
   wa.chunk = kWgradChunk;
   wa.part = n->wpart;
   wa.part_cap = n->wpart_cap;
+  wa.tensor_path = n->tensor_path;
+  wa.err = n->d_err;
   UCK(n, lbk::nn::wgrad3x3(wa, n->stream));  // weight and bias gradients
   if (gx) {
     lbk::nn::ConvArgs a{};

@@ -1,0 +1,93 @@
+// The 5th-generation tensor core instructions of the network's kernels
+// (tcgen05: matrix descriptors, products, tensor memory), one CTA per product.
+#pragma once
+
+#include <cuda.h>
+
+#include <cstdint>
+
+#include "tma.cuh"
+
+namespace lbk {
+namespace nn {
+
+constexpr int kTcSpin = 1 << 22;  // polls per barrier wait
+
+// swizzle of operand rows of n bf16 (one span per row): 128, 64 or 32 bytes
+inline CUtensorMapSwizzle swizzle_for(int n) {
+  return n == 64 ? CU_TENSOR_MAP_SWIZZLE_128B
+                 : (n == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+}
+
+// Shared-memory matrix descriptor of a K-major operand tile whose rows are
+// exactly one swizzle span long (BK bf16), 8-row core groups SBO bytes apart.
+__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t sbo, uint32_t mode) {
+  uint64_t d = 0;
+  d |= uint64_t((saddr & 0x3FFFFu) >> 4);           // start address
+  d |= uint64_t(1) << 16;                           // leading offset (unused: one span per row)
+  d |= uint64_t((sbo >> 4) & 0x3FFFu) << 32;        // stride between 8-row groups
+  d |= uint64_t(1) << 46;                           // descriptor version
+  d |= uint64_t(mode) << 61;                        // swizzle mode
+  return d;
+}
+
+// The same with the matrix starting `row` rows (of one swizzle span, rb
+// bytes) into a 1024-byte aligned swizzled buffer.  The swizzle phase follows
+// the absolute shared-memory address (as the TMA wrote it), so the start may
+// sit at any row with the base-offset field left at 0 (measured: setting it
+// to the row's phase, or starting at the aligned group with that phase,
+// gives wrong products).
+__device__ __forceinline__ uint64_t umma_desc_row(uint32_t saddr_aligned, int row, uint32_t rb,
+                                                  uint32_t sbo, uint32_t mode) {
+  return umma_desc(saddr_aligned + uint32_t(row) * rb, sbo, mode);
+}
+
+__device__ __forceinline__ void tc_fence_before() {
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+}
+__device__ __forceinline__ void tc_fence_after() {
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_alloc(uint32_t* holder, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                   smem_addr(holder)),
+               "r"(ncols)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
+               : "memory");
+}
+__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
+                                       uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// arrives on `bar` once every tcgen05 operation this thread issued so far is done
+__device__ __forceinline__ void tc_commit(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+          smem_addr(bar))
+      : "memory");
+}
+// 32 consecutive FP32 columns of this thread's tensor-memory lane
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
+        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
+        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+}  // namespace nn
+}  // namespace lbk

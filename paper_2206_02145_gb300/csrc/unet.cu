@@ -9,6 +9,8 @@
 //   element-wise     bias gradient, ReLU masks, 2x2 average pooling and its
 //                    gradient, nearest 2x upsampling and its gradient, the 1x1
 //                    head, MSE loss, Adam, weight transposition, input packing
+#include <algorithm>
+
 #include "lbpf_internal.cuh"
 #include "unet.cuh"
 #include "unet_ops.cuh"
@@ -800,13 +802,20 @@ size_t taps_bias_floats(const TapsShape& t) {
 
 size_t wgrad_scratch(int Cout, int Cin, int N, int H, int W, int chunk) {
   TapsShape t;
-  if (taps_shape(Cout, Cin, N, H, W, &t)) return taps_weight_floats(t) + taps_bias_floats(t);
+  const size_t tc = wgrad_tc_scratch(Cout, Cin, N, H, W);
+  if (taps_shape(Cout, Cin, N, H, W, &t))
+    return std::max(tc, taps_weight_floats(t) + taps_bias_floats(t));
   const long long npix = (long long)N * H * W;
   const int c = pertap_chunk(npix, chunk);
-  return size_t((npix + c - 1) / c) * 9 * Cout * Cin + bias_grad_scratch(Cout, npix);
+  return std::max(tc, size_t((npix + c - 1) / c) * 9 * Cout * Cin + bias_grad_scratch(Cout, npix));
 }
 
 cudaError_t wgrad3x3(const WgradArgs& args, cudaStream_t s) {
+  if (args.tensor_path) {
+    bool used = false;
+    const cudaError_t e = wgrad_tc(args, &used, s);
+    if (used || e != cudaSuccess) return e;
+  }
   WgradArgs a = args;
   TapsShape ts;
   const int N = int(a.npix / ((long long)a.H * a.W));

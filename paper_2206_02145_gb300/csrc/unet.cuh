@@ -69,7 +69,13 @@ struct WgradArgs {
   // or null: the per-tap kernel with atomics, and no bias gradient (error)
   float* part;
   size_t part_cap;
+  int tensor_path;  // 1: tcgen05 kernel (wgrad_tc.cu) where the shape allows; 0: mma.sync
+  unsigned* err;    // device word: bit 2 set if a tcgen05 kernel timed out waiting
 };
+// the tcgen05 weight gradient: floats of scratch it wants (0: shape not taken);
+// launches it and sets *used, or leaves the call to the others
+size_t wgrad_tc_scratch(int Cout, int Cin, int N, int H, int W);
+cudaError_t wgrad_tc(const WgradArgs& a, bool* used, cudaStream_t s);
 cudaError_t wgrad3x3(const WgradArgs& a, cudaStream_t s);
 // floats of scratch wgrad3x3 needs for a layer (the nine-tap kernel's
 // partials where its shape allows it, else the per-tap kernel's partials at

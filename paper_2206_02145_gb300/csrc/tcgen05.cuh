@@ -31,17 +31,6 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t sbo, uint
   return d;
 }
 
-// The same with the matrix starting `row` rows (of one swizzle span, rb
-// bytes) into a 1024-byte aligned swizzled buffer.  The swizzle phase follows
-// the absolute shared-memory address (as the TMA wrote it), so the start may
-// sit at any row with the base-offset field left at 0 (measured: setting it
-// to the row's phase, or starting at the aligned group with that phase,
-// gives wrong products).
-__device__ __forceinline__ uint64_t umma_desc_row(uint32_t saddr_aligned, int row, uint32_t rb,
-                                                  uint32_t sbo, uint32_t mode) {
-  return umma_desc(saddr_aligned + uint32_t(row) * rb, sbo, mode);
-}
-
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
@@ -59,13 +48,25 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
                : "memory");
 }
-__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                       uint32_t accumulate) {
+// D += A B (or =).  Descriptors as their two words: the first holds the address / 16
+// (below 2^14) and the leading offset, so that an offset into the operand is
+// one addition to it; the second is the same for a whole loop.
+__device__ __forceinline__ void tc_mma(uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                          uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+      "setp.ne.b32 p, %6, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}" ::"r"(d),
+      "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
       : "memory");
+}
+// one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
 }
 // arrives on `bar` once every tcgen05 operation this thread issued so far is done
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {

@@ -26,9 +26,9 @@
 // BN / 4 cycles of tensor work; per 16 pixels 9.2 KB of x come in per 64
 // channels.  In FP32 sums a run is at most 32 patches (256 products in a row).
 // Minibatch of 8 x 256 x 512 pixels, per layer, against the warp-level
-// mma.sync kernels (unet.cu): 16 -> 32 channels 173 -> 37 us, 32 -> 32 84 -> 42,
-// 64 -> 32 165 -> 93, at half the width and height 128 -> 64 163 -> 50, at a
-// quarter 256 -> 128 163 -> 50, at an eighth 256 -> 256 84 -> 30.
+// mma.sync kernels (unet.cu): 16 -> 32 channels 173 -> 34 us, 32 -> 32 84 -> 40,
+// 64 -> 32 165 -> 70, at half the width and height 128 -> 64 163 -> 40, at a
+// quarter 256 -> 128 163 -> 38, at an eighth 256 -> 256 84 -> 24.
 // Every wait is bounded, as in conv_tc.cu.
 #include "tcgen05.cuh"
 #include "tma_host.h"
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kWgThreads, WgShape<CB, BN>::CTAS)
   __shared__ uint32_t tmem_base;
   __shared__ float sbias[1024 / BN][BN + 1];
   uint8_t* smem = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int tile = blockIdx.x / a.nchunks, ck = blockIdx.x % a.nchunks;
   const int ci0 = (tile % a.ncb) * CB, co0 = (tile / a.ncb) * BN;
   const int pbeg = ck * a.run, pend = min(pbeg + a.run, a.patches);
@@ -147,33 +147,41 @@ __global__ void __launch_bounds__(kWgThreads, WgShape<CB, BN>::CTAS)
     // every issued copy has landed before the CTA may finish
     for (int j = it > S ? it - S : 0; j < it; ++j)
       if (!mbar_wait_bounded(&full[j % S], uint32_t(j / S) & 1u, kTcSpin)) atomicOr(a.err, 2u);
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
+    // the whole warp walks the patches, one lane issues
     const uint32_t s0 = smem_addr(smem);
+    const uint64_t da = umma_desc_mn(s0, Sh::step(0), 8 * Sh::PA, Sh::mode(CB));
+    const uint64_t db = umma_desc_mn(s0 + Sh::X_BYTES, 0, 8 * Sh::PB, Sh::mode(BN));
+    const uint32_t a_hi = uint32_t(da >> 32), b_hi = uint32_t(db >> 32);
+    const bool leader = elect_one();
     bool ok = true;
-    for (int p = pbeg, it = 0; p < pend && ok; ++p, ++it) {
+    for (int p = pbeg, it = 0; p < pend; ++p, ++it) {
       const int st = it % S;
-      if (!mbar_wait_bounded(&full[st], uint32_t(it / S) & 1u, kTcSpin)) {
-        atomicOr(a.err, 2u);
-        ok = false;
-        break;
-      }
+      ok = mbar_wait_bounded(&full[st], uint32_t(it / S) & 1u, kTcSpin);
+      if (!(ok = __all_sync(0xffffffffu, ok))) break;
       tc_fence_after();
-      const uint32_t sa = s0 + uint32_t(st * Sh::STAGE), sb = sa + Sh::X_BYTES;
+      const uint32_t so = uint32_t(st * Sh::STAGE) >> 4;
+      const uint32_t a_lo = uint32_t(da) + so, b_lo = uint32_t(db) + so;
+      if (leader) {
 #pragma unroll
-      for (int k = 0; k < kWgPix / 16; ++k) {
-        const uint32_t ka = uint32_t(k * 16 * Sh::PA), kb = uint32_t(k * 16 * Sh::PB);
-        const uint64_t db = umma_desc_mn(sb + kb, 0, 8 * Sh::PB, Sh::mode(BN));
+        for (int k = 0; k < kWgPix / 16; ++k)
 #pragma unroll
-        for (int t = 0; t < Sh::NT; ++t)
-          tc_mma(tmem + uint32_t(t * BN),
-                 umma_desc_mn(sa + ka + uint32_t(Sh::start(t)), Sh::step(t), 8 * Sh::PA,
-                              Sh::mode(CB)),
-                 db, Sh::IDESC, (it | k) != 0);
+          for (int t = 0; t < Sh::NT; ++t)
+            tc_mma(tmem + uint32_t(t * BN),
+                   a_lo + uint32_t((k * 16 * Sh::PA + Sh::start(t)) >> 4) +
+                       (uint32_t((Sh::step(t) - Sh::step(0)) >> 4) << 16),
+                   a_hi, b_lo + uint32_t((k * 16 * Sh::PB) >> 4), b_hi, Sh::IDESC,
+                   k != 0 || it != 0);
+        tc_commit(&empty[st]);
       }
-      tc_commit(&empty[st]);
+      __syncwarp();
     }
-    tc_commit(&done);  // (also after a time-out: products in flight end before the CTA does)
-    if (!mbar_wait_bounded(&done, 0u, kTcSpin)) atomicOr(a.err, 2u);
+    if (!ok && leader) atomicOr(a.err, 2u);
+    if (leader) {
+      tc_commit(&done);  // (also after a time-out: products in flight end before the CTA does)
+      if (!mbar_wait_bounded(&done, 0u, kTcSpin)) atomicOr(a.err, 2u);
+    }
+    __syncwarp();
   } else if (warp >= 2) {
     const int q = warp & 3, tid = q * 32 + lane;
     bool ok = true;

@@ -124,6 +124,7 @@ struct TcArgs {
   int Cout;              // output channels (bias entries)
   const float* bias;
   const bf16* mask;
+  int mask_ch;  // masked channels, from the first
   bf16* y;
   unsigned* err;
 };
@@ -308,11 +309,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const long long o = p * a.Cy + a.co_off + n0 + c;
         uint32_t out[16];
         uint4 mk[4];
-        mask_rows(mk, lane, a.Cy, a.mask ? a.mask + o : nullptr);
+        const bool masked = a.mask && n0 + c < a.mask_ch;
+        mask_rows(mk, lane, a.Cy, masked ? a.mask + o : nullptr);
         finish32(tmem + (uint32_t(q * 32) << 16) + uint32_t(buf * Sh::ACC + g * BN + c),
                  sbias + n0 + c, a.relu, out);
         out_put(rows, lane, out);
-        out_rows(rows, lane, a.y + o, a.Cy, a.mask != nullptr, mk);
+        out_rows(rows, lane, a.y + o, a.Cy, masked, mk);
       }
       // this warp's reads of the accumulator are done: hand it back
       tc_fence_before();
@@ -379,6 +381,7 @@ struct HaloArgs {
   int Cy, co_off, relu, Cout;
   const float* bias;
   const bf16* mask;
+  int mask_ch;  // masked channels, from the first
   bf16* y;
   unsigned* err;
   // fused 1x1 head (null head_y: none): with one channel tile holding all
@@ -553,6 +556,18 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     uint8_t* const rows = smem + Sh::OUT_OFF + (warp - 2) * 2048;
     int tc = 0;
     for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++tc) {
+      int img, h0, w0, n0;
+      tile_at(t, img, h0, w0, n0);
+      const long long p0 = ((long long)img * a.H + h0) * a.W + w0 + q * 32;
+      // the mask of an item (a row's 32 channels), one item ahead: its latency
+      // passes during the wait and the item before (32 -> 64 channels, half of them
+      // masked, at 8 x 256 x 512: 71 us, asked for in place 84, without a mask 54)
+      uint4 mk[4];
+      auto item_at = [&](int e) {
+        return (p0 + (long long)(e / (BN / 32)) * a.W) * a.Cy + a.co_off + n0 + e % (BN / 32) * 32;
+      };
+      auto masked = [&](int e) { return a.mask && n0 + e % (BN / 32) * 32 < a.mask_ch; };
+      if (we < G * (BN / 32)) mask_rows(mk, lane, a.Cy, masked(we) ? a.mask + item_at(we) : nullptr);
       const int buf = tc & 1;
       bool ok = mbar_wait_bounded(&acc_full[buf], uint32_t(tc >> 1) & 1u, kTcSpin);
       ok = __all_sync(0xffffffffu, ok);
@@ -561,10 +576,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         break;
       }
       tc_fence_after();
-      int img, h0, w0, n0;
-      tile_at(t, img, h0, w0, n0);
       const uint32_t ta = tmem + (uint32_t(q * 32) << 16) + uint32_t(buf * Sh::ACC);
-      const long long p0 = ((long long)img * a.H + h0) * a.W + w0 + q * 32;
       bool pooled = false;
       if constexpr (G % 2 == 0) {
         if (pool) {
@@ -658,14 +670,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       } else if (!pooled) {
 #pragma unroll 1
         for (int e = we; e < G * (BN / 32); e += kEpi) {
-          const int g = e / (BN / 32), c = e % (BN / 32) * 32;
-          const long long o = (p0 + (long long)g * a.W) * a.Cy + a.co_off + n0 + c;
+          const int g = e / (BN / 32), c = e % (BN / 32) * 32, en = e + kEpi;
+          uint4 cur[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) cur[i] = mk[i];
+          if (en < G * (BN / 32))
+            mask_rows(mk, lane, a.Cy, masked(en) ? a.mask + item_at(en) : nullptr);
           uint32_t out[16];
-          uint4 mk[4];
-          mask_rows(mk, lane, a.Cy, a.mask ? a.mask + o : nullptr);
           finish32(ta + uint32_t(g * BN + c), sbias + n0 + c, a.relu, out);
           out_put(rows, lane, out);
-          out_rows(rows, lane, a.y + o, a.Cy, a.mask != nullptr, mk);
+          out_rows(rows, lane, a.y + item_at(e), a.Cy, masked(e), cur);
         }
       }
       tc_fence_before();
@@ -830,6 +844,7 @@ static cudaError_t conv3x3_tc_halo(const ConvArgs& a, unsigned* err, cudaStream_
   t.Cout = a.Cout;
   t.bias = a.bias;
   t.mask = a.mask;
+  t.mask_ch = a.mask_ch;
   t.y = a.y;
   t.err = err;
   // the head rides along when one tile holds every channel of a pixel
@@ -916,6 +931,7 @@ cudaError_t conv3x3_tc(const ConvArgs& a, unsigned* err, cudaStream_t s) {
   t.relu = a.relu;
   t.bias = a.bias;
   t.mask = a.mask;
+  t.mask_ch = a.mask_ch;
   t.y = a.y;
   t.err = err;
   t.mtiles = int(npix / 128);

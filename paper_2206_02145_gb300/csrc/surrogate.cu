@@ -12,6 +12,7 @@
 // Activations and weights are bf16 (weights keep an FP32 master copy for
 // Adam); every GEMM accumulates in FP32.  Inputs are padded to 16 channels.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -207,9 +208,10 @@ int conv_fwd(lbpf_unet* n, const ConvLayer& l, const Act& x, int xoff, const Act
 
 // backward of one layer whose input is x[xoff..] and whose pre-activation
 // gradient is g[goff..]: weight and bias gradients, and (if gx) the input
-// gradient, optionally masked by `mask` (same layout as gx).
+// gradient, optionally masked by `mask` (same layout as gx) in its first mask_ch
+// channels.
 int conv_bwd(lbpf_unet* n, const ConvLayer& l, const Act& x, int xoff, const Act& g, int goff,
-             const Act* gx, int gxoff, const Act* mask) {
+             const Act* gx, int gxoff, const Act* mask, int mask_ch = INT_MAX) {
   const long long npix = (long long)n->cfg.batch * x.h * x.w;
   lbk::nn::WgradArgs wa{};
   wa.x = x.p;
@@ -248,6 +250,7 @@ int conv_bwd(lbpf_unet* n, const ConvLayer& l, const Act& x, int xoff, const Act
     a.W = x.w;
     a.relu = 0;
     a.mask = mask ? mask->p : nullptr;
+    a.mask_ch = mask_ch;
     a.tensor_path = n->tensor_path;
     a.err = n->d_err;
     UCK(n, lbk::nn::conv3x3(a, n->stream));
@@ -318,10 +321,11 @@ int backward(lbpf_unet* n, const float* t) {
   for (int l = 0; l < L - 1; ++l) {
     if ((rc = conv_bwd(n, n->dec_b[l], n->da[l], 0, n->g_db[l], 0, &n->g_da[l], 0, &n->da[l])))
       return rc;
-    if ((rc = conv_bwd(n, n->dec_a[l], n->cat[l], 0, n->g_da[l], 0, &n->g_cat[l], 0, nullptr)))
+    // the upsampled half of the concatenation is masked here (its ReLU), the skip
+    // half with the pooling's gradient below
+    if ((rc = conv_bwd(n, n->dec_a[l], n->cat[l], 0, n->g_da[l], 0, &n->g_cat[l], 0, &n->cat[l],
+                       n->C[l])))
       return rc;
-    UCK(n, lbk::nn::relu_mask(n->g_cat[l].p, n->g_cat[l].c, 0, n->cat[l].p, n->cat[l].c, 0,
-                              n->C[l], (long long)B * n->H[l] * n->W[l], n->stream));
     if ((rc = conv_bwd(n, n->up[l], n->u[l], 0, n->g_cat[l], 0, &n->g_u[l], 0, nullptr))) return rc;
     const Act& below = l + 1 < L - 1 ? n->db[l + 1] : n->bottom;
     Act& g_below = l + 1 < L - 1 ? n->g_db[l + 1] : n->g_bottom;

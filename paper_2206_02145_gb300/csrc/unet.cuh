@@ -29,6 +29,7 @@ struct ConvArgs {
   int N, H, W;
   int relu;            // apply max(0, .) to the output
   const bf16* mask;    // zero the output where mask <= 0 (same layout as y), or null
+  int mask_ch;         // ... in the first mask_ch output channels (a multiple of 32)
   int tensor_path;     // 1: tcgen05 kernel (conv_tc.cu) where the shape allows; 0: mma.sync
   unsigned* err;       // device word: bit 2 set if a tcgen05 kernel timed out waiting
   // optional 1x1 head on the output (head_y null: none), computed in the
@@ -87,8 +88,6 @@ size_t wgrad_scratch(int Cout, int Cin, int N, int H, int W, int chunk);
 size_t bias_grad_scratch(int C, long long npix);
 cudaError_t bias_grad(const bf16* g, int Cg, int off, int C, long long npix, float* db,
                       float* part, size_t part_cap, cudaStream_t s);
-cudaError_t relu_mask(bf16* g, int Cg, int goff, const bf16* act, int Ca, int aoff, int C,
-                      long long npix, cudaStream_t s);
 cudaError_t avgpool2(const bf16* x, int Cx, int xoff, bf16* y, int Cy, int yoff, int C, int B,
                      int H, int W, cudaStream_t s);
 cudaError_t avgpool2_bwd_add_mask(bf16* gs, const bf16* gp, const bf16* act, int Cs, int soff,

@@ -96,8 +96,11 @@ __device__ __forceinline__ void mask_rows(uint4 (&mk)[4], int lane, int C, const
       mk[k] = *reinterpret_cast<const uint4*>(mask + (long long)(k * 8 + (lane >> 2)) * C +
                                               (lane & 3) * 8);
 }
+// up: where the first pixel's block of the 2 x 2 upsampled output goes (null: none;
+// up_C channels, image rows up_row elements apart).
 __device__ __forceinline__ void out_rows(uint8_t* rows, int lane, bf16* y, int C, bool masked,
-                                         const uint4 (&mk)[4]) {
+                                         const uint4 (&mk)[4], bf16* up = nullptr, int up_C = 0,
+                                         long long up_row = 0) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int px = k * 8 + (lane >> 2), j = lane & 3;
@@ -112,6 +115,13 @@ __device__ __forceinline__ void out_rows(uint8_t* rows, int lane, bf16* y, int C
       }
     }
     *reinterpret_cast<uint4*>(y + (long long)px * C + j * 8) = v;
+    if (up) {
+      bf16* const d = up + (long long)(2 * px) * up_C + j * 8;
+      *reinterpret_cast<uint4*>(d) = v;
+      *reinterpret_cast<uint4*>(d + up_C) = v;
+      *reinterpret_cast<uint4*>(d + up_row) = v;
+      *reinterpret_cast<uint4*>(d + up_row + up_C) = v;
+    }
   }
 }
 
@@ -126,6 +136,7 @@ struct TcArgs {
   const bf16* mask;
   int mask_ch;  // masked channels, from the first
   bf16* y;
+  bf16* up_y;    // 2 x 2 upsampled output, Cout channels, or null
   unsigned* err;
 };
 
@@ -314,7 +325,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         finish32(tmem + (uint32_t(q * 32) << 16) + uint32_t(buf * Sh::ACC + g * BN + c),
                  sbias + n0 + c, a.relu, out);
         out_put(rows, lane, out);
-        out_rows(rows, lane, a.y + o, a.Cy, masked, mk);
+        bf16* const up =
+            a.up_y ? a.up_y + (((long long)img * a.H + h0 + q * 32 / a.BW) * 4 * a.W +
+                               2 * (w0 + q * 32 % a.BW)) * a.Cout + n0 + c
+                   : nullptr;
+        out_rows(rows, lane, a.y + o, a.Cy, masked, mk, up, a.Cout, 2ll * a.W * a.Cout);
       }
       // this warp's reads of the accumulator are done: hand it back
       tc_fence_before();
@@ -383,6 +398,7 @@ struct HaloArgs {
   const bf16* mask;
   int mask_ch;  // masked channels, from the first
   bf16* y;
+  bf16* up_y;    // 2 x 2 upsampled output, Cout channels, or null
   unsigned* err;
   // fused 1x1 head (null head_y: none): with one channel tile holding all
   // Cout channels of a pixel, head_y[p][o] = head_b[o] + sum_c head_w[o][c]
@@ -679,7 +695,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           uint32_t out[16];
           finish32(ta + uint32_t(g * BN + c), sbias + n0 + c, a.relu, out);
           out_put(rows, lane, out);
-          out_rows(rows, lane, a.y + item_at(e), a.Cy, masked(e), cur);
+          bf16* const up = a.up_y ? a.up_y + (((long long)img * a.H + h0 + g) * 4 * a.W +
+                                              2 * (w0 + q * 32)) * a.Cout + n0 + c
+                                  : nullptr;
+          out_rows(rows, lane, a.y + item_at(e), a.Cy, masked(e), cur, up, a.Cout,
+                   2ll * a.W * a.Cout);
         }
       }
       tc_fence_before();
@@ -862,6 +882,9 @@ static cudaError_t conv3x3_tc_halo(const ConvArgs& a, unsigned* err, cudaStream_
   t.pool_Cy = a.pool_Cy;
   t.pool_off = a.pool_off;
   if (a.pool_done) *a.pool_done = fpool ? 1 : 0;
+  const bool fup = a.up_y && !fuse && !fpool;
+  t.up_y = fup ? a.up_y : nullptr;
+  if (a.up_done) *a.up_done = fup ? 1 : 0;
   *used = true;
   switch (BK) {
     case 64: return launch_halo_bk<64>(BN, G, mx, mw, t, s);
@@ -933,6 +956,8 @@ cudaError_t conv3x3_tc(const ConvArgs& a, unsigned* err, cudaStream_t s) {
   t.mask = a.mask;
   t.mask_ch = a.mask_ch;
   t.y = a.y;
+  t.up_y = a.up_y;
+  if (a.up_done) *a.up_done = a.up_y ? 1 : 0;
   t.err = err;
   t.mtiles = int(npix / 128);
   t.ntiles_n = a.Cout / BN;

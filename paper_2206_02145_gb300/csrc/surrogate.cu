@@ -170,7 +170,8 @@ cudaError_t make_conv(lbpf_unet* n, ConvLayer* l, int cin, int cout, int real_ci
 // head: the 1x1 head to fuse into this layer's epilogue where the kernel can
 // (*head_done says whether it did)
 int conv_fwd(lbpf_unet* n, const ConvLayer& l, const Act& x, int xoff, const Act& y, int yoff,
-             int* head_done = nullptr, const Act* pool = nullptr, int* pool_done = nullptr) {
+             int* head_done = nullptr, const Act* pool = nullptr, int* pool_done = nullptr,
+             const Act* up = nullptr, int* up_done = nullptr) {
   lbk::nn::ConvArgs a{};
   a.x = x.p;
   a.Cx = x.c;
@@ -201,6 +202,10 @@ int conv_fwd(lbpf_unet* n, const ConvLayer& l, const Act& x, int xoff, const Act
     a.pool_Cy = pool->c;
     a.pool_off = 0;
     a.pool_done = pool_done;
+  }
+  if (up && up_done) {  // the upsampled input of the level above
+    a.up_y = up->p;
+    a.up_done = up_done;
   }
   UCK(n, lbk::nn::conv3x3(a, n->stream));
   return LBPF_OK;
@@ -268,7 +273,7 @@ std::vector<ConvLayer*> all_layers(lbpf_unet* n) {
 // forward pass on the packed input n->xin; output n->y (FP32 NHWC, out_ch)
 int forward(lbpf_unet* n) {
   const int L = n->L;
-  int rc;
+  int rc, up_done = 0;  // the upsampling rides in the epilogue of the layer below it
   for (int l = 0; l < L; ++l) {
     const Act& in = l == 0 ? n->xin : n->pool[l];
     if ((rc = conv_fwd(n, n->enc_a[l], in, 0, n->ea[l], 0))) return rc;
@@ -282,18 +287,22 @@ int forward(lbpf_unet* n) {
         UCK(n, lbk::nn::avgpool2(n->cat[l].p, n->cat[l].c, n->C[l], n->pool[l + 1].p, n->C[l], 0,
                                  n->C[l], n->cfg.batch, n->H[l], n->W[l], n->stream));
     } else {
-      if ((rc = conv_fwd(n, n->enc_b[l], n->ea[l], 0, n->bottom, 0))) return rc;
+      if ((rc = conv_fwd(n, n->enc_b[l], n->ea[l], 0, n->bottom, 0, nullptr, nullptr, nullptr,
+                         L > 1 ? &n->u[L - 2] : nullptr, &up_done)))
+        return rc;
     }
   }
   const Act* d = &n->bottom;
   int head_done = 0;
   for (int l = L - 2; l >= 0; --l) {
-    UCK(n, lbk::nn::upsample2(d->p, n->u[l].p, n->C[l + 1], n->cfg.batch, n->H[l], n->W[l],
-                              n->stream));
+    if (!up_done)
+      UCK(n, lbk::nn::upsample2(d->p, n->u[l].p, n->C[l + 1], n->cfg.batch, n->H[l], n->W[l],
+                                n->stream));
     if ((rc = conv_fwd(n, n->up[l], n->u[l], 0, n->cat[l], 0))) return rc;
     if ((rc = conv_fwd(n, n->dec_a[l], n->cat[l], 0, n->da[l], 0))) return rc;
     // the last convolution carries the 1x1 head in its epilogue where it can
-    if ((rc = conv_fwd(n, n->dec_b[l], n->da[l], 0, n->db[l], 0, l == 0 ? &head_done : nullptr)))
+    if ((rc = conv_fwd(n, n->dec_b[l], n->da[l], 0, n->db[l], 0, l == 0 ? &head_done : nullptr,
+                       nullptr, nullptr, l > 0 ? &n->u[l - 1] : nullptr, &up_done)))
       return rc;
     d = &n->db[l];
   }

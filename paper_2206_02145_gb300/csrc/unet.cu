@@ -770,6 +770,7 @@ int blocks_for(long long n) {
 cudaError_t conv3x3(const ConvArgs& a, cudaStream_t s) {
   if (a.head_done) *a.head_done = 0;
   if (a.pool_done) *a.pool_done = 0;
+  if (a.up_done) *a.up_done = 0;
   if (a.tensor_path && a.err && conv3x3_tc_supported(a)) return conv3x3_tc(a, a.err, s);
   if (a.W % 64 || a.Cin % 16 || a.Cx % 8 || a.Cy % 8 || a.ci_off % 8 || a.co_off % 8)
     return cudaErrorInvalidValue;

@@ -47,6 +47,10 @@ struct ConvArgs {
   bf16* pool_y;
   int pool_Cy, pool_off;
   int* pool_done;
+  // optional nearest 2 x 2 upsampling of the output (up_y null: none), written
+  // beside it by the tcgen05 kernels (*up_done = 1): up_y [N][2 H][2 W][Cout]
+  bf16* up_y;
+  int* up_done;
 };
 // requirements: W % 64 == 0, Cin % 16 == 0, Cout % 32 == 0, strides/offsets % 8 == 0
 cudaError_t conv3x3(const ConvArgs& a, cudaStream_t s);

@@ -45,11 +45,11 @@ sys.path.insert(0, ROOT)
 # the files each timed kernel is compiled from (a committed profile's counters
 # stand only while their digest is unchanged)
 SRC_2D = ["step2d.cu", "step2d_tile.cuh", "step2d_core.cuh", "lbpf_device.cuh", "tma.cuh"]
-SRC_3D = ["step3d.cu", "step3d_core.cuh", "lbpf_device.cuh"]
+SRC_3D = ["step3d.cu", "step3d_core.cuh", "lbpf_device.cuh", "tma.cuh"]
 SRC_BATCH = ["batch2d.cu", "batch2d_kernels.cuh", "batch2d_fp32.cu", "batch2d_fp16.cu",
              "batch2d_bf16.cu", "batch_schedule.h", "step2d_tile.cuh", "step2d_core.cuh",
              "lbpf_device.cuh", "tma.cuh"]
-SRC_CONV = ["conv_tc.cu", "tma.cuh"]
+SRC_CONV = ["conv_tc.cu", "tcgen05.cuh", "tma.cuh"]
 SRC_FACETS = ["facets.cu"]
 
 # bytes each node moves through HBM per step (populations read + written,
@@ -96,7 +96,7 @@ WORKLOADS = {
                     "0.04, sphere R=12, U0=0.3, inflow 0.005",
                dim=3, nx=256, ny=256, nz=256, flow=1, fold=0, eps=0.04, bc=(1, 0, 0),
                u_in=0.005, U_in=0.3, seed=(128.0, 128.0, 128.0, 12.0, 0.3, 0.01, 1),
-               storage="fp32", kernel="step3d_march_kernel", src=SRC_3D,
+               storage="fp32", kernel="step3d_column_kernel", src=SRC_3D,
                sample=dict(nx=48, ny=48, nz=48, seed=(24.0, 24.0, 24.0, 12.0, 0.3, 0.01, 1))),
     "c3_fp16": dict(base="c3", storage="fp16"),
     "c3s": dict(base="c3", nx=128, ny=128, nz=128, seed=(64.0, 64.0, 64.0, 12.0, 0.3, 0.01, 1),
@@ -114,9 +114,9 @@ WORKLOADS = {
                        "eps 0.04, sphere R=12, U0=0.3, inflow 0.005, the flow colliding by the "
                        "central Hermite MRT (trace of the second-order and the third/fourth-"
                        "order central moments relaxed at 1)",
-                  collision=1, kernel="step3d_march_kernel_chm"),
+                  collision=1, kernel="step3d_column_kernel_chm"),
     "f3_3ds": dict(base="c3", nx=128, ny=128, nz=128, collision=1,
-                   kernel="step3d_march_kernel_chm",
+                   kernel="step3d_column_kernel_chm",
                    seed=(64.0, 64.0, 64.0, 12.0, 0.3, 0.01, 1), desc_note=True,
                    desc="3D 128^3 case of f3_3d for profiler captures (D3Q19 flow colliding by "
                         "the central Hermite MRT, D3Q7 solute and phase field), cubic eps 0.04, "
@@ -1254,7 +1254,7 @@ def run_surrogate(args, w):
                    "sample": f"{osteps} LB steps of a 256x256 closed channel of the same family "
                              f"({n} nodes), {dt:.1f} s, FP64"}
         rep = head["report"]
-        launches = (K + 1) * 31 + rep["surrogate_blocks"] * 2 + (
+        launches = (K + 1) * 28 + rep["surrogate_blocks"] * 2 + (
             rep["judged_blocks"] + rep["fallback_blocks"]) * nb
         out = {
             "metric": "LB-equivalent MLUPS (learned block propagator)", "value": head["value"],

@@ -77,10 +77,9 @@ struct Model {
   int rel_g;
   __half* uring;
   // Solid nodes (walls, obstacles): one byte per node at (z * ny + y) * px +
-  // x, 1 = solid; null when there are none.  solid_tiles: in 2D one byte per
-  // 32 x 4 tile of the step (row-major over the tiles), in 3D one per 32 x 4 x 8
-  // block of nodes; 1 = the tile or block or its one-node halo
-  // holds a solid node
+  // x, 1 = solid; null when there are none.  solid_tiles: in 2D one byte per tile
+  // of the step (row-major over the tiles), in 3D one per 32 x 4 x 8 block of
+  // nodes; 1 = the tile or block or its one-node halo holds a solid node
   const unsigned char* solid;
   const unsigned char* solid_tiles;
 };

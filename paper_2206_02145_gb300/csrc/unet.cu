@@ -5,8 +5,10 @@
 //                    channels); also the data gradient, run on flipped /
 //                    transposed weights.  Shapes the tcgen05 kernel of
 //                    conv_tc.cu takes go there instead.
-//   wgrad3x3_kernel  weight gradient, K = pixels, split over CTAs, FP32 atomics
-//   element-wise     bias gradient, ReLU masks, 2x2 average pooling and its
+//   wgrad_taps_kernel, wgrad3x3_kernel
+//                    weight gradient on the same path, K = pixels; shapes the
+//                    kernel of wgrad_tc.cu takes go there instead
+//   element-wise     bias gradient, 2x2 average pooling and its
 //                    gradient, nearest 2x upsampling and its gradient, the 1x1
 //                    head, MSE loss, Adam, weight transposition, input packing
 #include <algorithm>
@@ -498,6 +500,7 @@ __global__ void avgpool_kernel(const bf16* x, int Cx, int xoff, bf16* y, int Cy,
 // g_skip = (g_skip + 0.25 g_pool[pooled position]) * (skip > 0)
 __global__ void pool_bwd_add_mask_kernel(bf16* gs, const bf16* gp, const bf16* act, int Cs,
                                          int soff, int C, int B, int H, int W) {
+  pdl_wait();
   const int groups = C / 8;
   const long long n = (long long)B * H * W * groups;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -541,6 +544,7 @@ __global__ void upsample_kernel(const bf16* x, bf16* y, int C, int B, int H, int
 // gradient of the upsampling (sum of the 2x2 block), masked by act > 0
 __global__ void upsample_bwd_mask_kernel(const bf16* g, bf16* gx, const bf16* act, int C, int B,
                                          int H, int W) {
+  pdl_wait();
   const int Ho = H / 2, Wo = W / 2, groups = C / 8;
   const long long n = (long long)B * Ho * Wo * groups;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -607,6 +611,7 @@ template <int O>
 __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16* x, const float* w,
                                                        const float* gy, long long npix, bf16* gx,
                                                        float* part) {
+  pdl_wait();
   constexpr int C = 32;
   __shared__ float red[8][O][C + 1];  // per warp: dw[o][c] at [o][c], db[o] at [o][C]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, c0 = (lane & 3) * 8;
@@ -669,6 +674,8 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16* x, const floa
 // row: a block takes 32 entries, its 32 warps every 32nd row each, summed in order
 __global__ void __launch_bounds__(1024) sum_rows_kernel(const float* __restrict__ part, int row,
                                                         int n, int rows, float* dw, float* db) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ float red[32][33];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, i = blockIdx.x * 32 + lane;
   float t = 0.f;
@@ -925,9 +932,8 @@ cudaError_t avgpool2(const bf16* x, int Cx, int xoff, bf16* y, int Cy, int yoff,
 cudaError_t avgpool2_bwd_add_mask(bf16* gs, const bf16* gp, const bf16* act, int Cs, int soff,
                                   int C, int B, int H, int W, cudaStream_t s) {
   if (!v8(C) || !v8(Cs) || !v8(soff)) return cudaErrorInvalidValue;
-  pool_bwd_add_mask_kernel<<<blocks_for((long long)B * H * W * C / 8), 256, 0, s>>>(
-      gs, gp, act, Cs, soff, C, B, H, W);
-  return cudaGetLastError();
+  return launch_pdl(pool_bwd_add_mask_kernel, dim3(blocks_for((long long)B * H * W * C / 8)),
+                    dim3(256), 0, s, gs, gp, act, Cs, soff, C, B, H, W);
 }
 cudaError_t upsample2(const bf16* x, bf16* y, int C, int B, int H, int W, cudaStream_t s) {
   if (!v8(C)) return cudaErrorInvalidValue;
@@ -937,9 +943,8 @@ cudaError_t upsample2(const bf16* x, bf16* y, int C, int B, int H, int W, cudaSt
 cudaError_t upsample2_bwd_mask(const bf16* g, bf16* gx, const bf16* act, int C, int B, int H,
                                int W, cudaStream_t s) {
   if (!v8(C)) return cudaErrorInvalidValue;
-  upsample_bwd_mask_kernel<<<blocks_for((long long)B * H * W * C / 32), 256, 0, s>>>(g, gx, act,
-                                                                                    C, B, H, W);
-  return cudaGetLastError();
+  return launch_pdl(upsample_bwd_mask_kernel, dim3(blocks_for((long long)B * H * W * C / 32)),
+                    dim3(256), 0, s, g, gx, act, C, B, H, W);
 }
 cudaError_t head_fwd(const bf16* x, int C, const float* w, const float* b, float* y, int O,
                      long long npix, cudaStream_t s) {
@@ -970,20 +975,20 @@ cudaError_t head_bwd(const bf16* x, int C, const float* w, const float* gy, int 
   const int blocks = head_bwd_blocks(npix), row = O * C + O;
   if (size_t(blocks) * row > part_cap) return cudaErrorInvalidValue;
   const dim3 g{unsigned(blocks)}, bl{256};
+  cudaError_t e;
   switch (O) {
-    case 1: head_bwd_kernel<1><<<g, bl, 0, s>>>(x, w, gy, npix, gx, part); break;
-    case 2: head_bwd_kernel<2><<<g, bl, 0, s>>>(x, w, gy, npix, gx, part); break;
-    case 3: head_bwd_kernel<3><<<g, bl, 0, s>>>(x, w, gy, npix, gx, part); break;
-    case 4: head_bwd_kernel<4><<<g, bl, 0, s>>>(x, w, gy, npix, gx, part); break;
-    case 5: head_bwd_kernel<5><<<g, bl, 0, s>>>(x, w, gy, npix, gx, part); break;
-    case 6: head_bwd_kernel<6><<<g, bl, 0, s>>>(x, w, gy, npix, gx, part); break;
-    case 7: head_bwd_kernel<7><<<g, bl, 0, s>>>(x, w, gy, npix, gx, part); break;
-    default: head_bwd_kernel<8><<<g, bl, 0, s>>>(x, w, gy, npix, gx, part); break;
+    case 1: e = launch_pdl(head_bwd_kernel<1>, g, bl, 0, s, x, w, gy, npix, gx, part); break;
+    case 2: e = launch_pdl(head_bwd_kernel<2>, g, bl, 0, s, x, w, gy, npix, gx, part); break;
+    case 3: e = launch_pdl(head_bwd_kernel<3>, g, bl, 0, s, x, w, gy, npix, gx, part); break;
+    case 4: e = launch_pdl(head_bwd_kernel<4>, g, bl, 0, s, x, w, gy, npix, gx, part); break;
+    case 5: e = launch_pdl(head_bwd_kernel<5>, g, bl, 0, s, x, w, gy, npix, gx, part); break;
+    case 6: e = launch_pdl(head_bwd_kernel<6>, g, bl, 0, s, x, w, gy, npix, gx, part); break;
+    case 7: e = launch_pdl(head_bwd_kernel<7>, g, bl, 0, s, x, w, gy, npix, gx, part); break;
+    default: e = launch_pdl(head_bwd_kernel<8>, g, bl, 0, s, x, w, gy, npix, gx, part); break;
   }
-  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  sum_rows_kernel<<<(row + 31) / 32, 1024, 0, s>>>(part, row, O * C, blocks, dw, db);
-  return cudaGetLastError();
+  return launch_pdl(sum_rows_kernel, dim3(unsigned((row + 31) / 32)), dim3(1024), 0, s,
+                    static_cast<const float*>(part), row, O * C, blocks, dw, db);
 }
 cudaError_t mse(const float* y, const float* t, long long n, float* gy, float* loss,
                 cudaStream_t s) {

@@ -270,6 +270,8 @@ __global__ void __launch_bounds__(256) wgrad_sum_kernel(const float* __restrict_
   __shared__ float4 red[G][NL];
   const int g = threadIdx.x / NL, l = threadIdx.x % NL;
   const int i = (blockIdx.x * NL + l) * 4;  // row and n are multiples of 4
+  pdl_trigger();
+  pdl_wait();
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
   if (i < row) {
     const float* p = part + i;
@@ -394,14 +396,12 @@ cudaError_t wgrad_tc(const WgradArgs& a, bool* used, cudaStream_t s) {
   }
   if (e != cudaSuccess) return e;
   const int n = int(wg_row(a.Cout, a.Cin, false));
-  if (row < size_t(2 * 152) * 128)
-    wgrad_sum_kernel<32><<<unsigned((row + 31) / 32), 256, 0, s>>>(a.part, int(row), n, p.nchunks,
-                                                                   a.dw, a.db);
-  else
-    wgrad_sum_kernel<8><<<unsigned((row + 127) / 128), 256, 0, s>>>(a.part, int(row), n, p.nchunks,
-                                                                    a.dw, a.db);
   *used = true;
-  return cudaGetLastError();
+  if (row < size_t(2 * 152) * 128)
+    return launch_pdl(wgrad_sum_kernel<32>, dim3(unsigned((row + 31) / 32)), dim3(256), 0, s,
+                      static_cast<const float*>(a.part), int(row), n, p.nchunks, a.dw, a.db);
+  return launch_pdl(wgrad_sum_kernel<8>, dim3(unsigned((row + 127) / 128)), dim3(256), 0, s,
+                    static_cast<const float*>(a.part), int(row), n, p.nchunks, a.dw, a.db);
 }
 
 }  // namespace nn

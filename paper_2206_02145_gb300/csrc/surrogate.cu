@@ -910,18 +910,23 @@ lbpf_status lbpf_surrogate_sample(lbpf_t* h, const lbpf_surrogate_cfg* cfg, floa
 
 namespace {
 
-// The prediction phase of a block, queued on s: read-out of the state and its
-// interface positions, the network, the predicted planes, their FP64 sums and
-// interface positions, and the copy of those results to pinned host memory.
-int queue_prediction(lbpf* h, lbpf_unet* net, const lbpf_surrogate_cfg* cfg, cudaStream_t s) {
-  const long long n = (long long)h->m.nx * h->m.ny;
-  const int nb = cfg->steps_per_block;
+// Read-out of the state and its interface positions, queued on s.
+int queue_readout(lbpf* h, lbpf_unet* net, const lbpf_surrogate_cfg* cfg, cudaStream_t s) {
   SCK(h, lbk::launch_surrogate_gather(h->m, h->pops[h->cur], h->cur, vec4(cfg->shift), vec4(cfg->scale),
                                       net->px, net->pF, s));
   plane_crossing_kernel<<<1, 128, 0, s>>>(net->pF, h->m.nx, h->m.ny, h->m.bc[0], h->m.bc[1], h->icx,
                                          h->icy, net->pcross + 4);
   SCK(h, cudaGetLastError());
+  return LBPF_OK;
+}
+
+// The prediction phase of a block, queued on s: the read-out, the network, the predicted planes, their FP64 sums and
+// interface positions, and the copy of those results to pinned host memory.
+int queue_prediction(lbpf* h, lbpf_unet* net, const lbpf_surrogate_cfg* cfg, cudaStream_t s) {
+  const long long n = (long long)h->m.nx * h->m.ny;
+  const int nb = cfg->steps_per_block;
   int rc;
+  if ((rc = queue_readout(h, net, cfg, s))) return rc;
   if ((rc = lbpf_unet_forward(net, net->px, net->py))) return sfail(h, rc, "network: %s", net->msg);
   apply_kernel<<<grid_of(n), 256, 0, s>>>(net->pF, net->py, vec4(cfg->res_scale), 1.0f / nb, n,
                                           net->pF1);
@@ -1051,14 +1056,24 @@ lbpf_status lbpf_surrogate_advance(lbpf_t* h, lbpf_unet_t* net, const lbpf_surro
   int rc;
   for (int b = 0; b <= blocks; ++b) {
     const bool last = b == blocks;  // only resolves the outcome of the final block
-    cudaGraphExec_t g = nullptr;
-    if ((rc = prediction_graph(h, net, cfg, &g))) return rc;
-    SCK(h, cudaGraphLaunch(g, s));
+    if (last) {  // no block follows: the interface positions are enough
+      if (lb_pending) {
+        if ((rc = queue_readout(h, net, cfg, s))) return rc;
+        SCK(h, cudaMemcpyAsync(net->hres + 7, net->pcross + 4, 4 * sizeof(double),
+                               cudaMemcpyDeviceToHost, s));
+      }
+    } else {
+      cudaGraphExec_t g = nullptr;
+      if ((rc = prediction_graph(h, net, cfg, &g))) return rc;
+      SCK(h, cudaGraphLaunch(g, s));
+    }
     SCK(h, cudaStreamSynchronize(s));
     const double* res = net->hres;
-    unsigned nerr = 0;
-    std::memcpy(&nerr, res + 11, sizeof(nerr));
-    if (nerr) return sfail(h, LBPF_ETIMEDOUT, "a tensor-core convolution gave up waiting");
+    if (!last) {
+      unsigned nerr = 0;
+      std::memcpy(&nerr, res + 11, sizeof(nerr));
+      if (nerr) return sfail(h, LBPF_ETIMEDOUT, "a tensor-core convolution gave up waiting");
+    }
     const double* posP = res + 3;
     const double* pos0 = res + 7;
     if (lb_pending) {

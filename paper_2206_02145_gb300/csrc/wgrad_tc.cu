@@ -13,8 +13,8 @@
 // fixed step apart: with CB = 64 the pairs (ky 0, 1) of each kx, the pair (kx 0,
 // 1) of ky 2, and ky 2, kx 2; with fewer channels ky = 0, 1, 2 of one kx per
 // product.  The step after the last tap reads whatever lies there, into rows of
-// D that nobody reads.  Pixels outside the image are zeros (the TMA's fill), in
-// x and, for the patches that reach over an edge, in dy.
+// D that nobody reads.  Pixels outside the image are zeros (the TMA's fill); a
+// patch's rows below the image are left out.
 //   warp 0     TMA producer, a ring of S patches
 //   warp 1     tensor memory; one lane issues the products (8 steps x NT per patch)
 //   warps 2-5  where asked, sum dy over the pixels meanwhile (the bias gradient, by
@@ -160,11 +160,15 @@ __global__ void __launch_bounds__(kWgThreads, WgShape<CB, BN>::CTAS)
       ok = mbar_wait_bounded(&full[st], uint32_t(it / S) & 1u, kTcSpin);
       if (!(ok = __all_sync(0xffffffffu, ok))) break;
       tc_fence_after();
+      // image rows of the patch: those below the image are left out, so that
+      // they don't multiply the halo's values by zero
+      const int rows = a.H % kWgRows ? min(kWgRows, a.H - p % (a.pw * a.ph) / a.pw * kWgRows) : kWgRows;
       const uint32_t so = uint32_t(st * Sh::STAGE) >> 4;
       const uint32_t a_lo = uint32_t(da) + so, b_lo = uint32_t(db) + so;
       if (leader) {
 #pragma unroll
-        for (int k = 0; k < kWgPix / 16; ++k)
+        for (int k = 0; k < kWgPix / 16; ++k) {
+          if (k / (kWgCols / 16) >= rows) break;
 #pragma unroll
           for (int t = 0; t < Sh::NT; ++t)
             tc_mma(tmem + uint32_t(t * BN),
@@ -172,6 +176,7 @@ __global__ void __launch_bounds__(kWgThreads, WgShape<CB, BN>::CTAS)
                        (uint32_t((Sh::step(t) - Sh::step(0)) >> 4) << 16),
                    a_hi, b_lo + uint32_t((k * 16 * Sh::PB) >> 4), b_hi, Sh::IDESC,
                    k != 0 || it != 0);
+        }
         tc_commit(&empty[st]);
       }
       __syncwarp();
@@ -307,7 +312,7 @@ struct WgPlan {
 // Runs: as many CTAs as the SMs hold at once, or a multiple of that where a run
 // would be longer than kWgMaxRun patches.
 bool wg_plan(int Cout, int Cin, int N, int H, int W, WgPlan* p) {
-  if (Cout % 32 || Cin % 16 || N < 1 || H < 1 || W < 1) return false;
+  if (Cout % 32 || Cin % 16 || N < 1 || H < 1 || W < 1 || W % kWgCols) return false;
   p->cb = Cin % 64 == 0 ? 64 : (Cin % 32 == 0 ? 32 : 16);
   p->bn = Cout % 64 == 0 ? 64 : 32;
   p->ncb = Cin / p->cb;

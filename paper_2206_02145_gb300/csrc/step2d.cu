@@ -261,18 +261,22 @@ int shape_of(const Model& m) {
   return tiles >= kPairTiles ? SH_PAIR : SH_SMALL;
 }
 
-// one thread per tx x ty tile: does the tile or its one-node halo (mapped
-// like the gradient stencil) hold a solid node?
+
+// A warp per tile of the TMA kernel: does the tile or its one-node halo (mapped
+// like the gradient stencil) hold a solid node?  (A thread per tile is a chain of
+// 204 loads: 120 us of lbpf_set_solid's 400 at 775 x 650.)
 __global__ void solid_tiles_kernel(const Model m, unsigned char* flags, int ntx, int nty, int tx,
                                    int ty) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x % 32;
   if (t >= ntx * nty) return;
   const int x0 = (t % ntx) * tx, y0 = (t / ntx) * ty;
   const int xe = x0 + tx < m.nx ? x0 + tx : m.nx, ye = y0 + ty < m.ny ? y0 + ty : m.ny;
   bool any = false;
+#pragma unroll 2
   for (int y = y0 - 1; y <= ye; ++y)
-    for (int x = x0 - 1; x <= xe; ++x) any |= solid_mapped(m, x, y);
-  flags[t] = any ? 1 : 0;
+    for (int x = x0 - 1 + lane; x <= xe; x += 32) any |= solid_mapped(m, x, y);
+  any = __any_sync(0xffffffffu, any);
+  if (lane == 0) flags[t] = any ? 1 : 0;
 }
 
 template <typename T, bool FLOW, int kTX, int kTY, bool PAIR>
@@ -446,7 +450,7 @@ cudaError_t launch_solid_tiles(const Model& m, unsigned char* flags, cudaStream_
   if (m.dim != 2 || !m.solid) return cudaErrorInvalidValue;
   const int tx = kShapeX[shape_of(m)], ty = kShapeY[shape_of(m)];
   const int ntx = (m.nx + tx - 1) / tx, nty = (m.ny + ty - 1) / ty;
-  solid_tiles_kernel<<<(ntx * nty + 127) / 128, 128, 0, s>>>(m, flags, ntx, nty, tx, ty);
+  solid_tiles_kernel<<<(ntx * nty + 3) / 4, 128, 0, s>>>(m, flags, ntx, nty, tx, ty);
   return cudaGetLastError();
 }
 

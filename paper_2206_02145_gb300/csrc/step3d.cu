@@ -479,11 +479,11 @@ cudaError_t launch3_column_t(const Model& m, const StepMaps& maps, int c, const 
   return cudaGetLastError();
 }
 
-// one thread per kFlagX x kFlagY x kFlagZ block of nodes: does it or its one-node
+// one warp per kFlagX x kFlagY x kFlagZ block of nodes: does it or its one-node
 // halo (mapped like the gradient stencil) hold a solid node?
 __global__ void solid_chunks_kernel(const Model m, unsigned char* flags, int ntx, int nty,
                                     int nzc) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x % 32;
   if (t >= ntx * nty * nzc) return;
   const int x0 = (t % ntx) * kFlagX, y0 = ((t / ntx) % nty) * kFlagY,
             z0 = (t / (ntx * nty)) * kFlagZ;
@@ -491,10 +491,13 @@ __global__ void solid_chunks_kernel(const Model m, unsigned char* flags, int ntx
   const int ye = y0 + kFlagY < m.ny ? y0 + kFlagY : m.ny;
   const int ze = z0 + kFlagZ < m.nz ? z0 + kFlagZ : m.nz;
   bool any = false;
-  for (int z = z0 - 1; z <= ze && !any; ++z)
-    for (int y = y0 - 1; y <= ye && !any; ++y)
-      for (int x = x0 - 1; x <= xe && !any; ++x) any = solid_mapped3(m, x, y, z);
-  flags[t] = any ? 1 : 0;
+  for (int z = z0 - 1; z <= ze && !any; ++z) {
+#pragma unroll 2
+    for (int y = y0 - 1; y <= ye; ++y)
+      for (int x = x0 - 1 + lane; x <= xe; x += 32) any |= solid_mapped3(m, x, y, z);
+    any = __any_sync(0xffffffffu, any);
+  }
+  if (lane == 0) flags[t] = any ? 1 : 0;
 }
 
 // ---- host side -------------------------------------------------------------------
@@ -536,7 +539,7 @@ cudaError_t launch_solid_chunks(const Model& m, unsigned char* flags, cudaStream
   const int ntx = (m.nx + kFlagX - 1) / kFlagX, nty = (m.ny + kFlagY - 1) / kFlagY,
             nzc = (m.nz + kFlagZ - 1) / kFlagZ;
   const int n = ntx * nty * nzc;
-  solid_chunks_kernel<<<(n + 127) / 128, 128, 0, s>>>(m, flags, ntx, nty, nzc);
+  solid_chunks_kernel<<<(n + 3) / 4, 128, 0, s>>>(m, flags, ntx, nty, nzc);
   return cudaGetLastError();
 }
 

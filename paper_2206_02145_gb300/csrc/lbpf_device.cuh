@@ -188,13 +188,17 @@ __device__ __forceinline__ void set_lane(N& v, int k, typename Lanes<N>::S s) {
   if constexpr (Lanes<N>::V == 2) (k ? v.y : v.x) = s;
   else v = s;
 }
-// are a, b and c finite (in every lane)?
+// 0 in every lane where a, b and c are finite, elsewhere NaN
 template <typename N>
-__device__ __forceinline__ bool all_finite(N a, N b, N c) {
+__device__ __forceinline__ N finite_mark(N a, N b, N c) {
   const N z = splat<N>(typename Lanes<N>::S(0));
-  const N t = fma_r(c, z, fma_r(b, z, mul_r(a, z)));
-  if constexpr (Lanes<N>::V == 2) return t.x + t.y == 0.f;
-  else return t == typename Lanes<N>::S(0);
+  return fma_r(c, z, fma_r(b, z, mul_r(a, z)));
+}
+// is the mark 0 in every lane?
+template <typename N>
+__device__ __forceinline__ bool all_finite(N mark) {
+  if constexpr (Lanes<N>::V == 2) return mark.x + mark.y == 0.f;
+  else return mark == typename Lanes<N>::S(0);
 }
 // v where |grad phi|^2 = g2 > 1e-12, elsewhere w
 __device__ __forceinline__ float where_steep(float g2, float v, float w) {

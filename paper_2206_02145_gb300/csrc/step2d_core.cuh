@@ -129,10 +129,10 @@ struct Node2D {
 
 // Moments, gradient, anisotropy and the coefficients above (Eqs. 3-23) of a
 // node with population deviations f, g, phi + 1 = dphi (dphi_prev one step
-// earlier), the g reference Rg and the eight neighbours' phi + 1.  False if
-// phi, U or rho is not finite.
+// earlier), the g reference Rg and the eight neighbours' phi + 1.  Returns the
+// finite_mark of phi, U and rho.
 template <typename N, bool FLOW, bool CHM>
-__device__ __forceinline__ bool node_2d(const Coef<N>& c, int fold, const N (&f)[9], const N (&g)[9], N dphi,
+__device__ __forceinline__ N node_2d(const Coef<N>& c, int fold, const N (&f)[9], const N (&g)[9], N dphi,
                                         N dphi_prev, N Rg, N pE, N pW, N pN, N pS, N pNE, N pNW,
                                         N pSE, N pSW, Node2D<N>& o, N (&fchm)[9]) {
   using S = typename Lanes<N>::S;
@@ -154,7 +154,7 @@ __device__ __forceinline__ bool node_2d(const Coef<N>& c, int fold, const N (&f)
     my = sub_r(add_r(sub_r(f[2], f[4]), add_r(f[5], f[6])), add_r(f[7], f[8]));
   }
   const N rho = add_r(one, drho);
-  const bool ok = all_finite(phi, U, rho);
+  const N mark = finite_mark(phi, U, rho);
   const N ph = clamp1(phi);
   const N mask = mul_r(half, sub_r(one, ph));  // (1 - phi)/2 of Eq. 7 and q(phi) of Eq. 18
   o.usx = o.usy = o.Fx = o.Fy = splat<N>(S(0));
@@ -219,7 +219,7 @@ __device__ __forceinline__ bool node_2d(const Coef<N>& c, int fold, const N (&f)
   o.H_d = sub_r(o.Hx, o.Hy);
   // Eq. 19: h_new = h* / a_s^2 + (1 - 1/a_s^2) h_old
   o.keep_old = sub_r(one, o.inv_a2);
-  return ok;
+  return mark;
 }
 
 // c_a . v from the components and their sum and difference (a a constant
@@ -342,9 +342,15 @@ __device__ __forceinline__ void collide_push_2d(
   }
   Node2D<N> nd;
   N fchm[9];
-  if (!node_2d<N, FLOW, CHM>(c, gr.fold, f, g, dphi, dphi_prev, Rg, pn[1], pn[3], pn[2], pn[4], pn[5],
-                             pn[6], pn[8], pn[7], nd, fchm))
-    atomicOr(err, 1u);
+  const N mark = node_2d<N, FLOW, CHM>(c, gr.fold, f, g, dphi, dphi_prev, Rg, pn[1], pn[3], pn[2],
+                                       pn[4], pn[5], pn[6], pn[8], pn[7], nd, fchm);
+  if (!all_finite(mark)) {
+    bool bad = !(MASK && EDGE);
+    if (MASK && EDGE)  // whatever a solid node holds takes no part in the step
+#pragma unroll
+      for (int k = 0; k < V; ++k) bad = bad || (!(sm[k] & 1u) && !(lane(mark, k) == S(0)));
+    if (bad) atomicOr(err, 1u);
+  }
   Unew = nd.U;
 
   if constexpr (!EDGE) {

@@ -180,12 +180,11 @@ struct Node3D {
 };
 
 // Moments, gradient, anisotropy and coefficients of a node; pn: the eighteen
-// neighbours' phi + 1.  False if phi, U or rho is not finite.
+// neighbours' phi + 1.  Returns the finite_mark of phi, U and rho.
 template <typename N, bool FLOW, bool CHM>
-__device__ __forceinline__ bool node_3d(const Coef<N>& c, const N (&f)[19], const N (&g)[7], N dphi,
-                                        N dphi_prev, N Rg, const N (&pn)[19], bool y_first,
-                                        Node3D<N>& o,
-                                        N (&fchm)[19]) {
+__device__ __forceinline__ N node_3d(const Coef<N>& c, const N (&f)[19], const N (&g)[7], N dphi,
+                                     N dphi_prev, N Rg, const N (&pn)[19], bool y_first,
+                                     Node3D<N>& o, N (&fchm)[19]) {
   using S = typename Lanes<N>::S;
   const N one = splat<N>(S(1)), half = splat<N>(S(0.5));
   // ---- local moments (Eqs. 11, 12, 17, 22) ----------------------------------
@@ -214,7 +213,7 @@ __device__ __forceinline__ bool node_3d(const Coef<N>& c, const N (&f)[19], cons
     }
   }
   const N rho = add_r(one, drho);
-  const bool ok = all_finite(phi, U, rho);
+  const N mark = finite_mark(phi, U, rho);
   const N ph = clamp1(phi);
   const N mask = mul_r(half, sub_r(one, ph));  // (1 - phi)/2 of Eq. 7 and q(phi) of Eq. 18
 #pragma unroll
@@ -293,7 +292,7 @@ __device__ __forceinline__ bool node_3d(const Coef<N>& c, const N (&f)[19], cons
   for (int d = 0; d < 3; ++d) o.H[d] = mul_r(wt, Nv[d]);
   // Eq. 19: h_new = h* / a_s^2 + (1 - 1/a_s^2) h_old
   o.keep_old = sub_r(one, o.inv_a2);
-  return ok;
+  return mark;
 }
 
 // c_a . v (a a constant after unrolling; not the rest direction)
@@ -417,7 +416,9 @@ __device__ __forceinline__ void collide_push_3d(
   for (int a = 0; a < 7; ++a) g[a] = own(QF + a);
   Node3D<R> nd;
   R fchm[19];
-  if (!node_3d<R, FLOW, CHM>(c, f, g, dphi, dphi_prev, Rg, pn, y_first, nd, fchm)) atomicOr(err, 1u);
+  const R mark = node_3d<R, FLOW, CHM>(c, f, g, dphi, dphi_prev, Rg, pn, y_first, nd, fchm);
+  // (whatever a solid node holds takes no part in the step)
+  if (!all_finite(mark) && !(MASK && EDGE && (sm & 1u))) atomicOr(err, 1u);
   Unew = nd.U;
 
   if constexpr (!EDGE) {

@@ -364,3 +364,100 @@ def test_3d_graph_restart_and_mask_removal(P, L):
     free.step(20)
     assert np.array_equal(g.state(), free.state())
 
+
+
+# what a masked array leaves inside an obstacle: (storage, size, collision) over the step
+# kernels of each storage type, the two-node tiles among them (16-bit, 901 x 397)
+MASKED = [("fp64", (70, 45), 0), ("fp64", (70, 45), 1), ("fp32", (70, 45), 0),
+          ("fp32", (70, 45), 1), ("fp32", (1024, 563), 0), ("fp16", (96, 64), 0),
+          ("fp16", (901, 397), 0), ("fp16", (901, 397), 1), ("bf16", (901, 397), 0),
+          ("fp64", (33, 21, 17), 0), ("fp32", (33, 21, 17), 0), ("fp32", (33, 21, 17), 1),
+          ("fp16", (33, 21, 17), 0)]
+
+
+def masked_fields(size):
+    """Seeded fields [z][y][x], an obstacle's mask (rows 14 and 15 of every four its top,
+    the last column and the first rows among its nodes) and a fluid node below it: the
+    other node of a two-node thread that holds one of the obstacle's."""
+    rng = np.random.default_rng(11)
+    shape = size[::-1]
+    r = np.sqrt(sum((g - n / 2.0) ** 2 for g, n in zip(np.indices(shape), shape)))
+    phi = np.tanh((9.0 - r) / (math.sqrt(2) * 2.0)) + 0.01 * rng.uniform(-1, 1, shape)
+    U = 0.3 + 0.05 * rng.uniform(-1, 1, shape)
+    rho = 1.0 + 1e-3 * rng.uniform(-1, 1, shape)
+    v = [1e-2 * rng.uniform(-1, 1, shape) for _ in range(3)]
+    mask = np.zeros(shape, np.uint8)
+    mask[..., 14:16, 5:20] = 1
+    mask[..., 0:2, -3:] = 1
+    mask[..., -6:-2, 9] = 1
+    return phi, U, rho, v, mask
+
+
+def masked_sim(L, storage, size, chm, fields, mask):
+    dim = len(size)
+    sim = L.Sim(dim=dim, nx=size[0], ny=size[1], nz=size[2] if dim == 3 else 1, bc=(0, 2, 0),
+                flow=1, storage=dict(fp64=L.FP64, fp32=L.FP32, fp16=L.FP16_SHIFTED,
+                                     bf16=L.BF16_SHIFTED)[storage],
+                fold=4 if dim == 2 else 0, eps_aniso=0.03, collision=chm)
+    phi, U, rho, v = fields
+    sim.init_fields(phi, U, rho, v[0], v[1], v[2] if dim == 3 else None)
+    sim.set_solid(mask)
+    return sim
+
+
+@pytest.mark.parametrize("storage,size,chm", MASKED, ids=str)
+def test_non_finite_state_inside_an_obstacle(P, L, storage, size, chm):
+    # the state of solid nodes takes no part in the step: NaN there neither fails the
+    # run nor changes a fluid node
+    phi, U, rho, v, mask = masked_fields(size)
+    sel = mask.astype(bool)
+    hole = lambda f: np.where(sel, np.nan, f)
+    names = ("phi", "U", "rho", "ux", "uy")
+    a = masked_sim(L, storage, size, chm, (hole(phi), U, hole(rho), [hole(c) for c in v]), mask)
+    b = masked_sim(L, storage, size, chm, (phi, U, rho, v), mask)
+    for s in (a, b):
+        s.step(3)
+    fa, fb = a.fields(names), b.fields(names)
+    for k in names:
+        assert np.isfinite(fa[k][~sel]).all(), k
+        assert np.array_equal(fa[k][~sel], fb[k][~sel]), k
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("storage,size,chm", MASKED, ids=str)
+def test_non_finite_fluid_node_beside_an_obstacle_is_reported(P, L, storage, size, chm):
+    phi, U, rho, v, mask = masked_fields(size)
+    sel = mask.astype(bool)
+    bad = np.where(sel, np.nan, rho)
+    bad[..., 12, 7] = np.nan  # two rows below a solid node
+    assert not mask[..., 12, 7].any() and mask[..., 14, 7].all()
+    s = masked_sim(L, storage, size, chm, (phi, U, bad, v), mask)
+    s.step(1)
+    with pytest.raises(L.LbpfError, match="non-finite"):
+        s.fields()
+    s.close()
+
+
+def test_batch_with_a_non_finite_state_inside_an_obstacle(P, L):
+    # every tile shape of the batched step (its tuner steps through all of them)
+    sims = []
+    for hole in (True, False):
+        kw = dict(dim=2, bc=(0, 2, 0), flow=1, storage=L.FP16_SHIFTED, fold=4, eps_aniso=0.03)
+        b = L.Batch([dict(nx=70, ny=45, **kw), dict(nx=130, ny=66, **kw)],
+                    [(35.0, 22.0, 0.0, 8.0, 0.3, 0.0, 1), (60.0, 30.0, 0.0, 8.0, 0.3, 0.0, 2)])
+        for i, size in enumerate(((70, 45), (130, 66))):
+            phi, U, rho, v, mask = masked_fields(size)
+            if hole:
+                phi, rho = (np.where(mask.astype(bool), np.nan, f) for f in (phi, rho))
+            b.instance(i).init_fields(phi, U, rho, v[0], v[1], None)
+            b.instance(i).set_solid(mask)
+        b.step(70)
+        sims.append(b)
+    for i, size in enumerate(((70, 45), (130, 66))):
+        sel = masked_fields(size)[4].astype(bool)
+        fa, fb = sims[0].instance(i).fields(), sims[1].instance(i).fields()
+        for k in fa:
+            assert np.array_equal(fa[k][~sel], fb[k][~sel]), (i, k)
+    for b in sims:
+        b.close()

@@ -130,7 +130,10 @@ __global__ void __launch_bounds__(TX* TY* TZ)
 // -> 250, FP16 284 -> 213; 64^3 FP32 31 -> 20, FP16 36 -> 22.  Columns of 32 x 4 (128 threads):
 // 844 and 724 us at 256^3 (a larger share of halo, 10 / 8 against 6 / 4 rows of
 // h); 64 x 4: 863 and 776 (its warps wait on one another's barriers); 256
-// threads are held to 128 registers, two CTAs an SM.
+// threads are held to 128 registers, two CTAs an SM.  Without flow a CTA has half
+// the data and arithmetic of a plane, and two do not keep an SM busy: three, at 80
+// registers without spills.  Per step, two CTAs -> three: 97 x 63 x 83 FP32 28.3 -> 22.7 us,
+// FP16 30.4 -> 25.4; 128^3 71.3 -> 63.3 and 72.4 -> 64.5; 256^3 451 -> 396 and 422 -> 358.
 //
 // 16-bit storage keeps g relative to a per-node U (two FP16 planes, as in
 // the 2D step): the node's own reference is read from plane c, its new U
@@ -166,10 +169,12 @@ struct Col3D {
 // blocks of nodes with a flag for solid nodes: rows of a column, so that a
 // column's flags are those of a few blocks
 constexpr int kFlagX = 32, kFlagY = 4, kFlagZ = 8;
+// CTAs (of 256 threads) an SM holds
+constexpr int col_ctas(bool flow) { return flow ? 2 : 3; }
 constexpr int kSpin3 = 1 << 22;  // bound on mbarrier polls before giving up
 
 template <typename T, bool FLOW, int TX, int TY, bool CHM, bool MASK>
-__global__ void __launch_bounds__(TX* TY, 512 / (TX * TY))
+__global__ void __launch_bounds__(TX* TY, col_ctas(FLOW))
     step3d_column_kernel(const __grid_constant__ CUtensorMap tm_fg,
                          const __grid_constant__ CUtensorMap tm_h,
                          const __grid_constant__ CUtensorMap tm_ring,
@@ -399,21 +404,23 @@ __global__ void __launch_bounds__(TX* TY, 512 / (TX * TY))
 }
 
 // A column's nodes (above), and the planes per chunk: the fewest plane steps
-// of the busiest slot, with 2 CTAs on each of 152 SMs and a chunk of zc planes
+// of the busiest slot, with col_ctas CTAs on each of 152 SMs and a chunk of zc planes
 // costing its first planes' h as well (about a plane and a half; 64^3: 49, 28 and
 // 20 us at 16, 8 and 4 planes).  At 256^3 4, 8 and 16 planes take 810, 797 and 820
 // us (FP16 725, 690 and 692), at 203 x 150 x 134 244, 250 and 275, at 40 x 44 x 48
-// 16.5, 29 and 53 (12.7 at the 2 planes chosen there): so never more than 8, but where gridDim.z asks for it.
-constexpr int kColX = 32, kColY = 8, kColSlots = 304;
+// 16.5, 29 and 53 (12.7 at the 2 planes chosen there): so never more than 8, but where
+// gridDim.z asks for it.
+constexpr int kColX = 32, kColY = 8;
 
 int col_planes(const Model& m) {
   const long long cols = (long long)((m.nx + kColX - 1) / kColX) * ((m.ny + kColY - 1) / kColY);
+  const int slots = 152 * col_ctas(m.flow);
   int best = 8;
   double cost = 1e300;
   const int least = (m.nz + 65534) / 65535;  // gridDim.z
   for (int zc = std::max(8, least); zc >= least; --zc) {
     const long long ctas = cols * ((m.nz + zc - 1) / zc);
-    const double t = double((ctas + kColSlots - 1) / kColSlots) * (zc + 1.5);
+    const double t = double((ctas + slots - 1) / slots) * (zc + 1.5);
     if (t < cost) cost = t, best = zc;
   }
   return std::min(best, m.nz);

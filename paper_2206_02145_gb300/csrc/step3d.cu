@@ -22,8 +22,13 @@ namespace lbk {
 namespace {
 
 // ---- FP64 step kernel: one tile per CTA -----------------------------------------
+// Bound by the FP64 pipe.  So a warp takes one path: a tile two rows from a face
+// holds nodes of both kinds in a warp, and a branch per node runs the arithmetic
+// twice (64^3 coupled 361 -> 231 us, 16 x 256 x 256 1661 -> 863).  Three CTAs an SM: with the central
+// Hermite MRT that takes 168 registers and a few spills, at 190 and two 6 x 69 x 44
+// takes 88 us instead of 75.
 template <typename T, typename R, bool FLOW, bool CHM, int TX, int TY, int TZ>
-__global__ void __launch_bounds__(TX* TY* TZ)
+__global__ void __launch_bounds__(TX* TY* TZ, 3)
     step3d_kernel(const Model m, const T* __restrict__ src, T* __restrict__ dst,
                   const R* __restrict__ ring_prev, R* __restrict__ ring_cur,
                   unsigned* __restrict__ err) {
@@ -84,9 +89,8 @@ __global__ void __launch_bounds__(TX* TY* TZ)
     sh_phi[lz][ly][lx] = s;
   }
   __syncthreads();
-  if (!active) return;
   unsigned sm = 0;  // solid neighbours
-  if (m.solid)
+  if (m.solid && active)
     for (int a = 0; a < 19; ++a)
       sm |= solid_mapped3(m, x + D3_CX[a], y + D3_CY[a], z + D3_CZ[a]) ? 1u << a : 0u;
   const Grid3D gr(m);
@@ -104,10 +108,12 @@ __global__ void __launch_bounds__(TX* TY* TZ)
         [](int, int, int) { return R(0); }, sm, R(coef<R>(m).ref_g),
         dst + ((long long)z * slab + (long long)y0 * px + x0), o, false, err, Unew);
   };
-  if (sm || x < 1 || x > nx - 2 || y < 1 || y > ny - 2 || z < 1 || z > nz - 2)
-    work(std::true_type{});
-  else
-    work(std::false_type{});
+  // one path per warp: a warp with nodes of both kinds would run both
+  const bool edge = __any_sync(
+      0xffffffffu, active && (sm || x < 1 || x > nx - 2 || y < 1 || y > ny - 2 || z < 1 || z > nz - 2));
+  if (!active) return;
+  if (edge) work(std::true_type{});
+  else work(std::false_type{});
   ring_cur[idx] = dphi;
 }
 

@@ -50,8 +50,13 @@ static_assert(offsetof(BatchDesc, m) % 16 == 0 &&
                   offsetof(BatchDesc, m) + kModelCopy <= sizeof(BatchDesc),
               "the model copy must be an aligned span of the descriptor");
 
-// Registers held to 16 resident warps per SM (12 where a thread holds two
-// nodes: at 16 those spill, 406 against 378 us per step of 32 FP16 instances).  MASK: solid nodes (each instance's
+// Registers held to 12 resident warps per SM where a thread holds two nodes (at 16
+// those spill, 406 against 378 us per step of 32 FP16 instances), to 20 in tiles of
+// 32 x 4 and without flow, elsewhere 16.  32 x 4 is the shape of instances that are
+// small or few, where the chain of a tile counts (16 -> 20 warps: 3 of 197 to 220
+// squared, FP32, central Hermite MRT 14.0 -> 11.3 us; 28 of 21 to 232, BF16 56 -> 50;
+// 18 of 418 to 566, FP16 without flow 185 -> 146; but 64 of 32 squared, a tile per
+// CTA, 7.7 -> 8.0).  MASK: solid nodes (each instance's
 // model points at the per-tile flags of this variant's tiles); CHM: the
 // central Hermite MRT flow collision.
 //
@@ -64,7 +69,7 @@ static_assert(offsetof(BatchDesc, m) % 16 == 0 &&
 // everything from shared memory: no global lookups on a tile's critical path.
 template <typename T, bool FLOW, int TX, int TY, bool PAIR, int S, bool MASK, bool CHM>
 __global__ void __launch_bounds__(tile_threads<TX, TY, PAIR>(),
-                                  (PAIR ? 384 : 512) / tile_threads<TX, TY, PAIR>())
+                                  (PAIR ? 384 : (TX == 32 || !FLOW ? 640 : 512)) / tile_threads<TX, TY, PAIR>())
     step2d_batch_kernel(const BatchDesc* __restrict__ descs, const BatchSeg* __restrict__ segs,
                         const int* __restrict__ cta_seg) {
   using L = Tiles2D<T, FLOW, TX, TY>;

@@ -165,9 +165,11 @@ struct StepMaps {
 
 // The 2D steps: a state (populations and rings of both buffers) of more than
 // kL2Bytes does not stay in the L2; then at most kStageBytes of pipeline stages
-// are kept resident per SM (step2d.cu).
+// are kept resident per SM (step2d.cu).  144 KB are five CTAs of the batched FP32
+// step without flow (14 of 402 to 445 squared: 96.6 us against 104 with four) and
+// three of the coupled one.
 constexpr double kL2Bytes = 129e6;
-constexpr int kStageBytes = 142 * 1024;
+constexpr int kStageBytes = 144 * 1024;
 
 // Launchers (each returns the launch error).
 cudaError_t prepare_step2d(const Model& m, void* const pops[2], void* const rings[2],

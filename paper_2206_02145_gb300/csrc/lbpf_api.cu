@@ -1,6 +1,7 @@
 // Host side of the C ABI declared in include/lbpf.h: parameter validation,
 // device memory, the step loop with its CUDA-graph replay, state export and
 // restore, field read-out and FP64 diagnostics.
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -328,6 +329,8 @@ lbpf_status lbpf_create(const lbpf_params* p, void* stream, lbpf_t** out) {
   }
   lbpf* h = new (std::nothrow) lbpf();
   if (!h) return LBPF_ENOMEM;
+  static std::atomic<unsigned long long> handles{0};
+  h->id = ++handles;
   h->p = *p;
   if (h->p.dim == 2) h->p.nz = 1;
   h->m = derive(h->p);

@@ -43,5 +43,6 @@ struct lbpf {
   int tail_next = 0;
   int status = LBPF_OK;
   int gen = 0;  // bumped whenever the state or the model constants are replaced
+  unsigned long long id = 0;  // of this handle alone, never used again
   char msg[256] = {0};
 };

@@ -42,6 +42,23 @@ struct Act {  // NHWC bf16 buffer
   int c = 0, h = 0, w = 0;
 };
 
+// What a captured prediction holds of the simulation, the settings and the
+// network besides their buffers: the simulation (its buffers and grid are one
+// handle's for good), the constants that initialisation or a restart replaces,
+// and the convolutions' path.
+struct PredictionKey {
+  unsigned long long sim = 0;
+  cudaStream_t stream = nullptr;
+  double ref_g = 0.0;
+  int icx = 0, icy = 0, tensor_path = 0;
+  lbpf_surrogate_cfg cfg{};
+  bool same(const PredictionKey& o) const {
+    return sim == o.sim && stream == o.stream && ref_g == o.ref_g && icx == o.icx &&
+           icy == o.icy && tensor_path == o.tensor_path &&
+           std::memcmp(&cfg, &o.cfg, sizeof(cfg)) == 0;
+  }
+};
+
 // SplitMix64-driven uniform numbers for the weight initialisation
 uint64_t mix(uint64_t z) {
   z += 0x9E3779B97F4A7C15ull;
@@ -88,9 +105,7 @@ struct lbpf_unet {
   // the prediction phase of a block as a CUDA graph per buffer parity, with
   // the key it was captured for; results land in pinned host memory
   cudaGraphExec_t pgraph[2] = {nullptr, nullptr};
-  const void* pkey_pops[2] = {nullptr, nullptr};
-  lbpf_surrogate_cfg pkey_cfg[2];
-  cudaStream_t pkey_stream[2] = {nullptr, nullptr};
+  PredictionKey pkey[2];
   double* hres = nullptr;  // [0..2] sums, [3..10] crossings (predicted, current), [11] error word
   std::vector<void*> allocs;
   size_t bytes = 0;
@@ -945,12 +960,19 @@ int queue_prediction(lbpf* h, lbpf_unet* net, const lbpf_surrogate_cfg* cfg, cud
 }
 
 // the graph of the prediction phase for the current buffer parity, captured
-// on first use and again whenever the state buffers, stream or settings change
+// on first use and again whenever what it holds (PredictionKey) has changed
 int prediction_graph(lbpf* h, lbpf_unet* net, const lbpf_surrogate_cfg* cfg,
                      cudaGraphExec_t* out) {
   const int c = h->cur;
-  if (net->pgraph[c] && net->pkey_pops[c] == h->pops[c] && net->pkey_stream[c] == h->stream &&
-      std::memcmp(&net->pkey_cfg[c], cfg, sizeof(*cfg)) == 0) {
+  PredictionKey key;
+  key.sim = h->id;
+  key.stream = h->stream;
+  key.ref_g = h->m.ref_g;
+  key.icx = h->icx;
+  key.icy = h->icy;
+  key.tensor_path = net->tensor_path;
+  key.cfg = *cfg;
+  if (net->pgraph[c] && net->pkey[c].same(key)) {
     *out = net->pgraph[c];
     return LBPF_OK;
   }
@@ -983,9 +1005,7 @@ int prediction_graph(lbpf* h, lbpf_unet* net, const lbpf_surrogate_cfg* cfg,
   e = cudaGraphInstantiate(&net->pgraph[c], g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) return sfail(h, LBPF_ECUDA, "prediction graph: %s", cudaGetErrorString(e));
-  net->pkey_pops[c] = h->pops[c];
-  net->pkey_stream[c] = h->stream;
-  net->pkey_cfg[c] = *cfg;
+  net->pkey[c] = key;
   *out = net->pgraph[c];
   return LBPF_OK;
 }

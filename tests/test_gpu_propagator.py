@@ -190,3 +190,83 @@ def test_two_propagators_on_unordered_streams(L, S):
         assert both[i][0] == alone[i][0], (both[i][0], alone[i][0])
         assert alone[i][0]["surrogate_blocks"] > 0, alone[i][0]
         np.testing.assert_array_equal(both[i][1], alone[i][1])
+
+
+def _quiet_net(L):
+    """Untrained, the head's weights small: predictions close to no change."""
+    net = _net(L)
+    w = net.weights()
+    w[-132:] *= 0.01
+    net.set_weights(w)
+    return net
+
+
+def _seeded(L, seed, sim=None, **kw):
+    """A simulation 100 steps after a seed (cx, cy, u0): a new one, or `sim` again."""
+    if sim is None:
+        sim = L.Sim(stream=L.current_stream(), nx=NX, ny=NY, flow=1,
+                    **dict(dict(bc=(0, 2, 0), eps_aniso=0.04), **kw))
+    sim.init_seed(seed[0], seed[1], 0.0, 12.0, seed[2], 0.01, 3)
+    sim.step(100)
+    return sim
+
+
+def _advance(L, sim, net, blocks=4):
+    cfg = L.surrogate_cfg(judge_every=0, iface_tol=5.0, drift_tol=0.05)
+    rep = L.lbpf_surrogate_advance(sim, net, cfg, blocks)
+    return rep, sim.state()
+
+
+FIRST, SECOND = (128, 128, 0.3), (90, 140, 0.42)
+
+
+def test_a_reinitialised_simulation_is_predicted_from_its_own_constants(L, S):
+    # another seed on the same handle: other constants (the reference U of the
+    # stored state, the node the interface is measured from), the same buffers
+    net = _quiet_net(L)
+    sim = _seeded(L, FIRST)
+    _advance(L, sim, net)
+    got = _advance(L, _seeded(L, SECOND, sim), net)
+    fresh_net = _quiet_net(L)
+    fresh = _seeded(L, SECOND)
+    want = _advance(L, fresh, fresh_net)
+    assert want[0]["surrogate_blocks"] > 0, want[0]
+    assert got[0] == want[0]
+    np.testing.assert_array_equal(got[1], want[1])
+    for s in (sim, fresh, net, fresh_net):
+        s.close()
+
+
+def test_the_convolutions_path_can_change_between_calls(L, S):
+    states = {}
+    for paths in ((True, False), (False,), (True,)):
+        net = _quiet_net(L)
+        for i, path in enumerate(paths):
+            net.set_tensor_path(path)
+            sim = _seeded(L, FIRST)
+            rep, states[paths] = _advance(L, sim, net)
+            assert rep["surrogate_blocks"] > 0, rep
+            sim.close()
+        net.close()
+    np.testing.assert_array_equal(states[(True, False)], states[(False,)])
+    assert not np.array_equal(states[(True,)], states[(False,)])  # the paths do differ
+
+
+@pytest.mark.parametrize("storage", ["FP32", "FP16_SHIFTED"])
+def test_simulations_that_follow_one_another_share_a_network(L, S, storage):
+    # a simulation created after another was destroyed, at the same addresses as
+    # likely as not, with other boundaries
+    st = getattr(L, storage)
+    net = _quiet_net(L)
+    for seed, bc in ((FIRST, (0, 2, 0)), (SECOND, (0, 0, 0)), (FIRST, (2, 2, 0))):
+        sim = _seeded(L, seed, bc=bc, storage=st)
+        got = _advance(L, sim, net)
+        sim.close()
+        fresh_net = _quiet_net(L)
+        sim = _seeded(L, seed, bc=bc, storage=st)
+        want = _advance(L, sim, fresh_net)
+        sim.close()
+        fresh_net.close()
+        assert got[0] == want[0], bc
+        np.testing.assert_array_equal(got[1], want[1])
+    net.close()

@@ -1175,6 +1175,16 @@ def surrogate_arm(args, w, nb, stream, dist, clk, rank):
     }, net, a, pcfg, K
 
 
+def propagator_launches(rep, nb):
+    """Kernels of one lbpf_surrogate_advance on the configured network, from its
+    report: every block's prediction (read-out 2, network 19, predicted planes 1,
+    their sums 2 and interface positions 1), two to commit a predicted block, nb
+    steps for the others (the two of the last read-out, where the last block was
+    the LB's, are not counted)."""
+    lb = rep["judged_blocks"] + rep["fallback_blocks"]
+    return rep["blocks"] * 25 + rep["surrogate_blocks"] * 2 + lb * nb
+
+
 def run_surrogate(args, w):
     """c5: for each block length (the configured 50 LB steps first, then 200),
     train the U-Net on LB trajectories and time the block propagator against
@@ -1254,8 +1264,7 @@ def run_surrogate(args, w):
                    "sample": f"{osteps} LB steps of a 256x256 closed channel of the same family "
                              f"({n} nodes), {dt:.1f} s, FP64"}
         rep = head["report"]
-        launches = (K + 1) * 28 + rep["surrogate_blocks"] * 2 + (
-            rep["judged_blocks"] + rep["fallback_blocks"]) * nb
+        launches = propagator_launches(rep, nb)
         out = {
             "metric": "LB-equivalent MLUPS (learned block propagator)", "value": head["value"],
             "unit": "MLUPS", "n_gpus": world, "steps": head["steps"], "warmup": nb,
@@ -1286,7 +1295,7 @@ def run_surrogate(args, w):
                               for k, r in arms.items()},
             "roofline": {"bound": "tensor", "achieved": tflops, "peak": peak_tf,
                          "unit": "TFLOP/s", "frac": tflops / peak_tf, "peak_source": peak_kind,
-                         "traffic": None, "kernel": "network forward (17 conv3x3_tc + 8 "
+                         "traffic": None, "kernel": "network forward (17 conv3x3_tc + 2 "
                          "element-wise launches), 512x512, batch 1",
                          "algorithmic_flops_per_forward": flop, "forward_ms": fwd_ms},
             "cpu_baseline": cpu,

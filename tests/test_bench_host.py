@@ -102,3 +102,12 @@ def test_profiled_traffic_follows_the_source_digest(bench, tmp_path, monkeypatch
     assert bench.profiled_traffic(dict(kernel="k", nx=8, storage="fp32", src=w["src"])) is None
     (prof / "k_8_fp32.md").write_text(f"source_sha256: {digest}\ndram_bytes_per_launch: 123\n")
     assert bench.profiled_traffic(dict(kernel="k", nx=8, storage="fp32", src=w["src"])) == 123.0
+
+
+def test_propagator_launches_follow_the_report(bench):
+    # a block's prediction is 25 kernels (a network pass with them); nothing runs
+    # after the last block but its read-out
+    rep = dict(blocks=0, surrogate_blocks=0, judged_blocks=0, fallback_blocks=0)
+    assert bench.propagator_launches(rep, 50) == 0
+    rep = dict(blocks=8, surrogate_blocks=5, judged_blocks=2, fallback_blocks=1)
+    assert bench.propagator_launches(rep, 50) == 8 * 25 + 5 * 2 + 3 * 50

@@ -42,15 +42,28 @@ import time
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
+
+def sources(*units):
+    """The units and every file of the library that they include, in a fixed order."""
+    found = []
+    todo = list(units)
+    while todo:
+        f = todo.pop(0)
+        if f in found:
+            continue
+        found.append(f)
+        text = open(os.path.join(ROOT, "paper_2206_02145_gb300", "csrc", f)).read()
+        todo += [i for i in re.findall(r'^#include "([^"]+)"', text, re.M) if "/" not in i]
+    return found
+
+
 # the files each timed kernel is compiled from (a committed profile's counters
 # stand only while their digest is unchanged)
-SRC_2D = ["step2d.cu", "step2d_tile.cuh", "step2d_core.cuh", "lbpf_device.cuh", "tma.cuh"]
-SRC_3D = ["step3d.cu", "step3d_core.cuh", "lbpf_device.cuh", "tma.cuh"]
-SRC_BATCH = ["batch2d.cu", "batch2d_kernels.cuh", "batch2d_fp32.cu", "batch2d_fp16.cu",
-             "batch2d_bf16.cu", "batch_schedule.h", "step2d_tile.cuh", "step2d_core.cuh",
-             "lbpf_device.cuh", "tma.cuh"]
-SRC_CONV = ["conv_tc.cu", "tcgen05.cuh", "tma.cuh"]
-SRC_FACETS = ["facets.cu"]
+SRC_2D = sources("step2d.cu")
+SRC_3D = sources("step3d.cu")
+SRC_BATCH = sources("batch2d.cu", "batch2d_fp32.cu", "batch2d_fp16.cu", "batch2d_bf16.cu")
+SRC_CONV = sources("conv_tc.cu")
+SRC_FACETS = sources("facets.cu")
 
 # bytes each node moves through HBM per step (populations read + written,
 # phi(t-1) read, phi(t) written)

@@ -111,3 +111,16 @@ def test_propagator_launches_follow_the_report(bench):
     assert bench.propagator_launches(rep, 50) == 0
     rep = dict(blocks=8, surrogate_blocks=5, judged_blocks=2, fallback_blocks=1)
     assert bench.propagator_launches(rep, 50) == 8 * 25 + 5 * 2 + 3 * 50
+
+
+def test_digest_covers_every_included_source(bench):
+    # a constant in a header (what the stages hold per SM, say) changes the traffic
+    # as the kernel's own file does
+    import re
+    csrc = os.path.join(ROOT, "paper_2206_02145_gb300", "csrc")
+    for name in bench.WORKLOADS:
+        src = bench.workload(name)["src"]
+        for f in src:
+            text = open(os.path.join(csrc, f)).read()
+            for i in re.findall(r'#include "([^"]+)"', text):
+                assert "/" in i or i in src, (name, f, i)

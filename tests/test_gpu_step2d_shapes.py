@@ -100,3 +100,100 @@ def test_solids_and_collision(P, size, chm):
     errs = P.max_errors(a, b)
     assert max(errs.values()) < 1e-5, errs
     a.close()
+
+
+# ---- the two-node tiles (and the 32 x 4 ones next to them) in 16-bit storage ----
+UNITS = [("fp16", 2.0 ** -11), ("bf16", 2.0 ** -8)]
+
+
+def within_storage_bounds(errs, u):
+    n = STEPS + 1  # the initial state is rounded too
+    assert errs["phi"] < n * u * 2.0 and errs["U"] < n * u * 0.5, errs
+    assert max(errs.get(k, 0.0) for k in ("rho", "ux", "uy")) < n * u * 0.1, errs
+
+
+def obstacles(size):
+    nx, ny = size
+    mask = np.zeros((ny, nx), bool)
+    mask[100:300, 60:68] = True      # across a tile edge
+    mask[0:3, 200:230] = True        # on the wall: rows 0 and 2 are one thread's
+    mask[41, 300:303] = True         # one of a thread's two nodes
+    mask[-2:, -40:-37] = True        # in the last tiles
+    return mask
+
+
+def solid_pair(P, size, bounds, storage, chm):
+    import oracle
+    import paper_2206_02145_gb300 as L
+    p, (phi, U, rho, v) = problem(P, size, bounds)
+    kw = dict(dim=2, nx=p["nx"], ny=p["ny"], bc=p["bc"], flow=1, fold=5, theta0=0.2,
+              u_inlet=p["u_in"], u0_inlet=p["U_in"], collision=chm)
+    a = L.Sim(storage=P.STORAGE[storage], eps_aniso=0.03, body_force=p["body"], **kw)
+    b = oracle.Oracle(oracle.Params(eps=0.03, body=p["body"], **kw))
+    for s in (a, b):
+        s.init_fields(phi, U, rho, v[0], v[1], None)
+        s.set_solid(obstacles(size))
+    return a, b
+
+
+@pytest.mark.parametrize("storage,u", UNITS)
+@pytest.mark.parametrize("bounds", [k for k in BOUNDS if k != "inflow"])
+@pytest.mark.parametrize("size", SIZES16, ids=str)
+def test_16bit_boundaries(P, size, bounds, storage, u):
+    p, fields = problem(P, size, bounds)
+    a, b = P.pair(p, storage, fields=fields)
+    a.step(STEPS)
+    b.step(STEPS, P.THREADS)
+    within_storage_bounds(P.max_errors(a, b), u)
+    a.close()
+
+
+@pytest.mark.parametrize("storage,u", UNITS)
+@pytest.mark.parametrize("bounds", ["periodic", "walls_x"])
+@pytest.mark.parametrize("size", SIZES16[:2], ids=str)
+def test_16bit_without_flow(P, size, bounds, storage, u):
+    p, fields = problem(P, size, bounds, flow=0)
+    a, b = P.pair(p, storage, fields=fields)
+    a.step(STEPS)
+    b.step(STEPS, P.THREADS)
+    within_storage_bounds(P.max_errors(a, b, ("phi", "U")), u)
+    a.close()
+
+
+@pytest.mark.parametrize("storage,u", UNITS)
+@pytest.mark.parametrize("chm", [0, 1])
+@pytest.mark.parametrize("bounds", ["inflow_walls", "periodic"])
+@pytest.mark.parametrize("size", SIZES16, ids=str)
+def test_16bit_solids_and_collision(P, size, bounds, chm, storage, u):
+    a, b = solid_pair(P, size, bounds, storage, chm)
+    a.step(STEPS)
+    b.step(STEPS, P.THREADS)
+    within_storage_bounds(P.max_errors(a, b), u)
+    a.close()
+
+
+@pytest.mark.parametrize("solids", [False, True])
+@pytest.mark.parametrize("chm", [0, 1])
+@pytest.mark.parametrize("bounds", BOUNDS)
+def test_two_nodes_per_thread_round_like_one(P, bounds, chm, solids):
+    # the batched step runs every one- and two-node shape in turn while it tunes; the
+    # single step of this size holds two nodes per thread: the same bits
+    import paper_2206_02145_gb300 as L
+    size = SIZES16[1]
+    p, (phi, U, rho, v) = problem(P, size, bounds)
+    kw = dict(dim=2, nx=p["nx"], ny=p["ny"], bc=p["bc"], flow=1, fold=5, theta0=0.2,
+              eps_aniso=0.03, u_inlet=p["u_in"], u0_inlet=p["U_in"], body_force=p["body"],
+              storage=L.FP16_SHIFTED, collision=chm)
+    one = L.Sim(**kw)
+    batch = L.Batch([kw], [(10.0, 10.0, 0.0, 4.0, 0.4, 0.0, 1)])
+    for s in (one, batch.instance(0)):
+        s.init_fields(phi, U, rho, v[0], v[1], None)
+        if solids:
+            s.set_solid(obstacles(size))
+    one.step(60)
+    batch.step(60)
+    assert batch.tuning()["tuned"]
+    # (the header names the node of the batch's seed; the arrays follow it)
+    np.testing.assert_array_equal(one.state()[P.HDR:], batch.instance(0).state()[P.HDR:])
+    one.close()
+    batch.close()

@@ -97,3 +97,37 @@ def test_solids_and_collision(P, size, chm):
     errs = P.max_errors(a, b, ("phi", "U", "rho", "ux", "uy", "uz"))
     assert max(errs.values()) < 1e-5, errs
     a.close()
+
+
+# chunks of 8 planes (the longest), ragged columns and a ragged last chunk
+EIGHT = (60, 150, 62)
+
+
+@pytest.mark.parametrize("storage,u", [("fp32", 0.0), ("fp16", 2.0 ** -11)])
+def test_chunks_of_eight_planes(P, storage, u):
+    p, fields = problem(P, EIGHT, "inflow_walls")
+    a, b = P.pair(p, storage, fields=fields)
+    a.step(STEPS)
+    b.step(STEPS, P.THREADS)
+    errs = P.max_errors(a, b, ("phi", "U", "rho", "ux", "uy", "uz"))
+    n = STEPS + 1  # the initial state is rounded too
+    assert errs["phi"] < 1e-5 + n * u * 2.0 and errs["U"] < 1e-5 + n * u * 0.5, errs
+    assert max(errs[k] for k in ("rho", "ux", "uy", "uz")) < 1e-5 + n * u * 0.1, errs
+    a.close()
+
+
+@pytest.mark.parametrize("storage,u", [("fp32", 0.0), ("fp16", 2.0 ** -11), ("bf16", 2.0 ** -8)])
+@pytest.mark.parametrize("bounds", ["inflow_walls", "periodic"])
+@pytest.mark.parametrize("size", SIZES + [EIGHT], ids=str)
+def test_without_flow(P, size, bounds, storage, u):
+    nx, ny, nz = size
+    p, (phi, U, rho, v) = problem(P, size, bounds)
+    p = P.params(dim=3, nx=nx, ny=ny, nz=nz, flow=0, fold=0, eps=0.03,
+                 **{k: w for k, w in BOUNDS[bounds].items() if k != "body"})
+    a, b = P.pair(p, storage, fields=(phi, U, rho, v))
+    a.step(STEPS)
+    b.step(STEPS, P.THREADS)
+    errs = P.max_errors(a, b, ("phi", "U"))
+    n = STEPS + 1
+    assert errs["phi"] < 1e-5 + n * u * 2.0 and errs["U"] < 1e-5 + n * u * 0.5, errs
+    a.close()

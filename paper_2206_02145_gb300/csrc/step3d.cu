@@ -129,17 +129,22 @@ __global__ void __launch_bounds__(TX* TY* TZ, 3)
 // planes of the step before are read by nobody, and thread 0 issues the next
 // copies into them.
 //
-// Bound by HBM in FP32 (0.86 of the measured copy rate at 256^3), by
-// instruction issue with 16-bit storage (0.52).  Per step, against the
-// kernel that moved every tile's arrays to shared memory by the threads'
-// own loads: 256^3 FP32 957 -> 797 us, FP16 942 -> 698; 203 x 150 x 134 FP32 281
-// -> 250, FP16 284 -> 213; 64^3 FP32 31 -> 20, FP16 36 -> 22.  Columns of 32 x 4 (128 threads):
-// 844 and 724 us at 256^3 (a larger share of halo, 10 / 8 against 6 / 4 rows of
-// h); 64 x 4: 863 and 776 (its warps wait on one another's barriers); 256
-// threads are held to 128 registers, two CTAs an SM.  Without flow a CTA has half
-// the data and arithmetic of a plane, and two do not keep an SM busy: three, at 80
-// registers without spills.  Per step, two CTAs -> three: 97 x 63 x 83 FP32 28.3 -> 22.7 us,
-// FP16 30.4 -> 25.4; 128^3 71.3 -> 63.3 and 72.4 -> 64.5; 256^3 451 -> 396 and 422 -> 358.
+// Bound by HBM in FP32 (0.90 of the measured copy rate at 256^3); with 16-bit
+// storage (0.55) instruction issue and the waits of a plane's chain share the
+// time; on small grids that chain alone.  So the halo positions outside the domain get
+// their h from the thread that sums phi there: a pass and a barrier of their own
+// before that sum had cost the chain 0.35 us of 1.85 a plane (64^3 19.8 -> 17.8 us).
+// Per step, against the kernel that moved every tile's arrays to shared memory by
+// the threads' own loads: 256^3 FP32 957 -> 762 us, FP16 942 -> 659; 203 x 150 x 134
+// FP32 281 -> 229, FP16 284 -> 198; 64^3 FP32 31 -> 18, FP16 36 -> 19.  Columns of 32 x 4
+// (128 threads) and of 64 x 4, before that pass was joined: 844 and 863 us at 256^3
+// (797 for 32 x 8), FP16 724 and 776 (698): a larger share of halo, 10 / 8 against
+// 6 / 4 rows of h; warps that wait on one another's barriers.  256 threads are held to 128
+// registers, two CTAs an SM.  Without flow a CTA has half the data and arithmetic of a
+// plane, and two do not keep an SM busy: three, at 80 registers without spills.  Per
+// step, two CTAs -> three -> one barrier: 97 x 63 x 83 FP32 28.5 -> 22.7 -> 18.6 us, FP16 30.4
+// -> 25.4 -> 20.4; 128^3 71.3 -> 63.3 -> 55.5 and 72.4 -> 64.5 -> 54; 256^3 451 -> 396 -> 370 and
+// 422 -> 358 -> 328.
 //
 // 16-bit storage keeps g relative to a per-node U (two FP16 planes, as in
 // the 2D step): the node's own reference is read from plane c, its new U
@@ -237,40 +242,18 @@ __global__ void __launch_bounds__(TX* TY, col_ctas(FLOW))
     if (L::REL) tma_load_4d(own + L::OFF_UOWN, &tm_uown, bar, x0, y0, z, c);
     load_h(z + 1, bar);
   };
-  // h halo positions of plane z outside the domain: the nearest node, which
-  // the box holds, or across a periodic edge the far side
-  auto patch = [&](int z) {
-    T* const hs = h_slot(z);
-    __half* const us = u_slot(z);
-    const int gz = grad_coord(z, nz, gr.bc[2]);
-    for (int i = tid; i < PL; i += NT) {
-      const int lx = i % SX, ly = i / SX;
-      const int gx = x0 + lx - 1, gy = y0 + ly - 1;
-      if (gx >= 0 && gx < nx && gy >= 0 && gy < ny) continue;
-      if (gx > nx || gy > ny) continue;  // beyond the halo of a partial column
-      const int wx = grad_coord(gx, nx, gr.bc[0]), wy = grad_coord(gy, ny, gr.bc[1]);
-      const int sx = wx - x0 + 1, sy = wy - y0 + 1;  // the mapped node in the box
-      T* const hd = hs + ly * L::BXH + lx + L::HX - 1;
-      __half* const ud = us + ly * L::BXU + lx + L::HXU - 1;
-      if (sx >= 0 && sx < SX && sy >= 0 && sy < SY) {
-        const T* const hf = hs + sy * L::BXH + sx + L::HX - 1;
-#pragma unroll
-        for (int a = 0; a < 7; ++a) hd[a * HPLANE] = hf[a * HPLANE];
-        if (L::REL) *ud = us[sy * L::BXU + sx + L::HXU - 1];
-      } else {
-        const long long j = (long long)gz * slab + (long long)wy * px + wx, P = gr.plane;
-#pragma unroll
-        for (int a = 0; a < 7; ++a) hd[a * HPLANE] = src[(L::QFG + a) * P + j];
-        if (L::REL) *ud = m.uring[(c ^ 1) * P + j];
-      }
-    }
-  };
   // phi + 1 of plane z with halo (and the solid flags) from its h: each
   // thread's own node from the h it keeps for the collision, the ring around
-  // the column by a pass
+  // the column's nodes by one thread a position.  That thread also gives the
+  // positions outside the domain their h: the nearest node's, which the box
+  // holds, or across a periodic edge the far side's.  (In a partial column the ring
+  // runs through positions of idle threads.)
   const int oh = (ty + 1) * L::BXH + tx + L::HX, op = (ty + 1) * SX + tx + 1;
+  const int vx = nx - x0 < TX ? nx - x0 : TX, vy = ny - y0 < TY ? ny - y0 : TY;
+  const bool on_ring = (x == nx && y <= ny) || (y == ny && x <= nx);
+  static_assert(2 * SX + 2 * TY <= NT, "a thread for every position of the ring");
   auto sum_phi = [&](int z, float(&h)[7]) {
-    const T* const hs = h_slot(z);
+    T* const hs = h_slot(z);
     float* const ps = sh_phi + slot(z) * PL;
     float s = 0.f;
 #pragma unroll
@@ -278,21 +261,46 @@ __global__ void __launch_bounds__(TX* TY, col_ctas(FLOW))
       h[a] = Pop<T>::template ld<float>(hs + a * HPLANE + oh);
       s = a == 0 ? h[0] : add_r(s, h[a]);
     }
-    ps[op] = s;
-    constexpr int NRING = 2 * SX + 2 * TY;
-    for (int i = tid; i < NRING; i += NT) {
-      int lx, ly;
-      if (i < 2 * SX) {
-        lx = i < SX ? i : i - SX;
-        ly = i < SX ? 0 : SY - 1;
+    if (!on_ring) ps[op] = s;
+    if (tid < 2 * (vx + 2) + 2 * vy) {
+      int lx, ly, i = tid;
+      if (i < 2 * (vx + 2)) {
+        lx = i < vx + 2 ? i : i - (vx + 2);
+        ly = i < vx + 2 ? 0 : vy + 1;
       } else {
-        lx = (i - 2 * SX) & 1 ? SX - 1 : 0;
-        ly = 1 + (i - 2 * SX) / 2;
+        i -= 2 * (vx + 2);
+        lx = i & 1 ? vx + 1 : 0;
+        ly = 1 + i / 2;
       }
-      const T* const p = hs + ly * L::BXH + lx + L::HX - 1;
+      T* const p = hs + ly * L::BXH + lx + L::HX - 1;
+      T v[7];
+      const int gx = x0 + lx - 1, gy = y0 + ly - 1;
+      if (!rim || (gx >= 0 && gx < nx && gy >= 0 && gy < ny)) {
+#pragma unroll
+        for (int a = 0; a < 7; ++a) v[a] = p[a * HPLANE];
+      } else {
+        const int wx = grad_coord(gx, nx, gr.bc[0]), wy = grad_coord(gy, ny, gr.bc[1]);
+        const int sx = wx - x0 + 1, sy = wy - y0 + 1;  // the mapped node in the box
+        __half* const us = u_slot(z);
+        __half* const ud = us + ly * L::BXU + lx + L::HXU - 1;
+        if (sx >= 0 && sx < SX && sy >= 0 && sy < SY) {
+          const T* const hf = hs + sy * L::BXH + sx + L::HX - 1;
+#pragma unroll
+          for (int a = 0; a < 7; ++a) v[a] = hf[a * HPLANE];
+          if (L::REL) *ud = us[sy * L::BXU + sx + L::HXU - 1];
+        } else {
+          const int gz = grad_coord(z, nz, gr.bc[2]);
+          const long long j = (long long)gz * slab + (long long)wy * px + wx, P = gr.plane;
+#pragma unroll
+          for (int a = 0; a < 7; ++a) v[a] = src[(L::QFG + a) * P + j];
+          if (L::REL) *ud = m.uring[(c ^ 1) * P + j];
+        }
+#pragma unroll
+        for (int a = 0; a < 7; ++a) p[a * HPLANE] = v[a];
+      }
       float r = 0.f;
 #pragma unroll
-      for (int a = 0; a < 7; ++a) r += Pop<T>::template ld<float>(p + a * HPLANE);
+      for (int a = 0; a < 7; ++a) r += Pop<T>::template ld<float>(&v[a]);
       ps[ly * SX + lx] = r;
     }
     if (MASK && solids) {
@@ -322,11 +330,6 @@ __global__ void __launch_bounds__(TX* TY, col_ctas(FLOW))
     load_step(zs);
   }
   bool ok = mbar_wait_bounded(&first[0], 0, kSpin3);
-  if (rim) {
-    patch(zs - 1);
-    patch(zs);
-    __syncthreads();
-  }
   float h[7], hn[7];  // the node's own h in planes z and z + 1
   sum_phi(zs - 1, h);
   sum_phi(zs, h);
@@ -336,10 +339,6 @@ __global__ void __launch_bounds__(TX* TY, col_ctas(FLOW))
   for (int z = zs; z < ze; ++z) {
     const int k = z - zs;
     ok = mbar_wait_bounded(&full[k & 1], uint32_t(k >> 1) & 1u, kSpin3) && ok;
-    if (rim) {
-      patch(z + 1);
-      __syncthreads();
-    }
     sum_phi(z + 1, hn);
     if (__syncthreads_or(!ok)) {
       // a plane never arrived: report, let the copies in flight land, stop
@@ -411,11 +410,12 @@ __global__ void __launch_bounds__(TX* TY, col_ctas(FLOW))
 
 // A column's nodes (above), and the planes per chunk: the fewest plane steps
 // of the busiest slot, with col_ctas CTAs on each of 152 SMs and a chunk of zc planes
-// costing its first planes' h as well (about a plane and a half; 64^3: 49, 28 and
-// 20 us at 16, 8 and 4 planes).  At 256^3 4, 8 and 16 planes take 810, 797 and 820
-// us (FP16 725, 690 and 692), at 203 x 150 x 134 244, 250 and 275, at 40 x 44 x 48
-// 16.5, 29 and 53 (12.7 at the 2 planes chosen there): so never more than 8, but where
-// gridDim.z asks for it.
+// costing its first planes' h as well (about a plane and a half; 64^3: 46, 24 and
+// 18 us at 16, 8 and 4 planes).  At 256^3 4, 8 and 16 planes take 779, 763 and 773
+// us (FP16 697, 660 and 657), at 203 x 150 x 134 229, 229 and 236, at 40 x 44 x 48
+// 14.1, 24.5 and 45.5 (11.2 at the 2 planes chosen there): so never more than 8, but
+// where gridDim.z asks for it.  On 17 grids the choice is within 8 % of the best of 1 to
+// 32 planes.
 constexpr int kColX = 32, kColY = 8;
 
 int col_planes(const Model& m) {

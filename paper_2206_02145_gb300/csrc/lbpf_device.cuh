@@ -83,7 +83,9 @@ __device__ __forceinline__ bool finite_r(float v) { return isfinite(v); }
 // pushes are written with these so that the compiler cannot fuse them
 // differently in different code paths (interior vs edge tiles, single vs
 // batched kernels): every path then rounds identically and a node's result
-// does not depend on how the grid was tiled.
+// does not depend on how the grid was tiled.  Two exceptions in 3D: 16-bit grids
+// keep an order of one sum that follows their blocks (aniso_3d), and the central
+// Hermite MRT there is written as plain expressions.
 __device__ __forceinline__ float fma_r(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_r(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float mul_r(float a, float b) { return __fmul_rn(a, b); }
@@ -273,7 +275,10 @@ __device__ __forceinline__ void aniso_2d(const Coef<N>& c, int fold, N gx, N gy,
 // y_first: |grad|^2 takes x's square rounded and adds y's exactly, else the other
 // way round.  An FP32 rounding apart, but with 16-bit storage it turns over a
 // stored value here and there, which spreads over the run; results keep to the
-// order that each part of a 16-bit grid has always had.
+// order that each part of a 16-bit grid has always had: y first in the blocks of
+// 32 x 4 nodes that touch no face and, of 32 x 4 x 8, hold and border no solid node.
+// Neither order is the more exact; a state moved by a node along a periodic axis may
+// differ by such roundings.
 template <typename N>
 __device__ __forceinline__ void aniso_3d(const Coef<N>& c, const N (&g)[3], bool y_first, N& as,
                                          N (&Nv)[3]) {

@@ -163,7 +163,7 @@ struct StepMaps {
   int ctas_v[4] = {0, 0, 0, 0};  // 2D: CTAs of the variant MASK + 2 CHM
 };
 
-// The 2D steps: a state (populations and rings of both buffers) of more than
+// The 2D steps on this GPU, 129 MB of L2: a state (populations and rings of both buffers) of more than
 // kL2Bytes does not stay in the L2; then at most kStageBytes of pipeline stages
 // are kept resident per SM (step2d.cu).  144 KB are five CTAs of the batched FP32
 // step without flow (14 of 402 to 445 squared: 96.6 us against 104 with four) and

@@ -34,10 +34,10 @@
 //    2480 x 2080 step against 587) and the step takes 224 us instead of 177.
 //    1024^2: 48.4 -> 40.1 us (0.87 of the copy rate); 2480 x 2080: 250 -> 177
 //    (0.98).
-//  - 16-bit storage: issue slots.  A thread of a large grid holds two nodes, 2
-//    rows apart, on the packed two-lane FP32 instructions (lbpf_device.cuh): 606
-//    warp instructions per 32 nodes instead of 906.  1024^2: 38.2 -> 29.1 us;
-//    2480 x 2080: 119.
+//  - 16-bit storage: instructions, and the waits between them.  A thread of a large
+//    grid holds two nodes, 2 rows apart, on the packed two-lane FP32 instructions
+//    (lbpf_device.cuh): 590 warp instructions per 32 nodes instead of 906, 2.3 issued
+//    per cycle and SM instead of 2.8.  1024^2: 38.2 -> 29.1 us; 2480 x 2080: 119.
 //  - small grids: the chain of a tile.  Tiles of 32 x 4 with one node per
 //    thread give the most CTAs; boundary tiles run the same arithmetic as inner
 //    ones with precomputed steps.  128^2 without flow: 3.6 -> 3.2 us.

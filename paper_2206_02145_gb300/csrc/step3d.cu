@@ -247,7 +247,8 @@ __global__ void __launch_bounds__(TX* TY, col_ctas(FLOW))
   // the column's nodes by one thread a position.  That thread also gives the
   // positions outside the domain their h: the nearest node's, which the box
   // holds, or across a periodic edge the far side's.  (In a partial column the ring
-  // runs through positions of idle threads.)
+  // runs through positions of idle threads, which write nothing there and store no
+  // result.)
   const int oh = (ty + 1) * L::BXH + tx + L::HX, op = (ty + 1) * SX + tx + 1;
   const int vx = nx - x0 < TX ? nx - x0 : TX, vy = ny - y0 < TY ? ny - y0 : TY;
   const bool on_ring = (x == nx && y <= ny) || (y == ny && x <= nx);

@@ -3,7 +3,9 @@
 // h (Eqs. 19-23, cubic anisotropy of Eq. 3), push streaming.  The caller has
 // the node's own population deviations, phi + 1 and the h deviations around
 // the node (one node in x, y and z) in shared memory.  As in 2D every
-// operation is written with its rounding; a thread holds one node (two, on
+// operation of the BGK collision, the solute and the phase field is written with its
+// rounding (the central Hermite MRT and the inflow's constants are plain
+// expressions, to FP32 and FP64 accuracy); a thread holds one node (two, on
 // the packed FP32 instructions, measured slower: 831 against 690 us per step of
 // 256^3 in FP16, the code of both paths no longer fits the instruction cache).
 #pragma once
